@@ -113,8 +113,7 @@ int solve_jobs_dispatch(ddp_ctx *ctx, int prec, std::vector<Job> &jobs, std::vec
 
 template <class P>
 int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *out, int prec);
-template <class P>
-int hop_power_impl(ddp_ctx *ctx, const Job &job, int p, const double *psi, double *out);
+int hop_power_fx(ddp_ctx *ctx, const Job &job, int p, const double *psi, double *out);
 template <class P>
 int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters, float *ms, double *bytes);
 
@@ -797,7 +796,7 @@ int ddp_hop_power(ddp_ctx *ctx, int domain_id, double kappa, int p, const double
     memcpy(j.e, d->e, sizeof(j.e));
     j.kappa = kappa;
     j.ncol = ncol;
-    if ((rc = hop_power_impl<PF64>(ctx, j, p, (const double *)si.dev, (double *)so.dev))) return rc;
+    if ((rc = hop_power_fx(ctx, j, p, (const double *)si.dev, (double *)so.dev))) return rc;
     if ((rc = so.copy_out())) return rc;
     DDP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return DDP_OK;

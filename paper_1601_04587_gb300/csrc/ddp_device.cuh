@@ -507,13 +507,11 @@ __device__ __forceinline__ void accumulate(cx<R> acc[4][3], const cx<R> w[2][3],
 }
 
 // Geometry of one hop d = 2 mu + (backward ? 1 : 0) from even-odd site h of
-// parity p: the neighbour's even-odd index (or -1 when the hop is dropped)
-// and the link the neighbour is transported with, U_mu(x) forward and
-// U_mu(x - mu)^+ backward, multiplied by the boundary factor of the hop
-// (-1 across an antiperiodic time boundary).
-template <class P>
-__device__ __forceinline__ int stage_hop(const Item &it, int h, int p, int d, cx<typename P::real> u[3][3]) {
-    using R = typename P::real;
+// parity p: the neighbour's even-odd index (or -1 when the hop is dropped), the
+// row of the link the neighbour is transported with, U_mu(x) forward and
+// U_mu(x - mu)^+ backward, and whether the hop changes sign (across an
+// antiperiodic time boundary).
+__device__ __forceinline__ int hop_geometry(const Item &it, int h, int p, int d, int64_t &row, bool &neg) {
     int k[4], x[4];
     decode_site(it, h, p, k);
 #pragma unroll
@@ -539,30 +537,46 @@ __device__ __forceinline__ int stage_hop(const Item &it, int h, int p, int d, cx
         else if (kn[mu] < 0)
             kn[mu] = it.e[mu] - 1;
     }
-    R f = R(1);
+    neg = false;
     if (mu == 0 && x[0] == (fwd ? it.L[0] - 1 : 0)) {
-        if (it.bc == 1) f = R(-1);
+        neg = it.bc == 1;
         if (it.bc == 2) ok = false;
     }
     if (!ok) return -1;
-    const void *lk = P::IS64 ? it.links64 : it.links;
     if (fwd) {
-        load_link<P>(lk, it.gV, mu, link_row(it, x, p), u);
+        row = link_row(it, x, p);
+    } else {
+        x[mu] = (x[mu] == 0) ? it.L[mu] - 1 : x[mu] - 1;
+        row = link_row(it, x, p ^ 1);
+    }
+    return local_lex(it, kn) >> 1;
+}
+
+// The neighbour's index of a hop and its link in storage format P, oriented and
+// multiplied by the boundary sign of the hop.
+template <class P>
+__device__ __forceinline__ int stage_hop(const Item &it, int h, int p, int d, cx<typename P::real> u[3][3]) {
+    using R = typename P::real;
+    int64_t row = 0;
+    bool neg;
+    const int nb = hop_geometry(it, h, p, d, row, neg);
+    if (nb < 0) return -1;
+    const R f = neg ? R(-1) : R(1);
+    if (!(d & 1)) {
+        load_link<P>(it.links, it.gV, d >> 1, row, u);
 #pragma unroll
         for (int i = 0; i < 3; i++)
 #pragma unroll
             for (int j = 0; j < 3; j++) u[i][j] = f * u[i][j];
     } else {
-        int xm[4] = {x[0], x[1], x[2], x[3]};
-        xm[mu] = (xm[mu] == 0) ? it.L[mu] - 1 : xm[mu] - 1;
         cx<R> v[3][3];
-        load_link<P>(lk, it.gV, mu, link_row(it, xm, p ^ 1), v);
+        load_link<P>(it.links, it.gV, d >> 1, row, v);
 #pragma unroll
         for (int i = 0; i < 3; i++)
 #pragma unroll
             for (int j = 0; j < 3; j++) u[i][j] = f * conj(v[j][i]);
     }
-    return local_lex(it, kn) >> 1;
+    return nb;
 }
 
 // acc += f (1 -/+ g_mu) u psi for hop D (compile-time), link u already

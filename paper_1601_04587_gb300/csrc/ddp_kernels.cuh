@@ -7,6 +7,7 @@
 
 #include "ddp_device.cuh"
 #include "clover.cuh"
+#include "fx64.cuh"
 
 namespace ddp {
 
@@ -206,14 +207,17 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
             cw = -R(1) / (R(2) * kap);
             ca = R(0.5);
         }
-#pragma unroll
-        for (int j = 0; j < 24; j++) o[j] = cw * w[j] + ca * h[j];
-        if (clov && EPI == EPI_RHS) clover_apply<R>(it.clovinv, it.gV, row, o);
         if (EPI == EPI_RESID) {
-            load_spinor<P>(a.v2, i, w);
+            // two multiply-adds a component (the FP64 pipe is this kernel's scarce unit)
+            R e[24];
+            load_spinor<P>(a.v2, i, e);
 #pragma unroll
-            for (int j = 0; j < 24; j++) o[j] += w[j];
+            for (int j = 0; j < 24; j++) o[j] = fma(ca, h[j], fma(cw, w[j], e[j]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 24; j++) o[j] = cw * w[j] + ca * h[j];
         }
+        if (clov && EPI == EPI_RHS) clover_apply<R>(it.clovinv, it.gV, row, o);
         if (DOT == DOT_TS) {
             // (t, s) = sum conj(t) s with t = out, s = v1 (reload v1: w was reused)
             R s1[24];
@@ -243,26 +247,20 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
     }
 }
 
-// A staged link in shared memory: 9 complex, one 8-byte (FP32 compute) or
-// 16-byte (FP64) access each.
-template <typename R>
-__device__ __forceinline__ void put_link(R *d, const cx<R> u[3][3]) {
-    using V2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
-    V2 *q = reinterpret_cast<V2 *>(d);
+// A staged link in shared memory: 9 complex, one 8-byte access each.
+__device__ __forceinline__ void put_link(float *d, const cx<float> u[3][3]) {
+    float2 *q = reinterpret_cast<float2 *>(d);
 #pragma unroll
-    for (int k = 0; k < 9; k++) q[k] = V2{u[k / 3][k % 3].re, u[k / 3][k % 3].im};
+    for (int k = 0; k < 9; k++) q[k] = make_float2(u[k / 3][k % 3].re, u[k / 3][k % 3].im);
 }
-template <typename R>
-__device__ __forceinline__ void get_link(const R *d, cx<R> u[3][3]) {
-    using V2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
-    const V2 *q = reinterpret_cast<const V2 *>(d);
+__device__ __forceinline__ void get_link(const float *d, cx<float> u[3][3]) {
+    const float2 *q = reinterpret_cast<const float2 *>(d);
 #pragma unroll
     for (int k = 0; k < 9; k++) {
-        const V2 c = q[k];
+        const float2 c = q[k];
         u[k / 3][k % 3] = mk(c.x, c.y);
     }
 }
-
 
 template <class P, int EPI, int DOT, bool CLOV = false>
 // Resident blocks per SM the register budget of the 32- and 16-bit stencils is fitted to
@@ -271,7 +269,7 @@ template <class P, int EPI, int DOT, bool CLOV = false>
 #define DDP_HOP_MINB 3
 #endif
 
-__global__ void __launch_bounds__(384, sizeof(typename P::real) == 8 ? 1 : DDP_HOP_MINB) k_hop(HopArgs a) {
+__global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
     using R = typename P::real;
     constexpr int TSMAX = HOP_TS;
     __shared__ Item it;
@@ -886,6 +884,184 @@ __global__ void k_unpack_low(PackArgs a, FieldView le, FieldView lo) {
     double2 *u = a.uout + ((int64_t)col * n + l) * 12;
 #pragma unroll
     for (int j = 0; j < 12; j++) u[j] = make_double2((double)v[2 * j], (double)v[2 * j + 1]);
+}
+
+// ------------------------------------------------ FP64 hopping on the integer pipe
+
+// An FP64 field into block fixed point (fx64.cuh), one pass; a.skip as in HopArgs.
+struct FxArgs {
+    Launch L;
+    FieldView in, fx;
+    const SolveState *st;
+    int skip;
+};
+
+static __global__ void __launch_bounds__(384) k_to_fx(FxArgs a) {
+    __shared__ Item it;
+    load_item(a.L, it);
+    const TileCoord tc = tile_coord(it, a.L);
+    if (!tc.valid) return;
+    if (a.skip) {
+        const SolveState &S = a.st[it.solve0 + tc.col];
+        if ((a.skip == 1) ? !S.active : S.outer_done) return;
+    }
+    double v[24];
+    load_spinor<PF64>(a.in, tc.cb + tc.h, v);
+    fx_store_doubles(a.fx, tc.cb + tc.h, v);
+}
+
+// k_hop at FP64 accuracy: a.in is in block fixed point, the epilogue and its operands are FP64
+// (OUTFX: the plain sums are stored in block fixed point instead, for the next hop).  Blocks as
+// k_hop: the oriented links of a 32-site tile are staged once, as integers, for the columns.
+// About 4300 integer instructions per site-column, 1728 of them multiply-adds, instead of 864 on
+// the FP64 pipe at 1/32 of the rate: 2.10 -> 0.59 ms for the plain sums of 110592 sites x 12
+// columns (16x24^3, one parity).  160 registers (48 of sums, 48 of a neighbour, 24 of its
+// projection), so one block of 12 warps per SM: the multiply-add pipe is 47% busy, the rest waits
+// for neighbours (L2) and for the staging.
+template <int EPI, int DOT, bool CLOV, bool OUTFX>
+__global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
+    constexpr int TS = HOP_TS;
+    __shared__ Item it;
+    __shared__ int s_nb[8 * TS];
+    __shared__ __align__(16) int4 s_u[8 * TS * 9];
+    load_item(a.L, it);
+    if (a.skip) {
+        const int cg = (blockIdx.x - it.blk0) / it.ntiles;
+        const int col = cg * a.L.CG + (int)threadIdx.x;
+        int live = 0;
+        if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
+            const SolveState &S = a.st[it.solve0 + col];
+            live = (a.skip == 1) ? S.active : !S.outer_done;
+        }
+        if (!__syncthreads_or(live)) return;
+    }
+    {
+        const int tile = (blockIdx.x - it.blk0) % it.ntiles;
+        for (int q = threadIdx.x; q < 8 * TS; q += blockDim.x) {
+            const int d = q / TS, h = tile * TS + (q - d * TS);
+            int nb = -1;
+            if (h < it.nh) {
+                int64_t row = 0;
+                bool neg;
+                nb = hop_geometry(it, h, a.p, d, row, neg);
+                if (nb >= 0) {
+                    const double2 *l = reinterpret_cast<const double2 *>(it.links64) + (int64_t)(d >> 1) * 9 * it.gV + row;
+                    const bool adj = d & 1;
+#pragma unroll
+                    for (int j = 0; j < 9; j++) {
+                        const double2 c = __ldg(l + j * it.gV);
+                        long long re = fx_link(c.x), im = fx_link(c.y);
+                        if (neg) re = -re;
+                        if (neg != adj) im = -im;  // the adjoint's conjugate, and the sign
+                        int4 e;
+                        fx_split(re, e.x, e.y);
+                        fx_split(im, e.z, e.w);
+                        s_u[q * 9 + (adj ? 3 * (j % 3) + j / 3 : j)] = e;
+                    }
+                }
+            }
+            s_nb[q] = nb;
+        }
+    }
+    __syncthreads();
+    TileCoord tc = tile_coord(it, a.L);
+    if (a.skip && tc.valid) {
+        const SolveState &S = a.st[it.solve0 + tc.col];
+        if ((a.skip == 1) ? !S.active : S.outer_done) tc.valid = false;
+    }
+    double cre = 0, cim = 0, nn = 0;
+    if (tc.valid) {
+        const int sl = tc.h - tc.tile * TS;
+        int e[8], top = FX_ZERO;
+#pragma unroll
+        for (int d = 0; d < 8; d++) {
+            const int nb = s_nb[d * TS + sl];
+            e[d] = nb >= 0 ? __ldg(fx_exponents(a.in) + tc.cb + nb) : FX_ZERO;
+            top = max(top, e[d]);
+        }
+        if (top != FX_RAW) {
+            long long sum[24];
+#pragma unroll
+            for (int j = 0; j < 24; j++) sum[j] = 0;
+#define DDP_FX_STEP(D)                                                                        \
+            {                                                                                 \
+                const int nb = s_nb[(D) * TS + sl];                                           \
+                if (nb >= 0) {                                                                \
+                    const int4 *b = reinterpret_cast<const int4 *>(a.in.p) + tc.cb + nb;      \
+                    int4 v[12];                                                               \
+                    _Pragma("unroll") for (int j = 0; j < 12; j++) v[j] = __ldg(b + j * a.in.stride); \
+                    fx_hop_step<D>(v, s_u + ((D) * TS + sl) * 9, sum, min(62, top - e[D]));   \
+                }                                                                             \
+            }
+            DDP_FX_STEP(0)
+            DDP_FX_STEP(1)
+            DDP_FX_STEP(2)
+            DDP_FX_STEP(3)
+            DDP_FX_STEP(4)
+            DDP_FX_STEP(5)
+            DDP_FX_STEP(6)
+            DDP_FX_STEP(7)
+#undef DDP_FX_STEP
+            if (OUTFX) {
+                fx_store_sums(a.out, tc.cb + tc.h, sum, top - FX_LINK);
+            } else {
+                cx<double> acc[4][3];
+#pragma unroll
+                for (int j = 0; j < 12; j++)
+                    acc[j / 3][j % 3] = mk(fx_value(sum[2 * j], top - FX_LINK), fx_value(sum[2 * j + 1], top - FX_LINK));
+                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, cre, cim, nn);
+            }
+        } else {
+            double o[24];
+            fx_slow<TS>(a.in, tc.cb, s_nb + sl, s_u + sl * 9, o);
+            if (OUTFX) {
+                fx_store_doubles(a.out, tc.cb + tc.h, o);
+            } else {
+                cx<double> acc[4][3];
+                for (int j = 0; j < 12; j++) acc[j / 3][j % 3] = mk(o[2 * j], o[2 * j + 1]);
+                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, cre, cim, nn);
+            }
+        }
+    }
+    if (DOT != DOT_NONE) block_partials(it, a.L, tc, cre, cim, nn, a.part, DOT == DOT_RHAT || DOT == DOT_TS,
+                                        DOT == DOT_TS || DOT == DOT_NORM);
+}
+
+// User layout <-> block fixed point (the stencil powers); unpacking multiplies by s.
+static __global__ void k_pack_fx(PackArgs a, FieldView le, FieldView lo) {
+    int64_t n = 2 * (int64_t)a.it.nh;
+    int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (g >= n * a.it.ncol) return;
+    int col = (int)(g / n);
+    int l = (int)(g - (int64_t)col * n);
+    int k[4];
+    local_coords(a.it, l, k);
+    int par = (a.it.par_o + k[0] + k[1] + k[2] + k[3]) & 1;
+    const double2 *u = a.user + ((int64_t)col * n + l) * 12;
+    double v[24];
+#pragma unroll
+    for (int j = 0; j < 12; j++) {
+        double2 c = u[j];
+        v[2 * j] = c.x;
+        v[2 * j + 1] = c.y;
+    }
+    fx_store_doubles(par ? lo : le, a.it.fbase + (int64_t)col * a.it.nh + (l >> 1), v);
+}
+
+static __global__ void k_unpack_fx(PackArgs a, FieldView le, FieldView lo, double s) {
+    int64_t n = 2 * (int64_t)a.it.nh;
+    int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (g >= n * a.it.ncol) return;
+    int col = (int)(g / n);
+    int l = (int)(g - (int64_t)col * n);
+    int k[4];
+    local_coords(a.it, l, k);
+    int par = (a.it.par_o + k[0] + k[1] + k[2] + k[3]) & 1;
+    double v[24];
+    fx_load_doubles(par ? lo : le, a.it.fbase + (int64_t)col * a.it.nh + (l >> 1), v);
+    double2 *u = a.uout + ((int64_t)col * n + l) * 12;
+#pragma unroll
+    for (int j = 0; j < 12; j++) u[j] = make_double2(s * v[2 * j], s * v[2 * j + 1]);
 }
 
 }  // namespace ddp

@@ -23,10 +23,35 @@
 
 namespace ddp {
 
-// One launch of the hopping term (CL: with the clover term of the items that have one).
+// One application of the hopping term (CL: with the clover term of the items that have one).
+// FP64: the input is brought into block fixed point in fx (a field of its size) first.
+// Returns the number of kernels launched.
 template <class Q, int EPI, int DOT, bool CL = false>
-inline void launch_hop(ddp_ctx *ctx, int nblocks, int threads, const HopArgs &a) {
-    k_hop<Q, EPI, DOT, CL><<<nblocks, threads, 0, ctx->stream>>>(a);
+inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const FieldView &fx) {
+    if constexpr (Q::IS64) {
+        FxArgs c;
+        c.L = a.L;
+        c.in = a.in;
+        c.fx = fx;
+        c.st = a.st;
+        c.skip = a.skip;
+        k_to_fx<<<nblocks, threads, 0, ctx->stream>>>(c);
+        a.in = fx;
+        k_hop_fx<EPI, DOT, CL, false><<<nblocks, threads, 0, ctx->stream>>>(a);
+        return 2;
+    } else {
+        (void)fx;
+        k_hop<Q, EPI, DOT, CL><<<nblocks, threads, 0, ctx->stream>>>(a);
+        return 1;
+    }
+}
+
+template <class Q, int EPI, int DOT, bool CL>
+inline const void *hop_kernel() {
+    if constexpr (Q::IS64)
+        return (const void *)k_hop_fx<EPI, DOT, CL, false>;
+    else
+        return (const void *)k_hop<Q, EPI, DOT, CL>;
 }
 
 // Preferred shared-memory carveout of the inner-loop stencils (percent of the unified
@@ -34,14 +59,11 @@ inline void launch_hop(ddp_ctx *ctx, int nblocks, int threads, const HopArgs &a)
 template <class Q, bool CL>
 inline cudaError_t set_hop_carveout(int percent) {
     if (percent < 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_hop<Q, EPI_PLAIN, DOT_NONE, CL>,
-                                         cudaFuncAttributePreferredSharedMemoryCarveout, percent);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_hop<Q, EPI_MHAT, DOT_RHAT, CL>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 percent);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_hop<Q, EPI_MHAT, DOT_TS, CL>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 percent);
+    const void *k[3] = {hop_kernel<Q, EPI_PLAIN, DOT_NONE, CL>(), hop_kernel<Q, EPI_MHAT, DOT_RHAT, CL>(),
+                        hop_kernel<Q, EPI_MHAT, DOT_TS, CL>()};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 3 && e == cudaSuccess; i++)
+        e = cudaFuncSetAttribute(k[i], cudaFuncAttributePreferredSharedMemoryCarveout, percent);
     return e;
 }
 
@@ -52,6 +74,9 @@ struct Engine {
     Plan plan;
     FieldView be, bo, xe, xo, re64, ro64;      // FP64
     FieldView r, rh, p, v, s, t, xi, tmp, ro;  // storage format P (rh: ShadowOf<P>)
+    // block fixed-point input of an FP64 hop, over fields that are dead at the time: the inner
+    // fields during a true residual, the FP64 residual during the inner loop of the FP64 path
+    FieldView fx_outer, fx_inner;
     Partials A, B;
     Item *d_items = nullptr;
     SolveState *d_st = nullptr;
@@ -89,8 +114,7 @@ struct Engine {
 
     template <class Q, int EPI, int DOT, bool CL = false>
     void hop(const HopArgs &a) {
-        launch_hop<Q, EPI, DOT, CL>(ctx, plan.nblocks, threads, a);
-        launches++;
+        launches += launch_hop<Q, EPI, DOT, CL>(ctx, plan.nblocks, threads, a, EPI == EPI_RESID ? fx_outer : fx_inner);
     }
 
     template <class Q, int OP>
@@ -221,7 +245,7 @@ struct Engine {
     int run_inner() {
         // launches per iteration: 4 stencils, 3 vector updates, 3 scalar-recurrence
         // kernels (the last of which also runs the loop control)
-        const long per_iter = 10;
+        const long per_iter = P::IS64 ? 14 : 10;  // FP64 stencils: conversion and hop
         if (ctx->prm.use_conditional) {
             DDP_CUDA(ctx, cudaGraphLaunch(loop_exec, ctx->stream));
         } else {
@@ -266,6 +290,18 @@ struct Engine {
         xi = carve_field<P>(a, cap);
         tmp = carve_field<P>(a, cap);
         ro = carve_field<P>(a, cap);
+        auto fx_over = [&](FieldView first) {
+            FieldView f;
+            f.stride = cap;
+            f.p = first.p;
+            f.scale = reinterpret_cast<float *>((char *)first.p + (size_t)cap * PFX::NCH * sizeof(PFX::chunk));
+            return f;
+        };
+        // 196 bytes a site-column: within r, rh, p, v, s, t (240 at the least, BF16) and within
+        // re64, ro64 (384), which lie one after another
+        static_assert((P::NCH * 5 + ShadowOf<P>::type::NCH) * 16 >= PFX::NCH * 16 + 4, "fixed-point field over the inner fields");
+        fx_outer = fx_over(r);
+        fx_inner = fx_over(re64);
         A.c = (double2 *)a.take(npart * sizeof(double2));
         A.n = (double *)a.take(npart * sizeof(double));
         B.c = (double2 *)a.take(npart * sizeof(double2));
@@ -469,12 +505,14 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
     Plan plan;
     make_plan(jobs, prec, ctx->prm, plan);
     const int64_t NF = plan.nfield;
-    size_t need = 4 * field_bytes<P>(NF) + sizeof(Item) + 1024;
+    size_t need = 4 * field_bytes<P>(NF) + (P::IS64 ? field_bytes<PFX>(NF) : 0) + sizeof(Item) + 1024;
     DDP_CUDA(ctx, ctx->scratch.reserve(need));
     Arena &a = ctx->scratch;
     a.reset();
     FieldView ie = carve_field<P>(a, NF), io = carve_field<P>(a, NF);
     FieldView oe = carve_field<P>(a, NF), oo = carve_field<P>(a, NF);
+    FieldView fx = {nullptr, nullptr, 0};
+    if (P::IS64) fx = carve_field<PFX>(a, NF);
     Item *d_items = (Item *)a.take(sizeof(Item));
     cudaStream_t st = ctx->stream;
     DDP_CUDA(ctx, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(Item), cudaMemcpyHostToDevice, st));
@@ -506,9 +544,9 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
     h.v1 = ie;
     auto dirac = [&]() {
         if (job.clov)
-            launch_hop<P, EPI_DIRAC, DOT_NONE, true>(ctx, plan.nblocks, plan.TS * plan.CG, h);
+            ctx->launches += launch_hop<P, EPI_DIRAC, DOT_NONE, true>(ctx, plan.nblocks, plan.TS * plan.CG, h, fx);
         else
-            launch_hop<P, EPI_DIRAC, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h);
+            ctx->launches += launch_hop<P, EPI_DIRAC, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h, fx);
     };
     dirac();
     h.p = 1;
@@ -517,76 +555,7 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
     h.v1 = io;
     dirac();
     k_unpack_low<P><<<nb, 256, 0, st>>>(pa, oe, oo);
-    ctx->launches += 4;
-    DDP_CUDA(ctx, cudaGetLastError());
-    return DDP_OK;
-}
-
-// out *= s over n complex numbers.
-static __global__ void k_scale_complex(double2 *out, int64_t n, double s) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = make_double2(s * out[i].x, s * out[i].y);
-}
-
-// out = (kappa D_hop)^p psi on a domain in FP64 (Eq. HPEtr with the
-// Dirichlet-restricted hopping term of Sec. 2): p pairs of plain hop launches
-// (odd -> even, even -> odd) between two even-odd field pairs, then kappa^p
-// applied once to the unpacked result.  psi and out: device pointers.
-template <class P>
-int hop_power_impl(ddp_ctx *ctx, const Job &job, int p, const double *psi, double *out) {
-    static_assert(P::IS64, "the hopping power is an FP64 operation");
-    std::vector<Job> jobs(1, job);
-    Plan plan;
-    make_plan(jobs, DDP_PREC_FP64, ctx->prm, plan);
-    const int64_t NF = plan.nfield;
-    size_t need = 4 * field_bytes<P>(NF) + sizeof(Item) + 1024;
-    DDP_CUDA(ctx, ctx->scratch.reserve(need));
-    Arena &a = ctx->scratch;
-    a.reset();
-    FieldView f[2][2] = {{carve_field<P>(a, NF), carve_field<P>(a, NF)}, {carve_field<P>(a, NF), carve_field<P>(a, NF)}};
-    Item *d_items = (Item *)a.take(sizeof(Item));
-    cudaStream_t st = ctx->stream;
-    DDP_CUDA(ctx, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(Item), cudaMemcpyHostToDevice, st));
-    PackArgs pa;
-    memset(&pa, 0, sizeof(pa));
-    pa.it = plan.items[0];
-    pa.user = (const double2 *)psi;
-    pa.uout = (double2 *)out;
-    const int64_t nt = 2 * (int64_t)pa.it.nh * pa.it.ncol;
-    const unsigned nb = (unsigned)((nt + 255) / 256);
-    k_pack_low<P><<<nb, 256, 0, st>>>(pa, f[0][0], f[0][1]);
-    Launch L;
-    L.items = d_items;
-    L.nitems = 1;
-    L.TS = plan.TS;
-    L.CG = plan.CG;
-    FieldView none = {nullptr, nullptr, 0};
-    HopArgs h;
-    h.st = nullptr;
-    h.skip = 0;
-    h.L = L;
-    h.v1 = none;
-    h.v2 = none;
-    h.rh = none;
-    h.part.c = nullptr;
-    h.part.n = nullptr;
-    int cur = 0;
-    for (int k = 0; k < p; k++) {
-        const int nxt = cur ^ 1;
-        h.p = 0;
-        h.in = f[cur][1];
-        h.out = f[nxt][0];
-        launch_hop<P, EPI_PLAIN, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h);
-        h.p = 1;
-        h.in = f[cur][0];
-        h.out = f[nxt][1];
-        launch_hop<P, EPI_PLAIN, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h);
-        cur = nxt;
-    }
-    k_unpack_low<P><<<nb, 256, 0, st>>>(pa, f[cur][0], f[cur][1]);
-    const int64_t nc = (int64_t)pa.it.ncol * 2 * pa.it.nh * 12;
-    k_scale_complex<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>((double2 *)out, nc, std::pow(job.kappa, p));
-    ctx->launches += 3 + 2 * (long)p;
+    ctx->launches += 2;
     DDP_CUDA(ctx, cudaGetLastError());
     return DDP_OK;
 }
@@ -607,12 +576,15 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     Plan plan;
     make_plan(jobs, prec, ctx->prm, plan);
     const int64_t NF = plan.nfield;
-    size_t need = 4 * field_bytes<P>(NF) + 2 * ((size_t)plan.npart * 24 + 1024) + sizeof(Item) + 1024;
+    size_t need = 4 * field_bytes<P>(NF) + (P::IS64 ? field_bytes<PFX>(NF) : 0) + 2 * ((size_t)plan.npart * 24 + 1024) +
+                  sizeof(Item) + 1024;
     DDP_CUDA(ctx, ctx->scratch.reserve(need));
     Arena &a = ctx->scratch;
     a.reset();
     FieldView in = carve_field<P>(a, NF), v1 = carve_field<P>(a, NF), rhv = carve_field<P>(a, NF),
               out = carve_field<P>(a, NF);
+    FieldView fx = {nullptr, nullptr, 0};
+    if (P::IS64) fx = carve_field<PFX>(a, NF);
     Partials A;
     A.c = (double2 *)a.take(plan.npart * sizeof(double2));
     A.n = (double *)a.take(plan.npart * sizeof(double));
@@ -648,11 +620,11 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     DDP_CUDA(ctx, (set_hop_carveout<P, false>(carveout_for(ctx->prm, prec))));
     auto launch = [&]() {
         if (kernel == DDP_HOP_PLAIN)
-            launch_hop<P, EPI_PLAIN, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h);
+            ctx->launches += launch_hop<P, EPI_PLAIN, DOT_NONE>(ctx, plan.nblocks, plan.TS * plan.CG, h, fx);
         else if (kernel == DDP_HOP_SCHUR_RHAT)
-            launch_hop<P, EPI_MHAT, DOT_RHAT>(ctx, plan.nblocks, plan.TS * plan.CG, h);
+            ctx->launches += launch_hop<P, EPI_MHAT, DOT_RHAT>(ctx, plan.nblocks, plan.TS * plan.CG, h, fx);
         else
-            launch_hop<P, EPI_MHAT, DOT_TS>(ctx, plan.nblocks, plan.TS * plan.CG, h);
+            ctx->launches += launch_hop<P, EPI_MHAT, DOT_TS>(ctx, plan.nblocks, plan.TS * plan.CG, h, fx);
     };
     cudaEvent_t e0, e1;
     DDP_CUDA(ctx, cudaEventCreate(&e0));
@@ -667,7 +639,6 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     DDP_CUDA(ctx, cudaGetLastError());
-    ctx->launches += 3 + iters;
     *ms = t / iters;
     const double site_cols = (double)plan.items[0].nh * job.ncol;
     const double spinor = (double)sizeof(typename P::chunk) * P::NCH + (P::SCALED ? 4.0 : 0.0);
