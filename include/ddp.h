@@ -328,7 +328,8 @@ int ddp_get_param(const ddp_ctx *ctx, const char *name, double *value);
 typedef enum {
     DDP_HOP_PLAIN = 0,        /* tmp = H_oe p (odd output sites) */
     DDP_HOP_SCHUR_RHAT = 1,   /* v = p - kappa^2 H_eo tmp, with the (rh, v) partial sums */
-    DDP_HOP_SCHUR_TS = 2      /* t = s - kappa^2 H_eo tmp, with the (t, s), (t, t) partial sums */
+    DDP_HOP_SCHUR_TS = 2      /* t = s - kappa^2 H_eo tmp, with the partial sums of (t, s), (t, t),
+                                 (s, s), (rh, s) and (rh, t) */
 } ddp_hop_kernel;
 
 /* Average duration (ms) of one inner-loop stencil variant (ddp_hop_kernel) on
@@ -337,8 +338,8 @@ typedef enum {
  * launches; bytes_per_launch receives the variant's algorithmic HBM bytes:
  * the spinors it reads or writes once per output site-column (2 for PLAIN,
  * 4 for SCHUR_RHAT, of which the shadow residual rh is counted in its own
- * storage: BF16 for FP32 storage, 3 for SCHUR_TS) plus the 8 links touching
- * every output site once for all columns. */
+ * storage: BF16 for FP32 storage, 3 for SCHUR_TS, whose read of rh is not
+ * counted) plus the 8 links touching every output site once for all columns. */
 int ddp_time_hop(ddp_ctx *ctx, int domain_id, double kappa, int ncol, int precision, int kernel, int iters,
                  float *ms_per_launch, double *bytes_per_launch);
 

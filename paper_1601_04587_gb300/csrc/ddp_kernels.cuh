@@ -25,13 +25,17 @@ struct SolveState {
     double delta;    // inner relative tolerance of the cycle
     double tol;      // requested relative tolerance
     double floor_delta;  // smallest useful inner tolerance of the storage format
-    int active;      // inner iteration running
+    int active;      // inner iteration: 1 running, 2 its last update of x and r pending, 0 done
     int iters;       // inner iterations of the current cycle
     int total_iters; // inner iterations over all cycles
     int status;      // inner: 0 running, 1 converged, 2 breakdown, 3 iteration cap, 4 skipped
     int outer_done;  // 1 once |eta - D x| <= tol |eta|
     int item, col;
     int maxit;       // inner iteration cap per cycle
+    // from the column's item, so that the scalar kernels reach the partials in one step
+    int ntiles;
+    int64_t pbase;   // first partial slot of the column
+    double kappa;
 };
 
 struct LoopCtl {
@@ -39,14 +43,14 @@ struct LoopCtl {
     int iter;
     int maxit;
     int pad;          // host-polled loop: 1 while the loop continues
-    int done_blocks;  // blocks of k_fin<FIN_RHO> finished in this iteration
+    int done_blocks;  // blocks of k_fin<FIN_OMEGA> finished in this iteration
 };
 
-// Reduction partial buffers: complex and real, per (item, column, tile).
+// Reduction partials: NV sums per (item, column, tile) at d[slot * NV + k], NV = dot_sums(DOT).
 struct Partials {
-    double2 *c;
-    double *n;
+    double *d;
 };
+constexpr int PART_MAX = 8;  // largest NV
 
 // Epilogues of the hopping kernel (acc = the hopping sum, v1, v2 operands at the
 // output site; T / T^-1 the clover matrices of the output site, identity without
@@ -55,7 +59,12 @@ struct Partials {
 //   AXPY_K v1 + kappa T^-1 acc      RHS   T^-1 (v1 + kappa acc)
 //   DIRAC  T v1 / (2 kappa) - acc/2 RESID v2 - T v1 / (2 kappa) + acc/2
 enum Epi { EPI_PLAIN = 0, EPI_MHAT = 1, EPI_AXPY_K = 2, EPI_DIRAC = 3, EPI_RESID = 4, EPI_RHS = 5 };
+// Dot products of the epilogue (o the output, v1 its operand):
+//   RHAT (rh, o)     NORM (o, o)     TS (o, v1), (rh, v1), (rh, o), (o, o), (v1, v1)
 enum Dot { DOT_NONE = 0, DOT_RHAT = 1, DOT_TS = 2, DOT_NORM = 3 };
+__host__ __device__ constexpr int dot_sums(int dot) {
+    return dot == DOT_RHAT ? 2 : dot == DOT_TS ? PART_MAX : dot == DOT_NORM ? 1 : 0;
+}
 
 struct HopArgs {
     Launch L;
@@ -64,11 +73,16 @@ struct HopArgs {
     FieldView out;  // output (parity p)
     FieldView v1;   // same-parity operand of the epilogue
     FieldView v2;   // second same-parity operand (EPI_RESID: eta)
-    FieldView rh;   // shadow residual for DOT_RHAT
+    FieldView rh;   // shadow residual for DOT_RHAT and DOT_TS
     Partials part;
     const SolveState *st;  // skip 1: leave columns whose inner solve is not active untouched;
     int skip;              // skip 2: leave columns whose outer solve has converged untouched
 };
+
+// Whether a kernel with the given skip mode leaves the column alone.
+__device__ __forceinline__ bool skipped(const SolveState &S, int skip) {
+    return (skip == 1) ? S.active != 1 : (skip == 2) && S.outer_done;
+}
 
 // Tiles are exactly HOP_TS = 32 sites (one warp per column of a tile); a
 // block holds at most HOP_MAX_CG = 12 columns.  The kernels use the tile size
@@ -109,47 +123,29 @@ __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L)
     return t;
 }
 
-// Block reduction of (complex, real) per column.  Each thread's products and
-// the 32-lane warp sums are formed in the compute precision R (FP32 for the
-// low-precision formats: FP64 arithmetic is a small fraction of GB300's FP32
-// rate); the sums across warps and, in the scalar kernels, across blocks are
-// FP64.  Lanes of a warp share one column (TS = 32); warps of the same
-// column are added in warp order.  Fixed order: results do not depend on
-// the batch around them.
-template <typename R>
-__device__ __forceinline__ void block_partials(const Item &it, const Launch &L, const TileCoord &tc, R cre, R cim,
-                                               R nn, Partials part, bool want_c, bool want_n, int blk = -1) {
-    __shared__ double s_re[32], s_im[32], s_nn[32];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (want_c) {
-        cre = warp_sum(cre);
-        cim = warp_sum(cim);
-    }
-    if (want_n) nn = warp_sum(nn);
-    if (lane == 0) {
-        s_re[warp] = (double)cre;
-        s_im[warp] = (double)cim;
-        s_nn[warp] = (double)nn;
-    }
-    __syncthreads();
-    constexpr int wpc = HOP_TS >> 5;  // warps per column
-    if ((int)threadIdx.x < L.CG) {
-        int cl = threadIdx.x;
-        int lb = (blk < 0 ? (int)blockIdx.x : blk) - it.blk0;
-        int cg = lb / it.ntiles;
-        int col = cg * L.CG + cl;
-        if (col < it.ncol) {
-            double a = 0, b = 0, c = 0;
-            for (int w = cl * wpc; w < (cl + 1) * wpc; w++) {
-                a += s_re[w];
-                b += s_im[w];
-                c += s_nn[w];
-            }
-            int64_t idx = it.pbase + (int64_t)col * it.ntiles + tc.tile;
-            if (want_c) part.c[idx] = make_double2(a, b);
-            if (want_n) part.n[idx] = c;
+// Sums of NV values over the 32 sites of a tile, which are one warp of one column.  Each
+// thread's products and the warp's sums are formed in the compute precision R (FP32 for the
+// low-precision formats: FP64 arithmetic is a small fraction of GB300's FP32 rate); the sums over
+// tiles, in the scalar kernels, are FP64.  Fixed order: results do not depend on the batch
+// around them.  The lanes split the values as the distance halves (9 shuffles for 8 values, not
+// 40): value k ends in lanes k * 32 / NV and following.
+template <int NV, typename R>
+__device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &tc, R v[NV], Partials part) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int n = NV; n > 1; n >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < n / 2; i++) {
+            const R keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
+#pragma unroll
+    for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    if (tc.col < it.ncol && (lane & (32 / NV - 1)) == 0)
+        part.d[(it.pbase + (int64_t)tc.col * it.ntiles + tc.tile) * NV + lane / (32 / NV)] = (double)v[0];
 }
 
 __device__ __forceinline__ void load_item(const Launch &L, Item &dst) {
@@ -166,8 +162,8 @@ __device__ __forceinline__ void load_item(const Launch &L, Item &dst) {
 // operands, stored in the storage format, plus the requested dot products.
 template <class P, int EPI, int DOT, bool CLOV>
 __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item &it, const TileCoord &tc,
-                                                   const cx<typename P::real> acc[4][3], typename P::real &cre,
-                                                   typename P::real &cim, typename P::real &nn) {
+                                                   const cx<typename P::real> acc[4][3],
+                                                   typename P::real sums[PART_MAX]) {
     using R = typename P::real;
     R o[24];
     int64_t i = tc.cb + tc.h;
@@ -218,16 +214,6 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
             for (int j = 0; j < 24; j++) o[j] = cw * w[j] + ca * h[j];
         }
         if (clov && EPI == EPI_RHS) clover_apply<R>(it.clovinv, it.gV, row, o);
-        if (DOT == DOT_TS) {
-            // (t, s) = sum conj(t) s with t = out, s = v1 (reload v1: w was reused)
-            R s1[24];
-            load_spinor<P>(a.v1, i, s1);
-#pragma unroll
-            for (int j = 0; j < 12; j++) {
-                cre += o[2 * j] * s1[2 * j] + o[2 * j + 1] * s1[2 * j + 1];
-                cim += o[2 * j] * s1[2 * j + 1] - o[2 * j + 1] * s1[2 * j];
-            }
-        }
     }
     store_spinor<P>(a.out, i, o);
     if (DOT == DOT_RHAT) {
@@ -235,15 +221,35 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
         load_spinor<typename ShadowOf<P>::type>(a.rh, i, r);
 #pragma unroll
         for (int j = 0; j < 12; j++) {
-            cre += r[2 * j] * o[2 * j] + r[2 * j + 1] * o[2 * j + 1];
-            cim += r[2 * j] * o[2 * j + 1] - r[2 * j + 1] * o[2 * j];
+            sums[0] += r[2 * j] * o[2 * j] + r[2 * j + 1] * o[2 * j + 1];
+            sums[1] += r[2 * j] * o[2 * j + 1] - r[2 * j + 1] * o[2 * j];
+        }
+    }
+    if (DOT == DOT_TS) {
+        // t = out, s = v1 (loaded again: its registers were reused)
+        R q[24];
+        load_spinor<P>(a.v1, i, q);
+#pragma unroll
+        for (int j = 0; j < 12; j++) {
+            sums[0] += o[2 * j] * q[2 * j] + o[2 * j + 1] * q[2 * j + 1];  // (t, s)
+            sums[1] += o[2 * j] * q[2 * j + 1] - o[2 * j + 1] * q[2 * j];
+            sums[7] += q[2 * j] * q[2 * j] + q[2 * j + 1] * q[2 * j + 1];  // (s, s)
+        }
+        R r[24];
+        load_spinor<typename ShadowOf<P>::type>(a.rh, i, r);
+#pragma unroll
+        for (int j = 0; j < 12; j++) {
+            sums[2] += r[2 * j] * q[2 * j] + r[2 * j + 1] * q[2 * j + 1];  // (rh, s)
+            sums[3] += r[2 * j] * q[2 * j + 1] - r[2 * j + 1] * q[2 * j];
+            sums[4] += r[2 * j] * o[2 * j] + r[2 * j + 1] * o[2 * j + 1];  // (rh, t)
+            sums[5] += r[2 * j] * o[2 * j + 1] - r[2 * j + 1] * o[2 * j];
         }
     }
     if (DOT == DOT_TS || DOT == DOT_NORM) {
-        R s = 0;
+        R n = 0;
 #pragma unroll
-        for (int j = 0; j < 24; j++) s += o[j] * o[j];
-        nn = s;
+        for (int j = 0; j < 24; j++) n += o[j] * o[j];
+        sums[DOT == DOT_TS ? 6 : 0] = n;
     }
 }
 
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
         int live = 0;
         if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
             const SolveState &S = a.st[it.solve0 + col];
-            live = (a.skip == 1) ? S.active : !S.outer_done;
+            live = !skipped(S, a.skip);
         }
         if (!__syncthreads_or(live)) return;
     }
@@ -321,9 +327,9 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
     TileCoord tc = tile_coord(it, a.L);
     if (a.skip && tc.valid) {
         const SolveState &S = a.st[it.solve0 + tc.col];
-        if ((a.skip == 1) ? !S.active : S.outer_done) tc.valid = false;
+        if (skipped(S, a.skip)) tc.valid = false;
     }
-    R cre = 0, cim = 0, nn = 0;
+    R sums[PART_MAX] = {};
     if (tc.valid) {
         cx<R> acc[4][3];
 #pragma unroll
@@ -352,10 +358,9 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
         DDP_HOP_STEP(6)
         DDP_HOP_STEP(7)
 #undef DDP_HOP_STEP
-        hop_store_epilogue<P, EPI, DOT, CLOV>(a, it, tc, acc, cre, cim, nn);
+        hop_store_epilogue<P, EPI, DOT, CLOV>(a, it, tc, acc, sums);
     }
-    if (DOT != DOT_NONE) block_partials(it, a.L, tc, cre, cim, nn, a.part, DOT == DOT_RHAT || DOT == DOT_TS,
-                                        DOT == DOT_TS || DOT == DOT_NORM);
+    if (DOT != DOT_NONE) warp_partials<DOT != DOT_NONE ? dot_sums(DOT) : 1>(it, tc, sums, a.part);
 }
 
 // ------------------------------------------------------------ vector updates
@@ -413,25 +418,7 @@ __device__ __forceinline__ uint4 reals_to_chunk<PF16>(const float *) {
     return make_uint4(0, 0, 0, 0);
 }
 
-// The reals of storage chunk j (of format P) of site-column i of the shadow residual,
-// stored in ShadowOf<P>.
-template <class P>
-__device__ __forceinline__ void shadow_reals(const FieldView &f, int j, int64_t i, typename P::real *v) {
-    chunk_to_reals<P>(__ldg(reinterpret_cast<const typename P::chunk *>(f.p) + j * f.stride + i), v);
-}
-template <>
-__device__ __forceinline__ void shadow_reals<PF32>(const FieldView &f, int j, int64_t i, float *v) {
-    // FP32 chunk j (reals 4j .. 4j+3) is half j % 2 of BF16 chunk j / 2
-    const uint2 c = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint4 *>(f.p) +
-                                                          (int64_t)(j >> 1) * f.stride + i) + (j & 1));
-    const float2 a0 = b2f(c.x), a1 = b2f(c.y);
-    v[0] = a0.x;
-    v[1] = a0.y;
-    v[2] = a1.x;
-    v[3] = a1.y;
-}
-
-enum BlasOp { OP_P_UPDATE = 0, OP_S_UPDATE = 1, OP_XR_UPDATE = 2, OP_INIT = 3, OP_NORM = 4 };
+enum BlasOp { OP_S_UPDATE = 1, OP_XRP_UPDATE = 2, OP_INIT = 3, OP_NORM = 4 };
 
 struct BlasArgs {
     Launch L;
@@ -441,6 +428,19 @@ struct BlasArgs {
     int skip;
 };
 
+// One complex component: x += alpha p + omega s ; s <- r = s - omega t ; p <- r + beta (p - omega v).
+template <typename R>
+__device__ __forceinline__ void xrp_update(R x[2], R p[2], R s[2], const R t[2], const R v[2], R ar, R ai, R wr, R wi,
+                                           R br, R bi) {
+    x[0] += (ar * p[0] - ai * p[1]) + (wr * s[0] - wi * s[1]);
+    x[1] += (ar * p[1] + ai * p[0]) + (wr * s[1] + wi * s[0]);
+    s[0] -= wr * t[0] - wi * t[1];
+    s[1] -= wr * t[1] + wi * t[0];
+    const R qr = p[0] - (wr * v[0] - wi * v[1]), qi = p[1] - (wr * v[1] + wi * v[0]);
+    p[0] = s[0] + (br * qr - bi * qi);
+    p[1] = s[1] + (br * qi + bi * qr);
+}
+
 template <class P, int OP>
 __global__ void __launch_bounds__(512) k_blas(BlasArgs a) {
     using R = typename P::real;
@@ -448,25 +448,11 @@ __global__ void __launch_bounds__(512) k_blas(BlasArgs a) {
     load_item(a.L, it);
     TileCoord tc = tile_coord(it, a.L);
     if (a.skip && tc.valid && !a.st[it.solve0 + tc.col].active) tc.valid = false;
-    R cre = 0, cim = 0, nn = 0;
+    R nn[1] = {0};
     if (tc.valid) {
         int64_t i = tc.cb + tc.h;
         const SolveState &S = a.st[it.solve0 + tc.col];
-        if (OP == OP_P_UPDATE) {  // p = r + beta (p - omega v)
-            R r[24], p[24], v[24];
-            load_spinor<P>(a.r, i, r);
-            load_spinor<P>(a.p, i, p);
-            load_spinor<P>(a.v, i, v);
-            const R br = (R)S.beta.x, bi = (R)S.beta.y, wr = (R)S.omega.x, wi = (R)S.omega.y;
-#pragma unroll
-            for (int j = 0; j < 12; j++) {
-                R qr = p[2 * j] - (wr * v[2 * j] - wi * v[2 * j + 1]);
-                R qi = p[2 * j + 1] - (wr * v[2 * j + 1] + wi * v[2 * j]);
-                p[2 * j] = r[2 * j] + (br * qr - bi * qi);
-                p[2 * j + 1] = r[2 * j + 1] + (br * qi + bi * qr);
-            }
-            store_spinor<P>(a.p, i, p);
-        } else if (OP == OP_S_UPDATE) {  // s = r - alpha v
+        if (OP == OP_S_UPDATE) {  // s = r - alpha v
             R r[24], v[24];
             load_spinor<P>(a.r, i, r);
             load_spinor<P>(a.v, i, v);
@@ -477,72 +463,54 @@ __global__ void __launch_bounds__(512) k_blas(BlasArgs a) {
                 r[2 * j + 1] -= ar * v[2 * j + 1] + ai * v[2 * j];
             }
             store_spinor<P>(a.s, i, r);
-        } else if (OP == OP_XR_UPDATE && !P::SCALED) {
-            // x += alpha p + omega s ; r = s - omega t ; dots -- one storage chunk at a
-            // time (the fields do not alias), so few registers and many loads in flight
+        } else if (OP == OP_XRP_UPDATE && !P::SCALED) {
+            // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v), one pass (beta
+            // is known beforehand, see FIN_OMEGA): 5 spinors read and 3 written, where the update
+            // of x and r with its dot products and that of p took 6.5 and 4.  One storage chunk at
+            // a time (the fields do not alias), so few registers and many loads in flight.
             using C = typename P::chunk;
             constexpr int NR = 24 / P::NCH;
             const C *__restrict__ cx_ = reinterpret_cast<const C *>(a.x.p);
             const C *__restrict__ cp_ = reinterpret_cast<const C *>(a.p.p);
             const C *__restrict__ cs_ = reinterpret_cast<const C *>(a.s.p);
             const C *__restrict__ ct_ = reinterpret_cast<const C *>(a.t.p);
-
+            const C *__restrict__ cv_ = reinterpret_cast<const C *>(a.v.p);
             C *__restrict__ ox = reinterpret_cast<C *>(a.x.p);
             C *__restrict__ orr = reinterpret_cast<C *>(a.r.p);
+            C *__restrict__ op = reinterpret_cast<C *>(a.p.p);
             const R ar = (R)S.alpha.x, ai = (R)S.alpha.y, wr = (R)S.omega.x, wi = (R)S.omega.y;
-            R n2 = 0;
+            const R br = (R)S.beta.x, bi = (R)S.beta.y;
 #pragma unroll
             for (int j = 0; j < P::NCH; j++) {
                 const int64_t o = j * a.x.stride + i;
-                R x[NR], p[NR], s[NR], t[NR], rh[NR];
+                R x[NR], p[NR], s[NR], t[NR], v[NR];
                 chunk_to_reals<P>(__ldg(cx_ + o), x);
                 chunk_to_reals<P>(__ldg(cp_ + o), p);
                 chunk_to_reals<P>(__ldg(cs_ + o), s);
                 chunk_to_reals<P>(__ldg(ct_ + o), t);
-                shadow_reals<P>(a.rh, j, i, rh);
+                chunk_to_reals<P>(__ldg(cv_ + o), v);
 #pragma unroll
-                for (int k = 0; k < NR / 2; k++) {
-                    x[2 * k] += (ar * p[2 * k] - ai * p[2 * k + 1]) + (wr * s[2 * k] - wi * s[2 * k + 1]);
-                    x[2 * k + 1] += (ar * p[2 * k + 1] + ai * p[2 * k]) + (wr * s[2 * k + 1] + wi * s[2 * k]);
-                    s[2 * k] -= wr * t[2 * k] - wi * t[2 * k + 1];
-                    s[2 * k + 1] -= wr * t[2 * k + 1] + wi * t[2 * k];
-                }
+                for (int k = 0; k < NR / 2; k++)
+                    xrp_update(x + 2 * k, p + 2 * k, s + 2 * k, t + 2 * k, v + 2 * k, ar, ai, wr, wi, br, bi);
                 ox[o] = reals_to_chunk<P>(x);
                 orr[o] = reals_to_chunk<P>(s);
-#pragma unroll
-                for (int k = 0; k < NR / 2; k++) {
-                    cre += rh[2 * k] * s[2 * k] + rh[2 * k + 1] * s[2 * k + 1];
-                    cim += rh[2 * k] * s[2 * k + 1] - rh[2 * k + 1] * s[2 * k];
-                    n2 += s[2 * k] * s[2 * k] + s[2 * k + 1] * s[2 * k + 1];
-                }
+                op[o] = reals_to_chunk<P>(p);
             }
-            nn = n2;
-        } else if (OP == OP_XR_UPDATE) {  // x += alpha p + omega s ; r = s - omega t ; dots
-            R x[24], p[24], s[24], t[24];
+        } else if (OP == OP_XRP_UPDATE) {  // the same with a whole site-column at a time (its scale)
+            R x[24], p[24], s[24], t[24], v[24];
             load_spinor<P>(a.x, i, x);
             load_spinor<P>(a.p, i, p);
             load_spinor<P>(a.s, i, s);
             load_spinor<P>(a.t, i, t);
+            load_spinor<P>(a.v, i, v);
             const R ar = (R)S.alpha.x, ai = (R)S.alpha.y, wr = (R)S.omega.x, wi = (R)S.omega.y;
+            const R br = (R)S.beta.x, bi = (R)S.beta.y;
 #pragma unroll
-            for (int j = 0; j < 12; j++) {
-                x[2 * j] += (ar * p[2 * j] - ai * p[2 * j + 1]) + (wr * s[2 * j] - wi * s[2 * j + 1]);
-                x[2 * j + 1] += (ar * p[2 * j + 1] + ai * p[2 * j]) + (wr * s[2 * j + 1] + wi * s[2 * j]);
-                s[2 * j] -= wr * t[2 * j] - wi * t[2 * j + 1];
-                s[2 * j + 1] -= wr * t[2 * j + 1] + wi * t[2 * j];
-            }
+            for (int k = 0; k < 12; k++)
+                xrp_update(x + 2 * k, p + 2 * k, s + 2 * k, t + 2 * k, v + 2 * k, ar, ai, wr, wi, br, bi);
             store_spinor<P>(a.x, i, x);
             store_spinor<P>(a.r, i, s);
-            R rh[24];
-            load_spinor<typename ShadowOf<P>::type>(a.rh, i, rh);
-            R n2 = 0;
-#pragma unroll
-            for (int j = 0; j < 12; j++) {
-                cre += rh[2 * j] * s[2 * j] + rh[2 * j + 1] * s[2 * j + 1];
-                cim += rh[2 * j] * s[2 * j + 1] - rh[2 * j + 1] * s[2 * j];
-                n2 += s[2 * j] * s[2 * j] + s[2 * j + 1] * s[2 * j + 1];
-            }
-            nn = n2;
+            store_spinor<P>(a.p, i, p);
         } else if (OP == OP_INIT) {  // rh = r ; p = r ; x = 0
             R r[24], z[24];
             load_spinor<P>(a.r, i, r);
@@ -557,11 +525,10 @@ __global__ void __launch_bounds__(512) k_blas(BlasArgs a) {
             R n2 = 0;
 #pragma unroll
             for (int j = 0; j < 24; j++) n2 += x[j] * x[j];
-            nn = n2;
+            nn[0] = n2;
         }
     }
-    if (OP == OP_XR_UPDATE || OP == OP_NORM)
-        block_partials(it, a.L, tc, cre, cim, nn, a.part, OP == OP_XR_UPDATE, true);
+    if (OP == OP_NORM) warp_partials<1>(it, tc, nn, a.part);
 }
 
 // ---------------------------------------------------- FP64 <-> storage format
@@ -617,16 +584,15 @@ __global__ void __launch_bounds__(512) k_accum(ConvArgs a) {
 
 // ------------------------------------------------------------ scalar updates
 
-enum FinOp { FIN_BNORM = 0, FIN_RESID = 1, FIN_INIT = 2, FIN_ALPHA = 3, FIN_OMEGA = 4, FIN_RHO = 5 };
+enum FinOp { FIN_BNORM = 0, FIN_RESID = 1, FIN_INIT = 2, FIN_ALPHA = 3, FIN_OMEGA = 4 };
 
 struct FinArgs {
-    const Item *items;
     SolveState *st;
     int nsolve;
     Partials A, B;  // B used by FIN_BNORM / FIN_RESID (odd parity)
     LoopCtl *ctl;
-    // FIN_RHO ends an inner-loop iteration: its last block to finish also runs the loop
-    // control (0: not in a loop; 1: sets the graph's WHILE condition; 2: host-polled)
+    // FIN_OMEGA decides whether an inner iteration is the last: its last block to finish also runs
+    // the loop control (0: not in a loop; 1: sets the graph's WHILE condition; 2: host-polled)
     int loop_mode;
     cudaGraphConditionalHandle loop;
 };
@@ -641,41 +607,52 @@ __device__ __forceinline__ double2 cmuld(double2 a, double2 b) {
 
 // One block per solve: fixed-order sum of the solve's tile partials, then the
 // scalar recurrences of BiCGStab (van der Vorst) or of the defect correction.
+//
+// FIN_OMEGA finds omega and, before r is formed, the scalars of the next iteration from the five
+// products of the (t, s) stencil: with r = s - omega t,
+//   (rh, r) = (rh, s) - omega (rh, t),   (r, r) = (s, s) - |(t, s)|^2 / (t, t),
+// so that x, r and p are updated in one pass and an iteration has two reductions.  (r, r) is then
+// good to the rounding of the sums times (s, s), an inner stopping criterion; the true residual
+// of the outer cycle decides convergence.
+constexpr int FIN_THREADS = 256;
 template <int FIN>
-__global__ void __launch_bounds__(256) k_fin(FinArgs a) {
-    int s = blockIdx.x;
-    if (s >= a.nsolve) return;
+__global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
+    constexpr int NV = FIN == FIN_OMEGA ? PART_MAX : FIN == FIN_ALPHA ? 2 : 1;
+    constexpr bool two = (FIN == FIN_BNORM || FIN == FIN_RESID);
+    __shared__ double sh[FIN_THREADS / 32][NV];
+    const int s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SolveState &S = a.st[s];
-    const Item &it = a.items[S.item];
-    int64_t base = it.pbase + (int64_t)S.col * it.ntiles;
-    const bool want_c = (FIN == FIN_ALPHA || FIN == FIN_OMEGA || FIN == FIN_RHO);
-    const bool two = (FIN == FIN_BNORM || FIN == FIN_RESID);
-    double cr = 0, ci = 0, nn = 0;
-    for (int t = threadIdx.x; t < it.ntiles; t += blockDim.x) {
-        if (want_c) {
-            double2 c = a.A.c[base + t];
-            cr += c.x;
-            ci += c.y;
+    const int nt = S.ntiles;
+    const int64_t base = S.pbase;
+    double v[NV] = {};
+    const bool wanted = !(FIN == FIN_ALPHA || FIN == FIN_OMEGA) || S.active == 1;
+    if (wanted)
+        for (int t = threadIdx.x; t < nt; t += FIN_THREADS) {
+            if (NV == 1) {
+                v[0] += a.A.d[base + t];
+                if (two) v[0] += a.B.d[base + t];
+            } else {
+                const double2 *q = reinterpret_cast<const double2 *>(a.A.d + (base + t) * NV);
+#pragma unroll
+                for (int k = 0; k < NV / 2; k++) {
+                    const double2 c = q[k];
+                    v[2 * k] += c.x;
+                    v[2 * k + 1] += c.y;
+                }
+            }
         }
-        if (FIN != FIN_ALPHA) nn += a.A.n[base + t];
-        if (two) nn += a.B.n[base + t];
-    }
-    __shared__ double sr[256], si[256], sn[256];
-    sr[threadIdx.x] = cr;
-    si[threadIdx.x] = ci;
-    sn[threadIdx.x] = nn;
+#pragma unroll
+    for (int k = 0; k < NV; k++) v[k] = warp_sum(v[k]);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NV; k++) sh[warp][k] = v[k];
     __syncthreads();
-    for (int o = blockDim.x >> 1; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            sr[threadIdx.x] += sr[threadIdx.x + o];
-            si[threadIdx.x] += si[threadIdx.x + o];
-            sn[threadIdx.x] += sn[threadIdx.x + o];
-        }
-        __syncthreads();
-    }
     if (threadIdx.x != 0) return;
-    double2 c = make_double2(sr[0], si[0]);
-    double n = sn[0];
+    for (int k = 0; k < NV; k++) {
+        v[k] = sh[0][k];
+        for (int w = 1; w < FIN_THREADS / 32; w++) v[k] += sh[w][k];
+    }
+    const double n = v[0];
     const double2 zero = make_double2(0, 0), one = make_double2(1, 0);
     if (FIN == FIN_BNORM) {
         S.bnorm2 = n;
@@ -694,7 +671,7 @@ __global__ void __launch_bounds__(256) k_fin(FinArgs a) {
             S.scale = 0;
         } else {
             S.sigma = sqrt(n);
-            S.scale = 2.0 * it.kappa / S.sigma;
+            S.scale = 2.0 * S.kappa / S.sigma;
             double d = 0.5 * S.tol * sqrt(S.bnorm2 / n);
             d = fmax(d, S.floor_delta);
             S.delta = fmin(d, 0.1);
@@ -712,7 +689,8 @@ __global__ void __launch_bounds__(256) k_fin(FinArgs a) {
         S.beta = zero;
         if (act) atomicAdd(&a.ctl->n_active, 1);
     } else if (FIN == FIN_ALPHA) {
-        if (S.active) {
+        if (S.active == 1) {
+            const double2 c = make_double2(v[0], v[NV - 1]);
             if (!(c.x * c.x + c.y * c.y > 0) || !isfinite(c.x) || !isfinite(c.y)) {
                 S.active = 0;
                 S.status = 2;
@@ -722,33 +700,37 @@ __global__ void __launch_bounds__(256) k_fin(FinArgs a) {
             } else {
                 S.alpha = cdiv(S.rho, c);
             }
+        } else {
+            S.active = 0;  // its last update has been made
         }
     } else if (FIN == FIN_OMEGA) {
-        if (S.active) S.omega = (n > 0) ? cdiv(c, make_double2(n, 0)) : zero;
-    } else if (FIN == FIN_RHO) {
-        if (S.active) {
+        if (S.active == 1) {
+            const double2 ts = make_double2(v[0], v[1 % NV]), hs = make_double2(v[2 % NV], v[3 % NV]),
+                          ht = make_double2(v[4 % NV], v[5 % NV]);
+            const double tt = v[6 % NV], ss = v[7 % NV];
+            S.omega = (tt > 0) ? cdiv(ts, make_double2(tt, 0)) : zero;
+            const double2 wh = cmuld(S.omega, ht);
+            const double2 c = make_double2(hs.x - wh.x, hs.y - wh.y);
+            const double rr = (tt > 0) ? ss - (ts.x * ts.x + ts.y * ts.y) / tt : ss;
+            const bool w0 = (S.omega.x == 0.0 && S.omega.y == 0.0);
             S.iters++;
             S.total_iters++;
-            S.rr = n;
-            bool w0 = (S.omega.x == 0.0 && S.omega.y == 0.0);
-            if (n <= S.target2) {
-                S.active = 0;
+            S.rr = fmax(rr, 0.0);
+            if (rr <= S.target2) {
+                S.active = 2;
                 S.status = 1;
-            } else if (!(c.x * c.x + c.y * c.y > 0) || w0 || !isfinite(n)) {
-                S.active = 0;
+            } else if (!(c.x * c.x + c.y * c.y > 0) || w0 || !isfinite(rr)) {
+                S.active = 2;
                 S.status = 2;
             } else if (S.iters >= S.maxit) {
-                S.active = 0;
+                S.active = 2;
                 S.status = 3;
+            }
+            if (S.active == 2) {
+                S.beta = zero;
             } else {
                 S.beta = cmuld(cdiv(c, S.rho), cdiv(S.alpha, S.omega));
                 S.rho = c;
-            }
-            if (!S.active) {
-                S.alpha = zero;
-                S.omega = zero;
-                S.beta = zero;
-            } else {
                 atomicAdd(&a.ctl->n_active, 1);
             }
         }
@@ -903,7 +885,7 @@ static __global__ void __launch_bounds__(384) k_to_fx(FxArgs a) {
     if (!tc.valid) return;
     if (a.skip) {
         const SolveState &S = a.st[it.solve0 + tc.col];
-        if ((a.skip == 1) ? !S.active : S.outer_done) return;
+        if (skipped(S, a.skip)) return;
     }
     double v[24];
     load_spinor<PF64>(a.in, tc.cb + tc.h, v);
@@ -931,7 +913,7 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
         int live = 0;
         if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
             const SolveState &S = a.st[it.solve0 + col];
-            live = (a.skip == 1) ? S.active : !S.outer_done;
+            live = !skipped(S, a.skip);
         }
         if (!__syncthreads_or(live)) return;
     }
@@ -967,9 +949,9 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
     TileCoord tc = tile_coord(it, a.L);
     if (a.skip && tc.valid) {
         const SolveState &S = a.st[it.solve0 + tc.col];
-        if ((a.skip == 1) ? !S.active : S.outer_done) tc.valid = false;
+        if (skipped(S, a.skip)) tc.valid = false;
     }
-    double cre = 0, cim = 0, nn = 0;
+    double sums[PART_MAX] = {};
     if (tc.valid) {
         const int sl = tc.h - tc.tile * TS;
         int e[8], top = FX_ZERO;
@@ -1009,7 +991,7 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
 #pragma unroll
                 for (int j = 0; j < 12; j++)
                     acc[j / 3][j % 3] = mk(fx_value(sum[2 * j], top - FX_LINK), fx_value(sum[2 * j + 1], top - FX_LINK));
-                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, cre, cim, nn);
+                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, sums);
             }
         } else {
             double o[24];
@@ -1019,12 +1001,11 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
             } else {
                 cx<double> acc[4][3];
                 for (int j = 0; j < 12; j++) acc[j / 3][j % 3] = mk(o[2 * j], o[2 * j + 1]);
-                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, cre, cim, nn);
+                hop_store_epilogue<PF64, EPI, DOT, CLOV>(a, it, tc, acc, sums);
             }
         }
     }
-    if (DOT != DOT_NONE) block_partials(it, a.L, tc, cre, cim, nn, a.part, DOT == DOT_RHAT || DOT == DOT_TS,
-                                        DOT == DOT_TS || DOT == DOT_NORM);
+    if (DOT != DOT_NONE) warp_partials<DOT != DOT_NONE ? dot_sums(DOT) : 1>(it, tc, sums, a.part);
 }
 
 // User layout <-> block fixed point (the stencil powers); unpacking multiplies by s.

@@ -138,15 +138,14 @@ struct Engine {
     template <int FIN>
     void fin() {
         FinArgs a;
-        a.items = d_items;
         a.st = d_st;
         a.nsolve = plan.nsolve;
         a.A = A;
         a.B = B;
         a.ctl = d_ctl;
-        a.loop_mode = FIN == FIN_RHO ? loop_mode : 0;
+        a.loop_mode = FIN == FIN_OMEGA ? loop_mode : 0;
         a.loop = loop_handle;
-        k_fin<FIN><<<plan.nsolve, 256, 0, ctx->stream>>>(a);
+        k_fin<FIN><<<plan.nsolve, FIN_THREADS, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -188,11 +187,9 @@ struct Engine {
         fin<FIN_ALPHA>();                                                               // alpha = rho / (rh, v)
         blas<P, OP_S_UPDATE>(A);                                                        // s = r - alpha v
         hop<P, EPI_PLAIN, DOT_NONE, CL>(hop_args(1, s, tmp, none, none, none, A, 1));   // tmp = T^-1 H_oe s
-        hop<P, EPI_MHAT, DOT_TS, CL>(hop_args(0, tmp, t, s, none, none, A, 1));        // t = s - k^2 T^-1 H_eo tmp
-        fin<FIN_OMEGA>();                                                               // omega = (t,s)/(t,t)
-        blas<P, OP_XR_UPDATE>(A);                                                       // x, r; (rh,r), (r,r)
-        fin<FIN_RHO>();                                                                 // beta, convergence
-        blas<P, OP_P_UPDATE>(A);                                                        // p = r + beta (p - omega v)
+        hop<P, EPI_MHAT, DOT_TS, CL>(hop_args(0, tmp, t, s, none, rh, A, 1));          // t = s - k^2 T^-1 H_eo tmp
+        fin<FIN_OMEGA>();                                      // omega, beta, convergence, loop control
+        blas<P, OP_XRP_UPDATE>(A);                                                      // x, r, p
     }
     void iteration_body() {
         if (clov)
@@ -224,7 +221,7 @@ struct Engine {
                                                         cudaStreamCaptureModeThreadLocal));
             loop_mode = 1;
             loop_handle = h;
-            iteration_body();  // its last kernel sets the loop condition
+            iteration_body();  // its FIN_OMEGA sets the loop condition
             loop_mode = 0;
             cudaGraph_t captured;
             cudaError_t e = cudaStreamEndCapture(st, &captured);
@@ -243,9 +240,9 @@ struct Engine {
     }
 
     int run_inner() {
-        // launches per iteration: 4 stencils, 3 vector updates, 3 scalar-recurrence
-        // kernels (the last of which also runs the loop control)
-        const long per_iter = P::IS64 ? 14 : 10;  // FP64 stencils: conversion and hop
+        // launches per iteration: 4 stencils (FP64: conversion and hop), 2 vector updates, 2
+        // scalar-recurrence kernels (the second of which also runs the loop control)
+        const long per_iter = P::IS64 ? 12 : 8;
         if (ctx->prm.use_conditional) {
             DDP_CUDA(ctx, cudaGraphLaunch(loop_exec, ctx->stream));
         } else {
@@ -268,7 +265,7 @@ struct Engine {
 
     static size_t bytes_needed(int64_t cap, int64_t npart, int nitems, int nsolve) {
         return 6 * field_bytes<PF64>(cap) + 9 * field_bytes<P>(cap) +
-               2 * ((size_t)npart * (sizeof(double2) + sizeof(double)) + 1024) + (size_t)nitems * sizeof(Item) +
+               (size_t)npart * (PART_MAX + 1) * sizeof(double) + 2048 + (size_t)nitems * sizeof(Item) +
                (size_t)nsolve * sizeof(SolveState) + sizeof(LoopCtl) + 8192;
     }
 
@@ -302,10 +299,8 @@ struct Engine {
         static_assert((P::NCH * 5 + ShadowOf<P>::type::NCH) * 16 >= PFX::NCH * 16 + 4, "fixed-point field over the inner fields");
         fx_outer = fx_over(r);
         fx_inner = fx_over(re64);
-        A.c = (double2 *)a.take(npart * sizeof(double2));
-        A.n = (double *)a.take(npart * sizeof(double));
-        B.c = (double2 *)a.take(npart * sizeof(double2));
-        B.n = (double *)a.take(npart * sizeof(double));
+        A.d = (double *)a.take(npart * PART_MAX * sizeof(double));
+        B.d = (double *)a.take(npart * sizeof(double));  // true-residual norms only
         d_items = (Item *)a.take(nitems * sizeof(Item));
         d_st = (SolveState *)a.take(nsolve * sizeof(SolveState));
         d_ctl = (LoopCtl *)a.take(sizeof(LoopCtl));
@@ -320,6 +315,12 @@ struct Engine {
         L.CG = plan.CG;
         threads = plan.TS * plan.CG;
         h_st = states;
+        for (SolveState &S : h_st) {
+            const Item &it = plan.items[S.item];
+            S.ntiles = it.ntiles;
+            S.pbase = it.pbase + (int64_t)S.col * it.ntiles;
+            S.kappa = it.kappa;
+        }
         DDP_CUDA(ctx, cudaMemcpyAsync(d_items, plan.items.data(), plan.items.size() * sizeof(Item),
                                       cudaMemcpyHostToDevice, st));
         DDP_CUDA(ctx, cudaMemcpyAsync(d_st, h_st.data(), plan.nsolve * sizeof(SolveState), cudaMemcpyHostToDevice,
@@ -536,8 +537,7 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
     h.L = L;
     h.v2 = none;
     h.rh = none;
-    h.part.c = nullptr;
-    h.part.n = nullptr;
+    h.part.d = nullptr;
     h.p = 0;
     h.in = io;
     h.out = oe;
@@ -565,10 +565,11 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
 // the context's stream around `iters` back-to-back launches after 3 warm-up
 // launches.  kernel: DDP_HOP_PLAIN  tmp = H_oe p;  DDP_HOP_SCHUR_RHAT  v = p -
 // kappa^2 H_eo tmp with the (rh, v) partials;  DDP_HOP_SCHUR_TS  t = s -
-// kappa^2 H_eo tmp with the (t, s), (t, t) partials.  Algorithmic bytes per
+// kappa^2 H_eo tmp with the partials of its five products.  Algorithmic bytes per
 // launch: the spinors the variant reads or writes once per output
 // site-column (2, 4 and 3 of them; the shadow residual of the (rh, v) variant
-// in its own storage, BF16 for FP32 storage) plus the 8 links touching each
+// in its own storage, BF16 for FP32 storage; that of the (t, s) variant is not
+// counted) plus the 8 links touching each
 // output site once for all columns.
 template <class P>
 int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters, float *ms, double *bytes) {
@@ -576,7 +577,7 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     Plan plan;
     make_plan(jobs, prec, ctx->prm, plan);
     const int64_t NF = plan.nfield;
-    size_t need = 4 * field_bytes<P>(NF) + (P::IS64 ? field_bytes<PFX>(NF) : 0) + 2 * ((size_t)plan.npart * 24 + 1024) +
+    size_t need = 4 * field_bytes<P>(NF) + (P::IS64 ? field_bytes<PFX>(NF) : 0) + (size_t)plan.npart * PART_MAX * 8 + 1024 +
                   sizeof(Item) + 1024;
     DDP_CUDA(ctx, ctx->scratch.reserve(need));
     Arena &a = ctx->scratch;
@@ -586,8 +587,7 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     FieldView fx = {nullptr, nullptr, 0};
     if (P::IS64) fx = carve_field<PFX>(a, NF);
     Partials A;
-    A.c = (double2 *)a.take(plan.npart * sizeof(double2));
-    A.n = (double *)a.take(plan.npart * sizeof(double));
+    A.d = (double *)a.take(plan.npart * PART_MAX * sizeof(double));
     Item *d_items = (Item *)a.take(sizeof(Item));
     cudaStream_t st = ctx->stream;
     DDP_CUDA(ctx, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(Item), cudaMemcpyHostToDevice, st));
@@ -615,7 +615,7 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     h.out = out;
     h.v1 = (kernel == DDP_HOP_PLAIN) ? none : v1;
     h.v2 = none;
-    h.rh = (kernel == DDP_HOP_SCHUR_RHAT) ? rhv : none;
+    h.rh = (kernel == DDP_HOP_PLAIN) ? none : rhv;
     h.part = A;
     DDP_CUDA(ctx, (set_hop_carveout<P, false>(carveout_for(ctx->prm, prec))));
     auto launch = [&]() {

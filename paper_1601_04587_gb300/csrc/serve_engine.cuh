@@ -53,7 +53,7 @@ struct Server : ServerBase {
         max_active = maxact;
         nsolve_cap = MAX_NCOL * maxact;
         // bytes per site-column of capacity (fields) plus the per-tile partials
-        double per = (double)Engine<P>::bytes_needed(1 << 20, 0, 0, 0) / (1 << 20) + 2.0 * 24.0 / 32.0;
+        double per = (double)Engine<P>::bytes_needed(1 << 20, 0, 0, 0) / (1 << 20) + (PART_MAX + 1) * 8.0 / 32.0;
         cap = (int64_t)((double)budget / per);
         cap = (cap / 32) * 32;
         if (cap < 1024) return DDP_ERR_OOM;

@@ -52,8 +52,7 @@ int hop_power_fx(ddp_ctx *ctx, const Job &job, int p, const double *psi, double 
     h.v1 = none;
     h.v2 = none;
     h.rh = none;
-    h.part.c = nullptr;
-    h.part.n = nullptr;
+    h.part.d = nullptr;
     int cur = 0;
     for (int k = 0; k < p; k++) {
         const int nxt = cur ^ 1;
