@@ -84,6 +84,10 @@ void make_plan(const std::vector<Job> &jobs, int prec, const EngineParams &prm, 
         it.links = j.g->links(prec);
         it.links64 = j.g->u64;
         it.gV = j.g->V;
+        it.by_hx = fast_div(it.e[3] / 2);
+        it.by_e2 = fast_div(it.e[2]);
+        it.by_e1 = fast_div(it.e[1]);
+        it.by_nt = fast_div(it.ntiles);
         if (j.clov) {
             it.clov = (prec == DDP_PREC_FP64) ? (const void *)j.clov->t64 : (const void *)j.clov->t32;
             it.clovinv = (prec == DDP_PREC_FP64) ? (const void *)j.clov->ti64 : (const void *)j.clov->ti32;
@@ -380,7 +384,7 @@ __device__ __forceinline__ void boundary_hop(const BoundaryArgs &a, const int x[
     }
     for (int i = 0; i < 3; i++)
         for (int k = 0; k < 3; k++) u[i][k] = f * u[i][k];
-    hop_step<D, true>(v, u, acc, 1.0);
+    hop_step<D>(v, u, acc, 1.0);
 }
 
 __global__ void k_boundary_source(BoundaryArgs a) {

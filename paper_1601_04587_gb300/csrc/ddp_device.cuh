@@ -188,30 +188,27 @@ __device__ __forceinline__ void load_spinor<PBF16>(const FieldView &f, int64_t i
     }
 }
 
-// Spinor as stored: FP16 values without their site-column scale, which is
-// returned in *s (1 for the other formats).
+// Spinor as stored, as (re, im) pairs: FP16 values without their site-column
+// scale, which is returned in *s (1 for the other formats).
+// off: the byte offsets of the storage chunks, kernel parameters, so that no strides are held in
+// registers.
 template <class P>
-__device__ __forceinline__ void load_spinor_raw(const FieldView &f, int64_t i, typename P::real v[24],
-                                                typename P::real *s) {
-    load_spinor<P>(f, i, v);
-    *s = typename P::real(1);
-}
-template <>
-__device__ __forceinline__ void load_spinor_raw<PF16>(const FieldView &f, int64_t i, float v[24], float *s) {
-    const uint4 *b = reinterpret_cast<const uint4 *>(f.p);
-    *s = __ldg(f.scale + i);
+__device__ __forceinline__ void load_pairs(const FieldView &f, const int64_t *off, int64_t i, float2 v[12], float *s) {
+    using C = typename P::chunk;
+    const char *b = reinterpret_cast<const char *>(f.p) + i * (int64_t)sizeof(C);
+    *s = P::SCALED ? __ldg(f.scale + i) : 1.f;
 #pragma unroll
-    for (int j = 0; j < 3; j++) {
-        uint4 c = __ldg(b + j * f.stride + i);
-        float2 a0 = h2f(c.x), a1 = h2f(c.y), a2 = h2f(c.z), a3 = h2f(c.w);
-        v[8 * j + 0] = a0.x;
-        v[8 * j + 1] = a0.y;
-        v[8 * j + 2] = a1.x;
-        v[8 * j + 3] = a1.y;
-        v[8 * j + 4] = a2.x;
-        v[8 * j + 5] = a2.y;
-        v[8 * j + 6] = a3.x;
-        v[8 * j + 7] = a3.y;
+    for (int j = 0; j < P::NCH; j++) {
+        const C c = __ldg(reinterpret_cast<const C *>(b + off[j]));
+        if constexpr (P::NCH == 6) {
+            v[2 * j] = make_float2(c.x, c.y);
+            v[2 * j + 1] = make_float2(c.z, c.w);
+        } else {
+            v[4 * j] = P::SCALED ? h2f(c.x) : b2f(c.x);
+            v[4 * j + 1] = P::SCALED ? h2f(c.y) : b2f(c.y);
+            v[4 * j + 2] = P::SCALED ? h2f(c.z) : b2f(c.z);
+            v[4 * j + 3] = P::SCALED ? h2f(c.w) : b2f(c.w);
+        }
     }
 }
 
@@ -332,7 +329,25 @@ __device__ __forceinline__ void load_link<PBF16>(const void *L, int64_t V, int m
 // [blk0, blk0 + ntiles*ncg).  Reduction partials of (column c, tile t) live at
 // pbase + c*ntiles + t.
 
-struct Item {
+// n / d for 0 <= n < 2^31 by a multiplication: q = n m >> s with m = floor(2^s / d) + 1,
+// s = 31 + ceil(log2 d).
+struct FastDiv {
+    unsigned m;
+    int s;
+};
+inline FastDiv fast_div(int d) {
+    int l = 0;
+    while ((1ll << l) < d) l++;
+    FastDiv f;
+    f.s = 31 + l;
+    f.m = (unsigned)((1ull << f.s) / (unsigned)d + 1);
+    return f;
+}
+__device__ __forceinline__ int fdiv(int n, const FastDiv &f) {
+    return (int)(((unsigned long long)(unsigned)n * f.m) >> f.s);
+}
+
+struct __align__(16) Item {
     int o[4];        // origin (global coordinates, reduced mod L)
     int e[4];        // extent
     int L[4];        // lattice
@@ -351,6 +366,7 @@ struct Item {
     const void *links;    // links of the launch's storage precision
     const void *links64;  // FP64 links
     int64_t gV;           // lattice volume (link field row length)
+    FastDiv by_hx, by_e2, by_e1, by_nt;  // division by e[3] / 2, e[2], e[1] and ntiles
     // clover term (clover.cuh), NULL without it: T and T^-1 in the launch's arithmetic
     // (FP64 packed for the FP64 path, FP32 packed otherwise) and T in FP64
     const void *clov;
@@ -358,10 +374,13 @@ struct Item {
     const void *clov64;
 };
 
+constexpr int INLINE_ITEMS = 4;  // a series of nested domains fits
+
 struct Launch {
     const Item *items;
     int nitems;
     int TS, CG;          // sites per tile (multiple of 32), columns per block
+    Item inl[INLINE_ITEMS];  // the items themselves where they are so few 
 };
 
 // Locate the item owning block b (items sorted by blk0).
@@ -380,13 +399,12 @@ __device__ __forceinline__ int find_item(const Item *items, int nitems, int b) {
 // Domain-local coordinates of the even-odd index h of parity p (requires e3 even):
 // the local lexicographic index l = ((k0 e1 + k1) e2 + k2) e3 + k3 satisfies h = l >> 1.
 __device__ __forceinline__ void decode_site(const Item &it, int h, int p, int k[4]) {
-    int hx = it.e[3] >> 1;
-    int row = h / hx;
-    int j = h - row * hx;
-    k[2] = row % it.e[2];
-    row /= it.e[2];
-    k[1] = row % it.e[1];
-    k[0] = row / it.e[1];
+    const int row = fdiv(h, it.by_hx);
+    const int j = h - row * (it.e[3] >> 1);
+    const int r1 = fdiv(row, it.by_e2);
+    k[2] = row - r1 * it.e[2];
+    k[0] = fdiv(r1, it.by_e1);
+    k[1] = r1 - k[0] * it.e[1];
     k[3] = 2 * j + ((p + it.par_o + k[0] + k[1] + k[2]) & 1);
 }
 
@@ -413,41 +431,26 @@ __device__ __forceinline__ int64_t link_row(const Item &it, const int x[4], int 
 // and (1 + g)psi = [h; A^+ h] with h = psi_up + A psi_dn, so only the two
 // rows of h are multiplied by the link.
 
-// w = u h.  FMA: one multiply-add chain per real component (6 instructions
-// instead of 8); it saves issue slots where the kernel is issue-bound (16-bit
-// storage) but holds more registers live, so the FP32-storage stencil keeps
-// the plain form.
-template <bool FMA, typename R>
+// w = u h, one multiply-add chain per real component.
+template <typename R>
 __device__ __forceinline__ void su3_mul_half(const cx<R> u[3][3], const cx<R> h[2][3], cx<R> w[2][3]) {
 #pragma unroll
     for (int s = 0; s < 2; s++)
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            if (FMA) {
-                R re = u[a][0].re * h[s][0].re;
-                R im = u[a][0].re * h[s][0].im;
-                re = fma(-u[a][0].im, h[s][0].im, re);
-                im = fma(u[a][0].im, h[s][0].re, im);
+            R re = u[a][0].re * h[s][0].re;
+            R im = u[a][0].re * h[s][0].im;
+            re = fma(-u[a][0].im, h[s][0].im, re);
+            im = fma(u[a][0].im, h[s][0].re, im);
 #pragma unroll
-                for (int b = 1; b < 3; b++) {
-                    re = fma(u[a][b].re, h[s][b].re, re);
-                    im = fma(u[a][b].re, h[s][b].im, im);
-                    re = fma(-u[a][b].im, h[s][b].im, re);
-                    im = fma(u[a][b].im, h[s][b].re, im);
-                }
-                w[s][a] = mk(re, im);
-            } else {
-                w[s][a] = u[a][0] * h[s][0] + u[a][1] * h[s][1] + u[a][2] * h[s][2];
+            for (int b = 1; b < 3; b++) {
+                re = fma(u[a][b].re, h[s][b].re, re);
+                im = fma(u[a][b].re, h[s][b].im, im);
+                re = fma(-u[a][b].im, h[s][b].im, re);
+                im = fma(u[a][b].im, h[s][b].re, im);
             }
+            w[s][a] = mk(re, im);
         }
-}
-template <typename R>
-__device__ __forceinline__ void su3_adj_mul_half(const cx<R> u[3][3], const cx<R> h[2][3], cx<R> w[2][3]) {
-#pragma unroll
-    for (int s = 0; s < 2; s++)
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-            w[s][a] = cmul(u[0][a], h[s][0]) + cmul(u[1][a], h[s][1]) + cmul(u[2][a], h[s][2]);
 }
 
 // Spin projection of direction MU, FWD = forward hop (1 - g_mu), else (1 + g_mu).
@@ -580,15 +583,110 @@ __device__ __forceinline__ int stage_hop(const Item &it, int h, int p, int d, cx
 }
 
 // acc += f (1 -/+ g_mu) u psi for hop D (compile-time), link u already
-// oriented; f is the FP16 site-column scale of psi, else 1.
-template <int D, bool FMA, typename R>
+// oriented, in plain arithmetic (the boundary source and the non-finite cases).
+template <int D, typename R>
 __device__ __forceinline__ void hop_step(const R v[24], const cx<R> u[3][3], cx<R> acc[4][3], R f) {
     constexpr int MU = D >> 1;
     constexpr bool FWD = !(D & 1);
     cx<R> h[2][3], w[2][3];
     project<MU, FWD>(v, h);
-    su3_mul_half<FMA>(u, h, w);
+    su3_mul_half(u, h, w);
     accumulate<MU, FWD>(acc, w, f);
+}
+
+// ------------------------------------------------ packed FP32 hopping step
+//
+// The low-precision stencils compute on (re, im) pairs with GB300's two-lane FP32
+// instructions (one issue slot for two multiply-adds).  u h = A + i B with the pairs
+// A = sum re(u) * h and B = sum im(u) * h, so that only the link's parts are duplicated, never a
+// spinor operand swapped: 72 FP instructions and 24 moves per hop, where the scalar form issues
+// 132.  (Links staged as (re, re, im, im) need no moves but twice the shared-memory reads, which
+// cost more: 0.36 against 0.28 ms for the plain FP32 stencil on 48x24^3, 12 columns.  Scalar
+// arithmetic: 0.305 ms; with the division-free set-up and the items as parameters, 0.264.)
+
+__device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 f2_add_i(float2 a, float2 b) { return f2(a.x - b.y, a.y + b.x); }  // a + i b
+__device__ __forceinline__ float2 f2_sub_i(float2 a, float2 b) { return f2(a.x + b.y, a.y - b.x); }
+
+template <int MU, bool FWD>
+__device__ __forceinline__ void f2_project(const float2 v[12], float2 h[2][3]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float2 p0 = v[a], p1 = v[3 + a], p2 = v[6 + a], p3 = v[9 + a];
+        if (MU == 0) {
+            h[0][a] = FWD ? f2_sub(p0, p2) : f2_add(p0, p2);
+            h[1][a] = FWD ? f2_sub(p1, p3) : f2_add(p1, p3);
+        } else if (MU == 1) {
+            h[0][a] = FWD ? f2_add_i(p0, p3) : f2_sub_i(p0, p3);
+            h[1][a] = FWD ? f2_add_i(p1, p2) : f2_sub_i(p1, p2);
+        } else if (MU == 2) {
+            h[0][a] = FWD ? f2_add(p0, p3) : f2_sub(p0, p3);
+            h[1][a] = FWD ? f2_sub(p1, p2) : f2_add(p1, p2);
+        } else {
+            h[0][a] = FWD ? f2_add_i(p0, p2) : f2_sub_i(p0, p2);
+            h[1][a] = FWD ? f2_sub_i(p1, p3) : f2_add_i(p1, p3);
+        }
+    }
+}
+
+// acc += f w, acc -= f w, acc += i f w, acc -= i f w (SCALED: f != 1)
+template <bool SCALED>
+__device__ __forceinline__ void f2_acc(float2 &acc, float2 w, float f) {
+    acc = SCALED ? __ffma2_rn(f2(f, f), w, acc) : __fadd2_rn(acc, w);
+}
+template <bool SCALED>
+__device__ __forceinline__ void f2_acc_neg(float2 &acc, float2 w, float f) {
+    acc = __ffma2_rn(SCALED ? f2(-f, -f) : f2(-1.f, -1.f), w, acc);
+}
+template <bool SCALED>
+__device__ __forceinline__ void f2_acc_i(float2 &acc, float2 w, float f) {
+    acc.x = SCALED ? fmaf(-f, w.y, acc.x) : acc.x - w.y;
+    acc.y = SCALED ? fmaf(f, w.x, acc.y) : acc.y + w.x;
+}
+template <bool SCALED>
+__device__ __forceinline__ void f2_acc_mi(float2 &acc, float2 w, float f) {
+    acc.x = SCALED ? fmaf(f, w.y, acc.x) : acc.x + w.y;
+    acc.y = SCALED ? fmaf(-f, w.x, acc.y) : acc.y - w.x;
+}
+
+// acc += f (1 -/+ g_mu) u psi for hop D; u: 9 staged entries.
+template <int D, bool SCALED>
+__device__ __forceinline__ void f2_hop_step(const float2 v[12], const float2 *u, float2 acc[4][3], float f) {
+    constexpr int MU = D >> 1;
+    constexpr bool FWD = !(D & 1);
+    float2 h[2][3];
+    f2_project<MU, FWD>(v, h);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        float2 A[2], B[2];
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            const float2 c = u[3 * a + b];
+#pragma unroll
+            for (int s = 0; s < 2; s++) {
+                A[s] = b ? __ffma2_rn(f2(c.x, c.x), h[s][b], A[s]) : __fmul2_rn(f2(c.x, c.x), h[s][b]);
+                B[s] = b ? __ffma2_rn(f2(c.y, c.y), h[s][b], B[s]) : __fmul2_rn(f2(c.y, c.y), h[s][b]);
+            }
+        }
+        const float2 w0 = f2_add_i(A[0], B[0]), w1 = f2_add_i(A[1], B[1]);
+        f2_acc<SCALED>(acc[0][a], w0, f);
+        f2_acc<SCALED>(acc[1][a], w1, f);
+        if (MU == 0) {
+            if (FWD) { f2_acc_neg<SCALED>(acc[2][a], w0, f); f2_acc_neg<SCALED>(acc[3][a], w1, f); }
+            else { f2_acc<SCALED>(acc[2][a], w0, f); f2_acc<SCALED>(acc[3][a], w1, f); }
+        } else if (MU == 1) {
+            if (FWD) { f2_acc_mi<SCALED>(acc[2][a], w1, f); f2_acc_mi<SCALED>(acc[3][a], w0, f); }
+            else { f2_acc_i<SCALED>(acc[2][a], w1, f); f2_acc_i<SCALED>(acc[3][a], w0, f); }
+        } else if (MU == 2) {
+            if (FWD) { f2_acc_neg<SCALED>(acc[2][a], w1, f); f2_acc<SCALED>(acc[3][a], w0, f); }
+            else { f2_acc<SCALED>(acc[2][a], w1, f); f2_acc_neg<SCALED>(acc[3][a], w0, f); }
+        } else {
+            if (FWD) { f2_acc_mi<SCALED>(acc[2][a], w0, f); f2_acc_i<SCALED>(acc[3][a], w1, f); }
+            else { f2_acc_i<SCALED>(acc[2][a], w0, f); f2_acc_mi<SCALED>(acc[3][a], w1, f); }
+        }
+    }
 }
 
 // --------------------------------------------------------- reductions

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <map>
 #include <memory>
@@ -208,6 +209,19 @@ struct Plan {
     int nblocks = 0;
     int nsolve = 0;
 };
+
+// The launch description of a plan whose items are at d_items on the device.
+inline Launch make_launch(const Plan &plan, const Item *d_items) {
+    Launch L;
+    memset(&L, 0, sizeof(L));
+    L.items = d_items;
+    L.nitems = (int)plan.items.size();
+    L.TS = plan.TS;
+    L.CG = plan.CG;
+    if (L.nitems <= INLINE_ITEMS)
+        for (int i = 0; i < L.nitems; i++) L.inl[i] = plan.items[i];
+    return L;
+}
 
 void make_plan(const std::vector<Job> &jobs, int prec, const EngineParams &prm, Plan &plan);
 

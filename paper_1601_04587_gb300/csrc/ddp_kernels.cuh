@@ -77,6 +77,7 @@ struct HopArgs {
     Partials part;
     const SolveState *st;  // skip 1: leave columns whose inner solve is not active untouched;
     int skip;              // skip 2: leave columns whose outer solve has converged untouched
+    int64_t off[6];        // byte offsets of the storage chunks of in (set by launch_hop)
 };
 
 // Whether a kernel with the given skip mode leaves the column alone.
@@ -112,8 +113,8 @@ struct TileCoord {
 __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L) {
     TileCoord t;
     int lb = blockIdx.x - it.blk0;
-    t.tile = lb % it.ntiles;
-    int cg = lb / it.ntiles;
+    const int cg = fdiv(lb, it.by_nt);
+    t.tile = lb - cg * it.ntiles;
     int cl = threadIdx.x / HOP_TS;
     int sl = threadIdx.x - cl * HOP_TS;
     t.col = cg * L.CG + cl;
@@ -148,9 +149,50 @@ __device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &t
         part.d[(it.pbase + (int64_t)tc.col * it.ntiles + tc.tile) * NV + lane / (32 / NV)] = (double)v[0];
 }
 
+// The block's item, copied by words by one warp: from the kernel parameters where the launch
+// carries its items there (Launch::inl), so that a block does not begin with a wait for memory.
+// Every block starts with this, so it counts: plain FP32 stencil on 48x24^3, 12 columns, 0.287 ms
+// with a copy by one thread, 0.267 from global memory, 0.264 from the
+// parameters.
 __device__ __forceinline__ void load_item(const Launch &L, Item &dst) {
-    if (threadIdx.x == 0) dst = L.items[find_item(L.items, L.nitems, blockIdx.x)];
+    static_assert(sizeof(Item) % 16 == 0, "copied by 16 bytes");
+    constexpr int N = sizeof(Item) / 16;
+    if (threadIdx.x < 32) {
+        if (L.nitems <= INLINE_ITEMS) {
+            int i = 0;
+#pragma unroll
+            for (int k = 1; k < INLINE_ITEMS; k++) i += (k < L.nitems && L.inl[k].blk0 <= (int)blockIdx.x) ? 1 : 0;
+            if (threadIdx.x < N)
+                reinterpret_cast<int4 *>(&dst)[threadIdx.x] = reinterpret_cast<const int4 *>(L.inl + i)[threadIdx.x];
+        } else {
+            const int4 *src = reinterpret_cast<const int4 *>(L.items + find_item(L.items, L.nitems, blockIdx.x));
+            if (threadIdx.x < N) reinterpret_cast<int4 *>(&dst)[threadIdx.x] = __ldg(src + threadIdx.x);
+        }
+    }
     __syncthreads();
+}
+
+// ------------------------------------------------------------ hopping kernel
+
+// The (re, im) pairs of a storage chunk, and a chunk of an unscaled format from them.
+template <class P>
+__device__ __forceinline__ void chunk_pairs(const typename P::chunk &c, float2 *v) {
+    if constexpr (std::is_same<P, PF32>::value) {
+        v[0] = f2(c.x, c.y);
+        v[1] = f2(c.z, c.w);
+    } else {
+        v[0] = P::SCALED ? h2f(c.x) : b2f(c.x);
+        v[1] = P::SCALED ? h2f(c.y) : b2f(c.y);
+        v[2] = P::SCALED ? h2f(c.z) : b2f(c.z);
+        v[3] = P::SCALED ? h2f(c.w) : b2f(c.w);
+    }
+}
+template <class P>
+__device__ __forceinline__ typename P::chunk pairs_chunk(const float2 *v) {
+    if constexpr (std::is_same<P, PF32>::value)
+        return make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    else
+        return make_uint4(f2b(v[0].x, v[0].y), f2b(v[1].x, v[1].y), f2b(v[2].x, v[2].y), f2b(v[3].x, v[3].y));
 }
 
 // ------------------------------------------------------------ hopping kernel
@@ -253,100 +295,156 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
     }
 }
 
-// A staged link in shared memory: 9 complex, one 8-byte access each.
-__device__ __forceinline__ void put_link(float *d, const cx<float> u[3][3]) {
-    float2 *q = reinterpret_cast<float2 *>(d);
+// The same for the low-precision formats without a clover term, one storage chunk at a time (few
+// registers live beside the sums) and in two-lane arithmetic.
+template <class P, int EPI, int DOT>
+__device__ __forceinline__ void hop_store_pairs(const HopArgs &a, float kap, int64_t i, float2 acc[12],
+                                                float sums[PART_MAX]) {
+    using SH = typename ShadowOf<P>::type;
+    using C = typename P::chunk;
+    constexpr int NC = 12 / P::NCH;  // complex components per chunk
+    constexpr bool WITH_V1 = EPI != EPI_PLAIN, WITH_RH = DOT == DOT_RHAT || DOT == DOT_TS;
+    const float cw = EPI == EPI_DIRAC ? 1.f / (2.f * kap) : 1.f;
+    const float ca = EPI == EPI_DIRAC ? -0.5f : EPI == EPI_MHAT ? -kap * kap : kap;
+    const float sw = (WITH_V1 && P::SCALED) ? __ldg(a.v1.scale + i) : 1.f;
+    const float sr = (WITH_RH && SH::SCALED) ? __ldg(a.rh.scale + i) : 1.f;
+    float2 oo = f2(0.f, 0.f), ww = oo, ow = oo, rw = oo, ro = oo;  // (x.re y.re, x.im y.im) sums
+    float owi = 0.f, rwi = 0.f, roi = 0.f;                          // imaginary parts
+    uint4 q = make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int k = 0; k < 9; k++) q[k] = make_float2(u[k / 3][k % 3].re, u[k / 3][k % 3].im);
-}
-__device__ __forceinline__ void get_link(const float *d, cx<float> u[3][3]) {
-    const float2 *q = reinterpret_cast<const float2 *>(d);
+    for (int j = 0; j < P::NCH; j++) {
+        float2 w[NC], r[NC];
+        if (WITH_V1) {
+            chunk_pairs<P>(__ldg(reinterpret_cast<const C *>(a.v1.p) + j * a.v1.stride + i), w);
 #pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const float2 c = q[k];
-        u[k / 3][k % 3] = mk(c.x, c.y);
+            for (int c = 0; c < NC; c++) {
+                if (P::SCALED) w[c] = __fmul2_rn(f2(sw, sw), w[c]);
+                acc[j * NC + c] = __ffma2_rn(f2(ca, ca), acc[j * NC + c], EPI == EPI_DIRAC ? __fmul2_rn(f2(cw, cw), w[c]) : w[c]);
+            }
+        }
+        if (!P::SCALED) reinterpret_cast<C *>(a.out.p)[j * a.out.stride + i] = pairs_chunk<P>(acc + j * NC);
+        if (WITH_RH) {
+            if constexpr (std::is_same<P, PF32>::value) {
+                // FP32 chunk j is half j % 2 of BF16 chunk j / 2
+                if (j % 2 == 0) q = __ldg(reinterpret_cast<const uint4 *>(a.rh.p) + (j / 2) * a.rh.stride + i);
+                r[0] = b2f(j % 2 ? q.z : q.x);
+                r[1] = b2f(j % 2 ? q.w : q.y);
+            } else {
+                chunk_pairs<P>(__ldg(reinterpret_cast<const C *>(a.rh.p) + j * a.rh.stride + i), r);
+                if (SH::SCALED)
+#pragma unroll
+                    for (int c = 0; c < NC; c++) r[c] = __fmul2_rn(f2(sr, sr), r[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+            const float2 o = acc[j * NC + c];
+            if (DOT == DOT_TS || DOT == DOT_NORM) oo = __ffma2_rn(o, o, oo);
+            if (DOT == DOT_TS) {
+                ww = __ffma2_rn(w[c], w[c], ww);
+                ow = __ffma2_rn(o, w[c], ow);
+                owi = fmaf(o.x, w[c].y, fmaf(-o.y, w[c].x, owi));
+                rw = __ffma2_rn(r[c], w[c], rw);
+                rwi = fmaf(r[c].x, w[c].y, fmaf(-r[c].y, w[c].x, rwi));
+            }
+            if (WITH_RH) {
+                ro = __ffma2_rn(r[c], o, ro);
+                roi = fmaf(r[c].x, o.y, fmaf(-r[c].y, o.x, roi));
+            }
+        }
+    }
+    if (P::SCALED) {
+        float o[24];
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+            o[2 * c] = acc[c].x;
+            o[2 * c + 1] = acc[c].y;
+        }
+        store_spinor<P>(a.out, i, o);
+    }
+    if (DOT == DOT_NORM) sums[0] = oo.x + oo.y;
+    if (DOT == DOT_RHAT) {
+        sums[0] = ro.x + ro.y;
+        sums[1] = roi;
+    }
+    if (DOT == DOT_TS) {
+        sums[0] = ow.x + ow.y;  // (t, s) with t = out, s = v1
+        sums[1] = owi;
+        sums[2] = rw.x + rw.y;  // (rh, s)
+        sums[3] = rwi;
+        sums[4] = ro.x + ro.y;  // (rh, t)
+        sums[5] = roi;
+        sums[6] = oo.x + oo.y;  // (t, t)
+        sums[7] = ww.x + ww.y;  // (s, s)
     }
 }
 
-template <class P, int EPI, int DOT, bool CLOV = false>
+// A staged link in shared memory: 9 entries.
+__device__ __forceinline__ void put_link(float2 *q, const cx<float> u[3][3]) {
+#pragma unroll
+    for (int k = 0; k < 9; k++) q[k] = f2(u[k / 3][k % 3].re, u[k / 3][k % 3].im);
+}
+
 // Resident blocks per SM the register budget of the 32- and 16-bit stencils is fitted to
 // (3: 56 registers a thread; 2: 80).
 #ifndef DDP_HOP_MINB
 #define DDP_HOP_MINB 3
 #endif
 
-__global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
-    using R = typename P::real;
-    constexpr int TSMAX = HOP_TS;
-    __shared__ Item it;
-    // oriented link of hop slot q at s_u[q * 18]: 9 complex; vector reads of
-    // consecutive slots by a warp fall in distinct banks
-    constexpr int LP = 18;
-    __shared__ int s_nb[8 * TSMAX];
-    __shared__ __align__(16) R s_u[8 * TSMAX * LP];
-    load_item(a.L, it);
+template <class P, int EPI, int DOT, bool CLOV = false>
+__global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(const __grid_constant__ HopArgs a) {
     constexpr int TS = HOP_TS;
+    // oriented link of hop slot q at s_u[q * 9]; consecutive slots fall in distinct banks
+    __shared__ __align__(16) Item it;
+    __shared__ int s_nb[8 * TS];
+    __shared__ float2 s_u[8 * TS * 9];
+    load_item(a.L, it);
+    const TileCoord tc0 = tile_coord(it, a.L);
     if (a.skip) {
         // a block whose columns are all finished has nothing to stage or compute
-        const int cg = (blockIdx.x - it.blk0) / it.ntiles;
-        const int col = cg * a.L.CG + (int)threadIdx.x;
+        const int col = tc0.col - (int)threadIdx.x / TS + (int)threadIdx.x;
         int live = 0;
-        if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
-            const SolveState &S = a.st[it.solve0 + col];
-            live = !skipped(S, a.skip);
-        }
+        if ((int)threadIdx.x < a.L.CG && col < it.ncol) live = !skipped(a.st[it.solve0 + col], a.skip);
         if (!__syncthreads_or(live)) return;
     }
-    if (std::is_same<P, PF32>::value) {
+    if (std::is_same<P, PF32>::value && tc0.valid) {
         // FP32 storage: the forward time-direction neighbour of this thread's site-column is
         // requested into L1 before the links are staged, so that its latency overlaps the
-        // staging (measured on 48x24^3, 12 columns: 2.7-3.3% off each inner-loop stencil;
-        // with the backward one too, or with 16-bit storage, less or nothing)
-        const TileCoord t0 = tile_coord(it, a.L);
-        if (t0.valid) {
-            const int v3h = it.nh / it.e[0];  // sites of one parity in a time slice
-            int nbf = t0.h + v3h;
-            if (nbf >= it.nh) nbf -= it.nh;
-            const float4 *base = reinterpret_cast<const float4 *>(a.in.p) + t0.cb + nbf;
+        // staging (with the backward one too, or with 16-bit storage, it gains less or nothing)
+        const int v3h = it.nh / it.e[0];  // sites of one parity in a time slice
+        int nbf = tc0.h + v3h;
+        if (nbf >= it.nh) nbf -= it.nh;
+        const float4 *base = reinterpret_cast<const float4 *>(a.in.p) + tc0.cb + nbf;
 #pragma unroll
-            for (int j = 0; j < P::NCH; j++) asm volatile("prefetch.global.L1 [%0];" ::"l"(base + j * a.in.stride));
-        }
+        for (int j = 0; j < P::NCH; j++) asm volatile("prefetch.global.L1 [%0];" ::"l"(base + j * a.in.stride));
     }
-    {
-        const int tile = (blockIdx.x - it.blk0) % it.ntiles;
-        for (int q = threadIdx.x; q < 8 * TS; q += blockDim.x) {
-            const int d = q / TS, sidx = q - d * TS, h = tile * TS + sidx;
-            int nb = -1;
-            cx<R> u[3][3];
-            if (h < it.nh) nb = stage_hop<P>(it, h, a.p, d, u);
-            s_nb[q] = nb;
-            if (nb >= 0) put_link(s_u + q * LP, u);
-        }
+    for (int q = threadIdx.x; q < 8 * TS; q += blockDim.x) {
+        const int d = q / TS, h = tc0.tile * TS + (q - d * TS);
+        int nb = -1;
+        cx<float> u[3][3];
+        if (h < it.nh) nb = stage_hop<P>(it, h, a.p, d, u);
+        s_nb[q] = nb;
+        if (nb >= 0) put_link(s_u + q * 9, u);
     }
     __syncthreads();
-    TileCoord tc = tile_coord(it, a.L);
-    if (a.skip && tc.valid) {
-        const SolveState &S = a.st[it.solve0 + tc.col];
-        if (skipped(S, a.skip)) tc.valid = false;
-    }
-    R sums[PART_MAX] = {};
-    if (tc.valid) {
-        cx<R> acc[4][3];
+    const TileCoord tc = tile_coord(it, a.L);  // formed again: nothing of it was held in registers meanwhile
+    const bool valid = tc.valid && !(a.skip && skipped(a.st[it.solve0 + tc.col], a.skip));
+    float sums[PART_MAX] = {};
+    if (valid) {
+        float2 acc[4][3];
 #pragma unroll
         for (int s2 = 0; s2 < 4; s2++)
 #pragma unroll
-            for (int c = 0; c < 3; c++) acc[s2][c] = mk<R>(0, 0);
+            for (int c = 0; c < 3; c++) acc[s2][c] = f2(0.f, 0.f);
         const int sl = tc.h - tc.tile * TS;
 #define DDP_HOP_STEP(D)                                                   \
         {                                                                 \
-            const int q = (D) * TS + sl;                                  \
-            const int nb = s_nb[q];                                       \
+            const int nb = s_nb[(D) * TS + sl];                           \
             if (nb >= 0) {                                                \
-                R v[24], f;                                               \
-                load_spinor_raw<P>(a.in, tc.cb + nb, v, &f);              \
-                cx<R> u[3][3];                                            \
-                get_link(s_u + q * LP, u);                                \
-                hop_step<D, P::NCH != 6>(v, u, acc, f);                   \
+                float2 v[12];                                             \
+                float f;                                                  \
+                load_pairs<P>(a.in, a.off, tc.cb + nb, v, &f);           \
+                f2_hop_step<D, P::SCALED>(v, s_u + ((D) * TS + sl) * 9, acc, f); \
             }                                                             \
         }
         DDP_HOP_STEP(0)
@@ -358,7 +456,14 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(HopArgs a) {
         DDP_HOP_STEP(6)
         DDP_HOP_STEP(7)
 #undef DDP_HOP_STEP
-        hop_store_epilogue<P, EPI, DOT, CLOV>(a, it, tc, acc, sums);
+        if constexpr (CLOV) {
+            cx<float> c4[4][3];
+#pragma unroll
+            for (int j = 0; j < 12; j++) c4[j / 3][j % 3] = mk(acc[j / 3][j % 3].x, acc[j / 3][j % 3].y);
+            hop_store_epilogue<P, EPI, DOT, true>(a, it, tc, c4, sums);
+        } else {
+            hop_store_pairs<P, EPI, DOT>(a, (float)it.kappa, tc.cb + tc.h, &acc[0][0], sums);
+        }
     }
     if (DOT != DOT_NONE) warp_partials<DOT != DOT_NONE ? dot_sums(DOT) : 1>(it, tc, sums, a.part);
 }
@@ -442,9 +547,9 @@ __device__ __forceinline__ void xrp_update(R x[2], R p[2], R s[2], const R t[2],
 }
 
 template <class P, int OP>
-__global__ void __launch_bounds__(512) k_blas(BlasArgs a) {
+__global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a) {
     using R = typename P::real;
-    __shared__ Item it;
+    __shared__ __align__(16) Item it;
     load_item(a.L, it);
     TileCoord tc = tile_coord(it, a.L);
     if (a.skip && tc.valid && !a.st[it.solve0 + tc.col].active) tc.valid = false;
@@ -545,9 +650,9 @@ struct ConvArgs {
 // lo = scale * hi  (scale = 2 kappa / sigma: the normalised defect), times T^-1
 // of the site when a.clov is set
 template <class P>
-__global__ void __launch_bounds__(512) k_to_low(ConvArgs a) {
+__global__ void __launch_bounds__(512) k_to_low(const __grid_constant__ ConvArgs a) {
     using R = typename P::real;
-    __shared__ Item it;
+    __shared__ __align__(16) Item it;
     load_item(a.L, it);
     TileCoord tc = tile_coord(it, a.L);
     if (!tc.valid) return;
@@ -564,9 +669,9 @@ __global__ void __launch_bounds__(512) k_to_low(ConvArgs a) {
 
 // hi += sigma * lo  (FP64 accumulation of the correction)
 template <class P>
-__global__ void __launch_bounds__(512) k_accum(ConvArgs a) {
+__global__ void __launch_bounds__(512) k_accum(const __grid_constant__ ConvArgs a) {
     using R = typename P::real;
-    __shared__ Item it;
+    __shared__ __align__(16) Item it;
     load_item(a.L, it);
     TileCoord tc = tile_coord(it, a.L);
     if (!tc.valid) return;
@@ -878,8 +983,8 @@ struct FxArgs {
     int skip;
 };
 
-static __global__ void __launch_bounds__(384) k_to_fx(FxArgs a) {
-    __shared__ Item it;
+static __global__ void __launch_bounds__(384) k_to_fx(const __grid_constant__ FxArgs a) {
+    __shared__ __align__(16) Item it;
     load_item(a.L, it);
     const TileCoord tc = tile_coord(it, a.L);
     if (!tc.valid) return;
@@ -901,14 +1006,14 @@ static __global__ void __launch_bounds__(384) k_to_fx(FxArgs a) {
 // projection), so one block of 12 warps per SM: the multiply-add pipe is 47% busy, the rest waits
 // for neighbours (L2) and for the staging.
 template <int EPI, int DOT, bool CLOV, bool OUTFX>
-__global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
+__global__ void __launch_bounds__(384, 1) k_hop_fx(const __grid_constant__ HopArgs a) {
     constexpr int TS = HOP_TS;
-    __shared__ Item it;
+    __shared__ __align__(16) Item it;
     __shared__ int s_nb[8 * TS];
     __shared__ __align__(16) int4 s_u[8 * TS * 9];
     load_item(a.L, it);
     if (a.skip) {
-        const int cg = (blockIdx.x - it.blk0) / it.ntiles;
+        const int cg = fdiv(blockIdx.x - it.blk0, it.by_nt);
         const int col = cg * a.L.CG + (int)threadIdx.x;
         int live = 0;
         if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
@@ -918,7 +1023,7 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(HopArgs a) {
         if (!__syncthreads_or(live)) return;
     }
     {
-        const int tile = (blockIdx.x - it.blk0) % it.ntiles;
+        const int lb = blockIdx.x - it.blk0, tile = lb - fdiv(lb, it.by_nt) * it.ntiles;
         for (int q = threadIdx.x; q < 8 * TS; q += blockDim.x) {
             const int d = q / TS, h = tile * TS + (q - d * TS);
             int nb = -1;

@@ -41,6 +41,7 @@ inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const F
         return 2;
     } else {
         (void)fx;
+        for (int j = 0; j < 6; j++) a.off[j] = (int64_t)j * a.in.stride * (int64_t)sizeof(typename Q::chunk);
         k_hop<Q, EPI, DOT, CL><<<nblocks, threads, 0, ctx->stream>>>(a);
         return 1;
     }
@@ -309,10 +310,7 @@ struct Engine {
     // Upload the work table of the current plan and the per-column states.
     int upload(const std::vector<SolveState> &states) {
         cudaStream_t st = ctx->stream;
-        L.items = d_items;
-        L.nitems = (int)plan.items.size();
-        L.TS = plan.TS;
-        L.CG = plan.CG;
+        L = make_launch(plan, d_items);
         threads = plan.TS * plan.CG;
         h_st = states;
         for (SolveState &S : h_st) {
@@ -525,11 +523,7 @@ int apply_dirac_impl(ddp_ctx *ctx, const Job &job, const double *psi, double *ou
     int64_t nt = 2 * (int64_t)pa.it.nh * pa.it.ncol;
     unsigned nb = (unsigned)((nt + 255) / 256);
     k_pack_low<P><<<nb, 256, 0, st>>>(pa, ie, io);
-    Launch L;
-    L.items = d_items;
-    L.nitems = 1;
-    L.TS = plan.TS;
-    L.CG = plan.CG;
+    const Launch L = make_launch(plan, d_items);
     FieldView none = {nullptr, nullptr, 0};
     HopArgs h;
     h.st = nullptr;
@@ -600,11 +594,7 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
         DDP_CUDA(ctx, cudaMemsetAsync(v1.scale, 0, NF * sizeof(float), st));
         DDP_CUDA(ctx, cudaMemsetAsync(rhv.scale, 0, NF * sizeof(float), st));
     }
-    Launch L;
-    L.items = d_items;
-    L.nitems = 1;
-    L.TS = plan.TS;
-    L.CG = plan.CG;
+    const Launch L = make_launch(plan, d_items);
     HopArgs h;
     FieldView none = {nullptr, nullptr, 0};
     h.st = nullptr;

@@ -281,14 +281,14 @@ __device__ __noinline__ void fx_slow(const FieldView &in, int64_t cb, const int 
             l[j / 3][j % 3] = mk(fx_value(fx_join(c.x, c.y), -FX_LINK), fx_value(fx_join(c.z, c.w), -FX_LINK));
         }
         switch (d) {
-            case 0: hop_step<0, true>(v, l, acc, 1.0); break;
-            case 1: hop_step<1, true>(v, l, acc, 1.0); break;
-            case 2: hop_step<2, true>(v, l, acc, 1.0); break;
-            case 3: hop_step<3, true>(v, l, acc, 1.0); break;
-            case 4: hop_step<4, true>(v, l, acc, 1.0); break;
-            case 5: hop_step<5, true>(v, l, acc, 1.0); break;
-            case 6: hop_step<6, true>(v, l, acc, 1.0); break;
-            default: hop_step<7, true>(v, l, acc, 1.0); break;
+            case 0: hop_step<0>(v, l, acc, 1.0); break;
+            case 1: hop_step<1>(v, l, acc, 1.0); break;
+            case 2: hop_step<2>(v, l, acc, 1.0); break;
+            case 3: hop_step<3>(v, l, acc, 1.0); break;
+            case 4: hop_step<4>(v, l, acc, 1.0); break;
+            case 5: hop_step<5>(v, l, acc, 1.0); break;
+            case 6: hop_step<6>(v, l, acc, 1.0); break;
+            default: hop_step<7>(v, l, acc, 1.0); break;
         }
     }
     for (int j = 0; j < 12; j++) {

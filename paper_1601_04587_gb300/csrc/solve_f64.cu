@@ -39,11 +39,7 @@ int hop_power_fx(ddp_ctx *ctx, const Job &job, int p, const double *psi, double 
     const int64_t nt = 2 * (int64_t)pa.it.nh * pa.it.ncol;
     const unsigned nb = (unsigned)((nt + 255) / 256);
     k_pack_fx<<<nb, 256, 0, st>>>(pa, f[0][0], f[0][1]);
-    Launch L;
-    L.items = d_items;
-    L.nitems = 1;
-    L.TS = plan.TS;
-    L.CG = plan.CG;
+    const Launch L = make_launch(plan, d_items);
     FieldView none = {nullptr, nullptr, 0};
     HopArgs h;
     h.st = nullptr;
