@@ -314,7 +314,10 @@ int ddp_poll(ddp_ctx *ctx, uint64_t ticket, int *done, ddp_solve_info *info);
  * tensor cores and the Cholesky-QR update A <- A R^-1 in double-FP32; 0: direct FP64
  * kernels), "overlap_downloads" (1, the default: ddp_propagator_series with host
  * outputs solves the smaller nested domains first and copies their results to the host
- * while the largest domain solves; 0: one batched solve, then the copies).
+ * while the largest domain solves; 0: one batched solve, then the copies),
+ * "small_domain_sites" (domains of at most that many sites per parity are solved on chip
+ * by one kernel per correction cycle, storage formats FP32, FP16 and BF16 without the clover
+ * term; default and maximum 1024, 0: none).
  * DDP_ERR_INVALID_ARG for unknown names or values. */
 int ddp_set_param(ddp_ctx *ctx, const char *name, double value);
 

@@ -105,6 +105,55 @@ void make_plan(const std::vector<Job> &jobs, int prec, const EngineParams &prm, 
     plan.npart = std::max<int64_t>(pbase, 1);
 }
 
+int small_cut(const int e[4], int max_cluster, int c[4], int b[4]) {
+    int best = 0;
+    int64_t surface = 0;
+    int t[4], x[4];
+    for (t[0] = 1; t[0] <= max_cluster; t[0]++)
+        for (t[1] = 1; t[0] * t[1] <= max_cluster; t[1]++)
+            for (t[2] = 1; t[0] * t[1] * t[2] <= max_cluster; t[2]++)
+                for (t[3] = 1; t[0] * t[1] * t[2] * t[3] <= max_cluster; t[3]++) {
+                    const int n = t[0] * t[1] * t[2] * t[3];
+                    int64_t vol = 1;
+                    bool ok = true;
+                    for (int m = 0; m < 4; m++) {
+                        x[m] = (e[m] + t[m] - 1) / t[m];
+                        if (m == 3) x[m] += x[m] & 1;
+                        ok = ok && (t[m] - 1) * x[m] < e[m];  // no empty block
+                        vol *= x[m];
+                    }
+                    if (!ok || vol / 2 > SMALL_SITES) continue;
+                    int64_t s = 0;  // sites of a block with a neighbour in another one
+                    for (int m = 0; m < 4; m++) s += t[m] > 1 ? vol / x[m] : 0;
+                    if (best && (n > best || (n == best && s >= surface))) continue;
+                    best = n;
+                    surface = s;
+                    memcpy(c, t, sizeof(t));
+                    memcpy(b, x, sizeof(x));
+                }
+    return best;
+}
+
+void plan_classes(const std::vector<int> &cls, int max_cluster, Plan &plan) {
+    plan.nlarge = plan.nblocks_large = plan.nsolve_large = 0;
+    plan.small.clear();
+    for (size_t i = 0; i < cls.size(); i++) {
+        Item &it = plan.items[i];
+        if (!cls[i]) {
+            plan.nlarge++;
+            plan.nblocks_large += it.ntiles * it.ncg;
+            plan.nsolve_large += it.ncol;
+            continue;
+        }
+        if (plan.small.empty() || plan.small.back().csize != cls[i]) plan.small.push_back({cls[i], (int)i, 0, 0});
+        Plan::Small &g = plan.small.back();
+        it.sblk0 = g.nclusters;
+        small_cut(it.e, max_cluster, it.sc, it.sb);
+        g.nitems++;
+        g.nclusters += (it.ncol + SMALL_COLS - 1) / SMALL_COLS;
+    }
+}
+
 int solve_jobs_dispatch(ddp_ctx *ctx, int prec, std::vector<Job> &jobs, std::vector<JobInfo> &infos) {
     switch (prec) {
         case DDP_PREC_FP64: return solve_jobs<PF64>(ctx, prec, jobs, infos);
@@ -1171,7 +1220,7 @@ static int prec_suffix(const std::string &n, const char *stem) {
 
 // Tuning knobs of the solver (names: max_outer, max_inner, delta_fp32,
 // delta_fp16, delta_bf16, delta_fp64, tile_sites, tile_cols, conditional, stencil_carveout, projector_tensor_cores, contraction_double_fp32,
-// overlap_downloads, tuned_cols_*, tuned_carveout_*).
+// overlap_downloads, small_domain_sites, tuned_cols_*, tuned_carveout_*).
 int ddp_set_param(ddp_ctx *ctx, const char *name, double value) {
     if (!ctx || !name) return DDP_ERR_INVALID_ARG;
     EngineParams &p = ctx->prm;
@@ -1191,6 +1240,10 @@ int ddp_set_param(ddp_ctx *ctx, const char *name, double value) {
     else if (n == "projector_tensor_cores") p.proj_tc = value != 0;
     else if (n == "contraction_double_fp32") p.contract_dd = value != 0;
     else if (n == "overlap_downloads") p.overlap_downloads = value != 0;
+    else if (n == "small_domain_sites") {
+        if (value < 0 || value > SMALL_MAX_NH) return DDP_ERR_INVALID_ARG;
+        p.small_sites = (int)value;
+    }
     else if (n == "stencil_carveout") {
         if (value < -1 || value > 100) return DDP_ERR_INVALID_ARG;
         p.carveout = (int)value;
@@ -1221,6 +1274,7 @@ int ddp_get_param(const ddp_ctx *ctx, const char *name, double *value) {
     else if (n == "projector_tensor_cores") *value = p.proj_tc;
     else if (n == "contraction_double_fp32") *value = p.contract_dd;
     else if (n == "overlap_downloads") *value = p.overlap_downloads;
+    else if (n == "small_domain_sites") *value = p.small_sites;
     else if (n == "stencil_carveout") *value = p.carveout;
     else if (prec_suffix(n, "tuned_cols") >= 0) *value = p.CG_prec[prec_suffix(n, "tuned_cols")];
     else if (prec_suffix(n, "tuned_carveout") >= 0) *value = p.carveout_prec[prec_suffix(n, "tuned_carveout")];

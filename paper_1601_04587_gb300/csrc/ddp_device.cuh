@@ -360,6 +360,9 @@ struct __align__(16) Item {
     int ncg;         // ceil(ncol / CG)
     int blk0;
     int solve0;      // first solve (column) index
+    // small domains (small.cuh): first cluster in the launch of their cluster size; blocks of a
+    // cluster along each direction, and the extents of a block's sub-box (the last one even)
+    int sblk0, sc[4], sb[4];
     int64_t fbase;
     int64_t pbase;
     double kappa;
@@ -509,14 +512,12 @@ __device__ __forceinline__ void accumulate(cx<R> acc[4][3], const cx<R> w[2][3],
     }
 }
 
-// Geometry of one hop d = 2 mu + (backward ? 1 : 0) from even-odd site h of
-// parity p: the neighbour's even-odd index (or -1 when the hop is dropped), the
-// row of the link the neighbour is transported with, U_mu(x) forward and
-// U_mu(x - mu)^+ backward, and whether the hop changes sign (across an
+// The neighbour of local coordinates k (replaced by the neighbour's) in hop d = 2 mu + (backward ?
+// 1 : 0) from parity p: false when the hop is dropped; the row of the link it is transported with,
+// U_mu(x) forward and U_mu(x - mu)^+ backward, and whether the hop changes sign (across an
 // antiperiodic time boundary).
-__device__ __forceinline__ int hop_geometry(const Item &it, int h, int p, int d, int64_t &row, bool &neg) {
-    int k[4], x[4];
-    decode_site(it, h, p, k);
+__device__ __forceinline__ bool hop_neighbour(const Item &it, int k[4], int p, int d, int64_t &row, bool &neg) {
+    int x[4];
 #pragma unroll
     for (int m = 0; m < 4; m++) {
         int t = it.o[m] + k[m];
@@ -524,35 +525,41 @@ __device__ __forceinline__ int hop_geometry(const Item &it, int h, int p, int d,
     }
     const int mu = d >> 1;
     const bool fwd = !(d & 1);
-    int kn[4] = {k[0], k[1], k[2], k[3]};
     bool ok = true;
     const bool restricted = (it.rmask >> mu) & 1;
     if (fwd) {
-        kn[mu] += 1;
+        k[mu] += 1;
         if (restricted)
-            ok = kn[mu] < it.e[mu];
-        else if (kn[mu] == it.e[mu])
-            kn[mu] = 0;
+            ok = k[mu] < it.e[mu];
+        else if (k[mu] == it.e[mu])
+            k[mu] = 0;
     } else {
-        kn[mu] -= 1;
+        k[mu] -= 1;
         if (restricted)
-            ok = kn[mu] >= 0;
-        else if (kn[mu] < 0)
-            kn[mu] = it.e[mu] - 1;
+            ok = k[mu] >= 0;
+        else if (k[mu] < 0)
+            k[mu] = it.e[mu] - 1;
     }
     neg = false;
     if (mu == 0 && x[0] == (fwd ? it.L[0] - 1 : 0)) {
         neg = it.bc == 1;
         if (it.bc == 2) ok = false;
     }
-    if (!ok) return -1;
+    if (!ok) return false;
     if (fwd) {
         row = link_row(it, x, p);
     } else {
         x[mu] = (x[mu] == 0) ? it.L[mu] - 1 : x[mu] - 1;
         row = link_row(it, x, p ^ 1);
     }
-    return local_lex(it, kn) >> 1;
+    return true;
+}
+
+// The same from even-odd site h: the neighbour's even-odd index, -1 when the hop is dropped.
+__device__ __forceinline__ int hop_geometry(const Item &it, int h, int p, int d, int64_t &row, bool &neg) {
+    int k[4];
+    decode_site(it, h, p, k);
+    return hop_neighbour(it, k, p, d, row, neg) ? local_lex(it, k) >> 1 : -1;
 }
 
 // The neighbour's index of a hop and its link in storage format P, oriented and

@@ -14,6 +14,7 @@
 #include "ddp.h"
 #include "ddp_kernels.cuh"
 #include "clover.cuh"
+#include "small.cuh"
 
 namespace ddp {
 
@@ -87,6 +88,7 @@ struct EngineParams {
     int carveout = 28;
     // the carveout ddp_autotune chose for a storage format (-2: none, use carveout)
     int carveout_prec[4] = {-2, -2, -2, -2};
+    int small_sites = SMALL_MAX_NH;  // largest domain (sites per parity) solved on chip in one kernel (0: none)
     int contract_dd = 1;        // nucleon contraction in double-FP32 arithmetic (0: FP64)
     int proj_tc = 1;            // projector-cut Gram blocks and colourless sums on the tensor cores (0: FP64 kernels)
     // ddp_propagator_series with host outputs: solve the smaller nested domains first and
@@ -139,6 +141,7 @@ struct ddp_ctx {
     ddp::Arena aux;       // partial sums of the projector-cut kernels
     cudaStream_t copy_stream = nullptr;  // device-to-host copies overlapped with compute (created on first use)
     void *serve = nullptr;
+    int max_cluster = -1;  // largest cluster of the small-domain kernel the device runs (-1: not asked yet)
     // instrumentation: per-kernel-class launch counts of the last solve
     long launches = 0;
 };
@@ -208,6 +211,13 @@ struct Plan {
     int64_t npart = 0;     // partial slots
     int nblocks = 0;
     int nsolve = 0;
+    // the leading items, which take the per-step kernels; the others are small domains
+    // (small.cuh), grouped by the number of blocks per cluster
+    int nlarge = 0, nblocks_large = 0, nsolve_large = 0;
+    struct Small {
+        int csize, item0, nitems, nclusters;
+    };
+    std::vector<Small> small;
 };
 
 // The launch description of a plan whose items are at d_items on the device.
@@ -224,6 +234,21 @@ inline Launch make_launch(const Plan &plan, const Item *d_items) {
 }
 
 void make_plan(const std::vector<Job> &jobs, int prec, const EngineParams &prm, Plan &plan);
+
+// The cut of a box into at most max_cluster sub-boxes (c blocks along each direction, extents b)
+// of at most SMALL_SITES sites per parity, b[3] even: fewest blocks first, then least surface.
+// Returns the number of blocks, 0 if there is no such cut.
+int small_cut(const int e[4], int max_cluster, int c[4], int b[4]);
+// The class of a job: 0 for the per-step kernels, else its blocks per cluster (small.cuh).  By the
+// job alone, not by what it is solved with.
+inline int job_class(const Job &j, int prec, const EngineParams &prm, int max_cluster) {
+    const int64_t nh = (int64_t)j.e[0] * j.e[1] * j.e[2] * j.e[3] / 2;
+    int c[4], b[4];
+    if (prec == DDP_PREC_FP64 || j.clov || nh > prm.small_sites) return 0;
+    return small_cut(j.e, max_cluster, c, b);
+}
+// Marks the large and the small items of a plan whose jobs are sorted by class.
+void plan_classes(const std::vector<int> &cls, int max_cluster, Plan &plan);
 
 template <class P>
 inline size_t field_bytes(int64_t nfield) {

@@ -68,6 +68,43 @@ inline cudaError_t set_hop_carveout(int percent) {
     return e;
 }
 
+// Launch configuration of the small-domain kernel.
+template <class P>
+inline void small_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute attr[1], int csize, int nclusters) {
+    cfg.gridDim = dim3((unsigned)(nclusters * csize));
+    cfg.blockDim = dim3(SMALL_THREADS);
+    cfg.dynamicSmemBytes = sizeof(SmallShared);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)csize;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
+// The largest cluster of the small-domain kernel this device runs (asked once per context), with
+// the kernel's attributes set; 0: none.
+template <class P>
+inline int small_clusters(ddp_ctx *ctx) {
+    if constexpr (P::IS64) {
+        return 0;
+    } else {
+        const bool set = cudaFuncSetAttribute(k_small<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)sizeof(SmallShared)) == cudaSuccess;
+        if (ctx->max_cluster < 0) {
+            ctx->max_cluster = 0;
+            for (int c = SMALL_MAX_CLUSTER; set && c > 0 && !ctx->max_cluster; c /= 2) {
+                cudaLaunchConfig_t cfg = {};
+                cudaLaunchAttribute attr[1];
+                small_config<P>(cfg, attr, c, 1);
+                int n = 0;
+                if (cudaOccupancyMaxActiveClusters(&n, k_small<P>, &cfg) == cudaSuccess && n > 0) ctx->max_cluster = c;
+            }
+            cudaGetLastError();
+        }
+        return ctx->max_cluster;
+    }
+}
+
 template <class P>
 struct Engine {
     ddp_ctx *ctx;
@@ -90,6 +127,7 @@ struct Engine {
     cudaGraphExec_t loop_exec = nullptr;
     cudaGraph_t loop_graph = nullptr;
     long launches = 0;
+    int grid = 0, solves = 0;  // blocks and columns of the next launches: of all items, or of the large ones
     bool clov = false;  // some item of the plan has a clover term
 
     ~Engine() {
@@ -115,7 +153,7 @@ struct Engine {
 
     template <class Q, int EPI, int DOT, bool CL = false>
     void hop(const HopArgs &a) {
-        launches += launch_hop<Q, EPI, DOT, CL>(ctx, plan.nblocks, threads, a, EPI == EPI_RESID ? fx_outer : fx_inner);
+        launches += launch_hop<Q, EPI, DOT, CL>(ctx, grid, threads, a, EPI == EPI_RESID ? fx_outer : fx_inner);
     }
 
     template <class Q, int OP>
@@ -132,7 +170,7 @@ struct Engine {
         a.t = t;
         a.st = d_st;
         a.part = part;
-        k_blas<Q, OP><<<plan.nblocks, threads, 0, ctx->stream>>>(a);
+        k_blas<Q, OP><<<grid, threads, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -140,13 +178,13 @@ struct Engine {
     void fin() {
         FinArgs a;
         a.st = d_st;
-        a.nsolve = plan.nsolve;
+        a.nsolve = solves;
         a.A = A;
         a.B = B;
         a.ctl = d_ctl;
         a.loop_mode = FIN == FIN_OMEGA ? loop_mode : 0;
         a.loop = loop_handle;
-        k_fin<FIN><<<plan.nsolve, FIN_THREADS, 0, ctx->stream>>>(a);
+        k_fin<FIN><<<solves, FIN_THREADS, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -158,7 +196,7 @@ struct Engine {
         a.x = f;
         a.st = d_st;
         a.part = part;
-        k_blas<PF64, OP_NORM><<<plan.nblocks, threads, 0, ctx->stream>>>(a);
+        k_blas<PF64, OP_NORM><<<grid, threads, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -172,9 +210,9 @@ struct Engine {
         a.p = par;
         a.clov = clov_inv ? 1 : 0;
         if (to_low)
-            k_to_low<P><<<plan.nblocks, threads, 0, ctx->stream>>>(a);
+            k_to_low<P><<<grid, threads, 0, ctx->stream>>>(a);
         else
-            k_accum<P><<<plan.nblocks, threads, 0, ctx->stream>>>(a);
+            k_accum<P><<<grid, threads, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -199,7 +237,16 @@ struct Engine {
             iteration_body_t<false>();
     }
 
+    // The inner loop of the large items as a graph (nothing to build without any).
     int build_loop_graph() {
+        if (!plan.nlarge) return DDP_OK;
+        large_items();
+        const int rc = capture_loop();
+        all_items();
+        return rc;
+    }
+
+    int capture_loop() {
         cudaStream_t st = ctx->stream;
         DDP_CUDA(ctx, (set_hop_carveout<P, false>(carveout_for(ctx->prm, prec))));
         DDP_CUDA(ctx, (set_hop_carveout<P, true>(carveout_for(ctx->prm, prec))));
@@ -307,11 +354,21 @@ struct Engine {
         d_ctl = (LoopCtl *)a.take(sizeof(LoopCtl));
     }
 
+    void all_items() {
+        grid = plan.nblocks;
+        solves = plan.nsolve;
+    }
+    void large_items() {
+        grid = plan.nblocks_large;
+        solves = plan.nsolve_large;
+    }
+
     // Upload the work table of the current plan and the per-column states.
     int upload(const std::vector<SolveState> &states) {
         cudaStream_t st = ctx->stream;
         L = make_launch(plan, d_items);
         threads = plan.TS * plan.CG;
+        all_items();
         h_st = states;
         for (SolveState &S : h_st) {
             const Item &it = plan.items[S.item];
@@ -422,7 +479,38 @@ struct Engine {
         conv(false, tmp, xo);
         return DDP_OK;
     }
-    int correction(bool r_is_eta) { return clov ? correction_t<true>(r_is_eta) : correction_t<false>(r_is_eta); }
+    int correction(bool r_is_eta) {
+        int rc = DDP_OK;
+        if constexpr (!P::IS64) {
+            for (const Plan::Small &g : plan.small)
+                if ((rc = correct_small(g, r_is_eta))) return rc;
+        }
+        if (!plan.nlarge) return DDP_OK;
+        large_items();
+        rc = clov ? correction_t<true>(r_is_eta) : correction_t<false>(r_is_eta);
+        all_items();
+        return rc;
+    }
+
+    // One correction of the small items of one cluster size (small.cuh), in one kernel.
+    int correct_small(const Plan::Small &g, bool r_is_eta) {
+        SmallArgs a;
+        a.items = d_items + g.item0;
+        a.nitems = g.nitems;
+        a.csize = g.csize;
+        a.re = r_is_eta ? be : re64;
+        a.ro = r_is_eta ? bo : ro64;
+        a.xe = xe;
+        a.xo = xo;
+        a.st = d_st;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        small_config<P>(cfg, attr, g.csize, g.nclusters);
+        cfg.stream = ctx->stream;
+        DDP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_small<P>, a));
+        launches++;
+        return DDP_OK;
+    }
 
     void drop_graph() {
         if (loop_exec) cudaGraphExecDestroy(loop_exec);
@@ -433,9 +521,25 @@ struct Engine {
 
     // ----------------------------------------------------------- one-shot solve
 
-    int run(std::vector<Job> &jobs, std::vector<JobInfo> &infos) {
+    int run(const std::vector<Job> &in, std::vector<JobInfo> &infos) {
         const EngineParams &prm = ctx->prm;
+        // the work table in the order of the classes: per-step items first
+        const int maxc = small_clusters<P>(ctx);
+        std::vector<int> cls(in.size());
+        std::vector<size_t> order(in.size());
+        for (size_t i = 0; i < in.size(); i++) {
+            cls[i] = job_class(in[i], prec, prm, maxc);
+            order[i] = i;
+        }
+        std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return cls[x] < cls[y]; });
+        std::vector<Job> jobs;
+        std::vector<int> sorted;
+        for (size_t i : order) {
+            jobs.push_back(in[i]);
+            sorted.push_back(cls[i]);
+        }
         make_plan(jobs, prec, prm, plan);
+        plan_classes(sorted, maxc, plan);
         clov = false;
         for (auto &j : jobs) clov = clov || j.clov;
         DDP_CUDA(ctx, ctx->ws.reserve(bytes_needed(plan.nfield, plan.npart, (int)plan.items.size(), plan.nsolve)));
@@ -467,7 +571,7 @@ struct Engine {
         infos.assign(jobs.size(), JobInfo());
         for (size_t i = 0; i < jobs.size(); i++) {
             const Item &it = plan.items[i];
-            JobInfo &inf = infos[i];
+            JobInfo &inf = infos[order[i]];
             inf.outer = cycles;
             inf.relres.resize(it.ncol);
             bool ok = true;

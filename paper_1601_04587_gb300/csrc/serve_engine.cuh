@@ -120,9 +120,19 @@ struct Server : ServerBase {
             *in_flight = 0;
             return DDP_OK;
         }
+        // the work table in the order of the classes: per-step items first
+        const int maxc = small_clusters<P>(ctx);
+        std::stable_sort(active.begin(), active.end(), [&](uint64_t x, uint64_t y) {
+            return job_class(reqs[x].job, prec, ctx->prm, maxc) < job_class(reqs[y].job, prec, ctx->prm, maxc);
+        });
         std::vector<Job> jobs;
-        for (uint64_t t : active) jobs.push_back(reqs[t].job);
+        std::vector<int> cls;
+        for (uint64_t t : active) {
+            jobs.push_back(reqs[t].job);
+            cls.push_back(job_class(reqs[t].job, prec, ctx->prm, maxc));
+        }
         make_plan(jobs, prec, ctx->prm, eng.plan);
+        plan_classes(cls, maxc, eng.plan);
         eng.clov = false;  // serving refuses the clover term (ddp_submit)
         std::vector<SolveState> states(eng.plan.nsolve);
         for (size_t i = 0; i < active.size(); i++) {
