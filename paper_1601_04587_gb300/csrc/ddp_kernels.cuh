@@ -8,15 +8,16 @@
 #include "ddp_device.cuh"
 #include "clover.cuh"
 #include "fx64.cuh"
+#include "recur.cuh"
 
 namespace ddp {
 
 // ------------------------------------------------------------ solver state
 
-// Per solve (one column of one request).  Complex scalars as double2.
+// Per solve (one column of one request).  The scalars of the inner recurrence are of the format's
+// scalar type (recur.cuh): FP64, or double-FP32 in the same 8 bytes; scalar() reads them.
 struct SolveState {
     double2 rho, alpha, omega, beta;
-    double rr;       // inner recursive |r|^2
     double target2;  // inner stopping threshold on |r|^2
     double bnorm2;   // |eta|^2 (FP64)
     double rr64;     // |eta - D_Gamma x|^2 of the current outer cycle (FP64)
@@ -38,17 +39,29 @@ struct SolveState {
     double kappa;
 };
 
+template <class T>
+__device__ __forceinline__ Cnum<T> &scalar(double2 &v) {
+    static_assert(sizeof(Cnum<T>) == sizeof(double2), "same storage");
+    return reinterpret_cast<Cnum<T> &>(v);
+}
+// A scalar of the recurrence in the compute precision (for double-FP32 its high part: no conversion).
+__device__ __forceinline__ double2 scalar_value(const double2 &v, double) { return v; }
+__device__ __forceinline__ float2 scalar_value(const double2 &v, float) {
+    const float4 c = reinterpret_cast<const float4 &>(v);
+    return make_float2(c.x, c.z);
+}
+
 struct LoopCtl {
-    int n_active;
+    unsigned long long arrived;  // this iteration: columns decided (low half), columns going on (high half)
     int iter;
     int maxit;
-    int pad;          // host-polled loop: 1 while the loop continues
-    int done_blocks;  // blocks of k_fin<FIN_OMEGA> finished in this iteration
+    int pad;  // host-polled loop: 1 while the loop continues
 };
 
-// Reduction partials: NV sums per (item, column, tile) at d[slot * NV + k], NV = dot_sums(DOT).
+// Reduction partials: NV sums per (item, column, tile) at d[slot * NV + k], NV = dot_sums(DOT), in
+// the precision they were formed in (FP32 or FP64).
 struct Partials {
-    double *d;
+    void *d;
 };
 constexpr int PART_MAX = 8;  // largest NV
 
@@ -127,7 +140,7 @@ __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L)
 // Sums of NV values over the 32 sites of a tile, which are one warp of one column.  Each
 // thread's products and the warp's sums are formed in the compute precision R (FP32 for the
 // low-precision formats: FP64 arithmetic is a small fraction of GB300's FP32 rate); the sums over
-// tiles, in the scalar kernels, are FP64.  Fixed order: results do not depend on the batch
+// tiles, in the scalar kernels, are FP64 or double-FP32.  Fixed order: results do not depend on the batch
 // around them.  The lanes split the values as the distance halves (9 shuffles for 8 values, not
 // 40): value k ends in lanes k * 32 / NV and following.
 template <int NV, typename R>
@@ -146,7 +159,7 @@ __device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &t
 #pragma unroll
     for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
     if (tc.col < it.ncol && (lane & (32 / NV - 1)) == 0)
-        part.d[(it.pbase + (int64_t)tc.col * it.ntiles + tc.tile) * NV + lane / (32 / NV)] = (double)v[0];
+        reinterpret_cast<R *>(part.d)[(it.pbase + (int64_t)tc.col * it.ntiles + tc.tile) * NV + lane / (32 / NV)] = v[0];
 }
 
 // The block's item, copied by words by one warp: from the kernel parameters where the launch
@@ -561,7 +574,8 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             R r[24], v[24];
             load_spinor<P>(a.r, i, r);
             load_spinor<P>(a.v, i, v);
-            const R ar = (R)S.alpha.x, ai = (R)S.alpha.y;
+            const auto al = scalar_value(S.alpha, R(0));
+            const R ar = al.x, ai = al.y;
 #pragma unroll
             for (int j = 0; j < 12; j++) {
                 r[2 * j] -= ar * v[2 * j] - ai * v[2 * j + 1];
@@ -583,8 +597,8 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             C *__restrict__ ox = reinterpret_cast<C *>(a.x.p);
             C *__restrict__ orr = reinterpret_cast<C *>(a.r.p);
             C *__restrict__ op = reinterpret_cast<C *>(a.p.p);
-            const R ar = (R)S.alpha.x, ai = (R)S.alpha.y, wr = (R)S.omega.x, wi = (R)S.omega.y;
-            const R br = (R)S.beta.x, bi = (R)S.beta.y;
+            const auto al = scalar_value(S.alpha, R(0)), om = scalar_value(S.omega, R(0)), be = scalar_value(S.beta, R(0));
+            const R ar = al.x, ai = al.y, wr = om.x, wi = om.y, br = be.x, bi = be.y;
 #pragma unroll
             for (int j = 0; j < P::NCH; j++) {
                 const int64_t o = j * a.x.stride + i;
@@ -608,8 +622,8 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             load_spinor<P>(a.s, i, s);
             load_spinor<P>(a.t, i, t);
             load_spinor<P>(a.v, i, v);
-            const R ar = (R)S.alpha.x, ai = (R)S.alpha.y, wr = (R)S.omega.x, wi = (R)S.omega.y;
-            const R br = (R)S.beta.x, bi = (R)S.beta.y;
+            const auto al = scalar_value(S.alpha, R(0)), om = scalar_value(S.omega, R(0)), be = scalar_value(S.beta, R(0));
+            const R ar = al.x, ai = al.y, wr = om.x, wi = om.y, br = be.x, bi = be.y;
 #pragma unroll
             for (int k = 0; k < 12; k++)
                 xrp_update(x + 2 * k, p + 2 * k, s + 2 * k, t + 2 * k, v + 2 * k, ar, ai, wr, wi, br, bi);
@@ -702,67 +716,77 @@ struct FinArgs {
     cudaGraphConditionalHandle loop;
 };
 
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-    double d = b.x * b.x + b.y * b.y;
-    return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
-}
-__device__ __forceinline__ double2 cmuld(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-// One block per solve: fixed-order sum of the solve's tile partials, then the
-// scalar recurrences of BiCGStab (van der Vorst) or of the defect correction.
-//
-// FIN_OMEGA finds omega and, before r is formed, the scalars of the next iteration from the five
-// products of the (t, s) stencil: with r = s - omega t,
-//   (rh, r) = (rh, s) - omega (rh, t),   (r, r) = (s, s) - |(t, s)|^2 / (t, t),
-// so that x, r and p are updated in one pass and an iteration has two reductions.  (r, r) is then
-// good to the rounding of the sums times (s, s), an inner stopping criterion; the true residual
-// of the outer cycle decides convergence.
+// One block per solve: fixed-order sum of the solve's tile partials (in R), then the scalar
+// recurrences of BiCGStab or of the defect correction.  FIN_OMEGA finds omega and the scalars of
+// the next iteration from the five products of the (t, s) stencil (bicg_omega), so that x, r and p
+// are updated in one pass and an iteration has two reductions.  (r, r) is then good to the rounding
+// of the sums times (s, s), an inner stopping criterion; the true residual of the outer cycle
+// decides convergence.
 constexpr int FIN_THREADS = 256;
-template <int FIN>
+template <int FIN, typename R>
 __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
+    using T = typename ScalarOf<R>::type;
     constexpr int NV = FIN == FIN_OMEGA ? PART_MAX : FIN == FIN_ALPHA ? 2 : 1;
     constexpr bool two = (FIN == FIN_BNORM || FIN == FIN_RESID);
-    __shared__ double sh[FIN_THREADS / 32][NV];
+    __shared__ T sh[FIN_THREADS / 32][NV];
     const int s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SolveState &S = a.st[s];
-    const int nt = S.ntiles;
+    const int nt = S.ntiles, active = S.active;
     const int64_t base = S.pbase;
-    double v[NV] = {};
-    const bool wanted = !(FIN == FIN_ALPHA || FIN == FIN_OMEGA) || S.active == 1;
-    if (wanted)
+    // the state the recurrence starts from, read while the partials are on their way
+    Cnum<T> rho = scalar<T>(S.rho), alpha = scalar<T>(S.alpha);
+    T v[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) nset(v[k], 0.0);
+    const bool wanted = !(FIN == FIN_ALPHA || FIN == FIN_OMEGA) || active == 1;
+    if (wanted) {
+        const R *A = reinterpret_cast<const R *>(a.A.d) + base * NV, *B = reinterpret_cast<const R *>(a.B.d) + base;
         for (int t = threadIdx.x; t < nt; t += FIN_THREADS) {
-            if (NV == 1) {
-                v[0] += a.A.d[base + t];
-                if (two) v[0] += a.B.d[base + t];
-            } else {
-                const double2 *q = reinterpret_cast<const double2 *>(a.A.d + (base + t) * NV);
+            R c[NV];
 #pragma unroll
-                for (int k = 0; k < NV / 2; k++) {
-                    const double2 c = q[k];
-                    v[2 * k] += c.x;
-                    v[2 * k + 1] += c.y;
-                }
-            }
+            for (int k = 0; k < NV; k++) c[k] = __ldg(A + (int64_t)t * NV + k);
+#pragma unroll
+            for (int k = 0; k < NV; k++) nsum(v[k], c[k]);
+            if (two) nsum(v[0], __ldg(B + t));
         }
-#pragma unroll
-    for (int k = 0; k < NV; k++) v[k] = warp_sum(v[k]);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; k++) sh[warp][k] = v[k];
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    for (int k = 0; k < NV; k++) {
-        v[k] = sh[0][k];
-        for (int w = 1; w < FIN_THREADS / 32; w++) v[k] += sh[w][k];
     }
-    const double n = v[0];
-    const double2 zero = make_double2(0, 0), one = make_double2(1, 0);
-    if (FIN == FIN_BNORM) {
-        S.bnorm2 = n;
-        S.outer_done = S.outer_done || (n == 0.0);
-    } else if (FIN == FIN_RESID) {
+#pragma unroll
+    for (int k = 0; k < NV; k++) nsum_end(v[k]);
+    // the lanes split the values as the distance halves: value k ends in lane k * 32 / NV
+    int off = 16;
+#pragma unroll
+    for (int n = NV; n > 1; n >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < n / 2; i++) {
+            const T keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
+            v[i] = nadd(keep, nshfl_xor(send, off));
+        }
+    }
+#pragma unroll
+    for (; off > 0; off >>= 1) v[0] = nadd(v[0], nshfl_xor(v[0], off));
+    if ((lane & (32 / NV - 1)) == 0) sh[warp][lane / (32 / NV)] = v[0];
+    __syncthreads();
+    if (warp != 0) return;
+    T q;
+    nset(q, 0.0);
+    if (lane < NV) {
+        const T p0 = nadd(sh[0][lane], sh[1][lane]), p1 = nadd(sh[2][lane], sh[3][lane]), p2 = nadd(sh[4][lane], sh[5][lane]),
+                p3 = nadd(sh[6][lane], sh[7][lane]);
+        q = nadd(nadd(p0, p1), nadd(p2, p3));
+    }
+#pragma unroll
+    for (int k = 0; k < NV; k++) v[k] = nshfl(q, k);
+    if (lane != 0) return;
+    T zero, one;
+    nset(zero, 0.0);
+    nset(one, 1.0);
+    const Cnum<T> c0 = {zero, zero}, c1 = {one, zero};
+    if constexpr (FIN == FIN_BNORM) {
+        S.bnorm2 = v[0];
+        S.outer_done = S.outer_done || (v[0] == 0.0);
+    } else if constexpr (FIN == FIN_RESID) {
+        const double n = v[0];
         if (S.outer_done) {  // converged earlier: its residual was not recomputed
             S.sigma = 0;
             S.scale = 0;
@@ -781,74 +805,61 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
             d = fmax(d, S.floor_delta);
             S.delta = fmin(d, 0.1);
         }
-    } else if (FIN == FIN_INIT) {
-        S.rr = n;
-        S.rho = make_double2(n, 0);
-        S.target2 = S.delta * S.delta * n;
+    } else if constexpr (FIN == FIN_INIT) {
+        T d2;
+        nset(d2, S.delta * S.delta);
+        scalar<T>(S.rho) = {v[0], zero};
+        reinterpret_cast<T &>(S.target2) = nmul(d2, v[0]);
         S.iters = 0;
-        bool act = (S.sigma > 0) && (n > 0);
+        const bool act = (S.sigma > 0) && npositive(v[0]);
         S.active = act ? 1 : 0;
         S.status = act ? 0 : 4;
-        S.alpha = act ? one : zero;
-        S.omega = act ? one : zero;
-        S.beta = zero;
-        if (act) atomicAdd(&a.ctl->n_active, 1);
-    } else if (FIN == FIN_ALPHA) {
-        if (S.active == 1) {
-            const double2 c = make_double2(v[0], v[NV - 1]);
-            if (!(c.x * c.x + c.y * c.y > 0) || !isfinite(c.x) || !isfinite(c.y)) {
+        scalar<T>(S.alpha) = act ? c1 : c0;
+        scalar<T>(S.omega) = act ? c1 : c0;
+        scalar<T>(S.beta) = c0;
+    } else if constexpr (FIN == FIN_ALPHA) {
+        if (active == 1) {
+            if (bicg_alpha(rho, Cnum<T>{v[0], v[1]}, alpha)) {
+                scalar<T>(S.alpha) = alpha;
+            } else {
                 S.active = 0;
                 S.status = 2;
-                S.alpha = zero;
-                S.omega = zero;
-                S.beta = zero;
-            } else {
-                S.alpha = cdiv(S.rho, c);
+                scalar<T>(S.alpha) = c0;
+                scalar<T>(S.omega) = c0;
+                scalar<T>(S.beta) = c0;
             }
         } else {
             S.active = 0;  // its last update has been made
         }
-    } else if (FIN == FIN_OMEGA) {
-        if (S.active == 1) {
-            const double2 ts = make_double2(v[0], v[1 % NV]), hs = make_double2(v[2 % NV], v[3 % NV]),
-                          ht = make_double2(v[4 % NV], v[5 % NV]);
-            const double tt = v[6 % NV], ss = v[7 % NV];
-            S.omega = (tt > 0) ? cdiv(ts, make_double2(tt, 0)) : zero;
-            const double2 wh = cmuld(S.omega, ht);
-            const double2 c = make_double2(hs.x - wh.x, hs.y - wh.y);
-            const double rr = (tt > 0) ? ss - (ts.x * ts.x + ts.y * ts.y) / tt : ss;
-            const bool w0 = (S.omega.x == 0.0 && S.omega.y == 0.0);
-            S.iters++;
+    } else if constexpr (FIN == FIN_OMEGA) {
+        int going = 0;
+        if (active == 1) {
+            Cnum<T> omega, rc;
+            int status = bicg_omega(v, reinterpret_cast<T &>(S.target2), omega, rc);
+            const int iters = S.iters + 1;
+            S.iters = iters;
             S.total_iters++;
-            S.rr = fmax(rr, 0.0);
-            if (rr <= S.target2) {
+            if (!status && iters >= S.maxit) status = 3;
+            scalar<T>(S.omega) = omega;
+            if (status) {
                 S.active = 2;
-                S.status = 1;
-            } else if (!(c.x * c.x + c.y * c.y > 0) || w0 || !isfinite(rr)) {
-                S.active = 2;
-                S.status = 2;
-            } else if (S.iters >= S.maxit) {
-                S.active = 2;
-                S.status = 3;
-            }
-            if (S.active == 2) {
-                S.beta = zero;
+                S.status = status;
+                scalar<T>(S.beta) = c0;
             } else {
-                S.beta = cmuld(cdiv(c, S.rho), cdiv(S.alpha, S.omega));
-                S.rho = c;
-                atomicAdd(&a.ctl->n_active, 1);
+                scalar<T>(S.beta) = bicg_beta(rc, rho, alpha, omega);
+                scalar<T>(S.rho) = rc;
+                going = 1;
             }
         }
         if (a.loop_mode) {
-            // the last solve's block decides whether the loop goes on (every block's
-            // n_active increment is ordered before its arrival by the fence)
-            __threadfence();
-            if (atomicAdd(&a.ctl->done_blocks, 1) == a.nsolve - 1) {
-                __threadfence();
-                LoopCtl *c = a.ctl;
-                const int cont = (atomicAdd(&c->n_active, 0) > 0) && (++c->iter < c->maxit);
-                c->n_active = 0;
-                c->done_blocks = 0;
+            // the block that decides the last solve also decides whether the loop goes on: one
+            // atomic carries both counts, so no fence is needed
+            LoopCtl *c = a.ctl;
+            const unsigned long long mine = 1ull + ((unsigned long long)going << 32);
+            const unsigned long long sum = atomicAdd(&c->arrived, mine) + mine;
+            if ((unsigned)sum == (unsigned)a.nsolve) {
+                const int cont = (sum >> 32) > 0 && (++c->iter < c->maxit);
+                c->arrived = 0;
                 if (a.loop_mode == 1)
                     cudaGraphSetConditional(a.loop, cont ? 1u : 0u);
                 else

@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <type_traits>
 
@@ -184,7 +185,8 @@ struct Engine {
         a.ctl = d_ctl;
         a.loop_mode = FIN == FIN_OMEGA ? loop_mode : 0;
         a.loop = loop_handle;
-        k_fin<FIN><<<solves, FIN_THREADS, 0, ctx->stream>>>(a);
+        using R = typename std::conditional<FIN == FIN_BNORM || FIN == FIN_RESID, double, typename P::real>::type;
+        k_fin<FIN, R><<<solves, FIN_THREADS, 0, ctx->stream>>>(a);
         launches++;
     }
 
@@ -347,8 +349,8 @@ struct Engine {
         static_assert((P::NCH * 5 + ShadowOf<P>::type::NCH) * 16 >= PFX::NCH * 16 + 4, "fixed-point field over the inner fields");
         fx_outer = fx_over(r);
         fx_inner = fx_over(re64);
-        A.d = (double *)a.take(npart * PART_MAX * sizeof(double));
-        B.d = (double *)a.take(npart * sizeof(double));  // true-residual norms only
+        A.d = a.take(npart * PART_MAX * sizeof(double));
+        B.d = a.take(npart * sizeof(double));  // true-residual norms only
         d_items = (Item *)a.take(nitems * sizeof(Item));
         d_st = (SolveState *)a.take(nsolve * sizeof(SolveState));
         d_ctl = (LoopCtl *)a.take(sizeof(LoopCtl));
@@ -380,7 +382,7 @@ struct Engine {
                                       cudaMemcpyHostToDevice, st));
         DDP_CUDA(ctx, cudaMemcpyAsync(d_st, h_st.data(), plan.nsolve * sizeof(SolveState), cudaMemcpyHostToDevice,
                                       st));
-        LoopCtl c0 = {0, 0, ctx->prm.max_inner, 0, 0};
+        LoopCtl c0 = {0, 0, ctx->prm.max_inner, 0};
         DDP_CUDA(ctx, cudaMemcpyAsync(d_ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, st));
         return DDP_OK;
     }
@@ -469,7 +471,7 @@ struct Engine {
         conv(true, ro, r_is_eta ? bo : ro64, 1, CL);                                  // ro = T_oo^-1 r'_o
         hop<P, EPI_RHS, DOT_NORM, CL>(hop_args(0, ro, r, s, none, none, A));         // r = T_ee^-1 (r'_e + k H_eo ro)
         blas<P, OP_INIT>(A, 0);
-        DDP_CUDA(ctx, cudaMemsetAsync(d_ctl, 0, 2 * sizeof(int), ctx->stream));
+        DDP_CUDA(ctx, cudaMemsetAsync(d_ctl, 0, offsetof(LoopCtl, maxit), ctx->stream));
         fin<FIN_INIT>();
         DDP_CUDA(ctx, cudaGetLastError());
         int rc = run_inner();
@@ -685,7 +687,7 @@ int time_hop_impl(ddp_ctx *ctx, const Job &job, int prec, int kernel, int iters,
     FieldView fx = {nullptr, nullptr, 0};
     if (P::IS64) fx = carve_field<PFX>(a, NF);
     Partials A;
-    A.d = (double *)a.take(plan.npart * PART_MAX * sizeof(double));
+    A.d = a.take(plan.npart * PART_MAX * sizeof(double));
     Item *d_items = (Item *)a.take(sizeof(Item));
     cudaStream_t st = ctx->stream;
     DDP_CUDA(ctx, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(Item), cudaMemcpyHostToDevice, st));

@@ -14,10 +14,7 @@
 // all take the same decisions.
 //
 // Arithmetic is FP32 on FP32 vectors for every storage format (links as stored); sums over sites
-// are FP32 within a warp, as in the per-step kernels.  Beyond, and in the scalar recurrences, they
-// are double-FP32 (48 bits) where the per-step kernels use FP64: they add at most 64 values that
-// are good to 24 bits, their results are rounded to FP32 when used, and a chain of 20 FP64
-// operations costs 1.8 us here, twice per iteration.
+// are FP32 within a warp, double-FP32 beyond, as in the per-step kernels (recur.cuh).
 //
 // What bounds it is latency: a block's 8 warps spend about 5000 cycles on an application of the
 // hopping term (2700 of them shared-memory wavefronts), 1000 on a barrier.  Propagators of 12
@@ -32,7 +29,6 @@
 // solved with it.
 #pragma once
 
-#include "ddfloat.cuh"
 #include "ddp_kernels.cuh"
 
 namespace ddp {
@@ -87,26 +83,6 @@ __device__ __forceinline__ unsigned cluster_addr(unsigned a, unsigned rank) {
     unsigned r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
-}
-
-// a / b to about 2^-45: the FP32 quotient and that of the remainder.
-__device__ __forceinline__ dd dd_div(dd a, dd b) {
-    const float q = a.hi / b.hi;
-    const dd r = dd_sub(a, dd_mul(dd(q, 0.f), b));
-    return dd_renorm(q, r.hi / b.hi);
-}
-__device__ __forceinline__ Cdd cdd_div(Cdd a, Cdd b) {
-    // b scaled by a power of two, so that its square stays in range
-    const int e = 127 - (int)((__float_as_uint(fmaxf(fabsf(b.re.hi), fabsf(b.im.hi))) >> 23) & 0xFF);
-    const float f = __int_as_float((127 + max(-126, min(126, e))) << 23);
-    b = {dd_scale2(b.re, f), dd_scale2(b.im, f)};
-    const dd n = dd_add(dd_mul(b.re, b.re), dd_mul(b.im, b.im));
-    const Cdd c = cmulc(a, Cdd{b.re, dd_neg(b.im)});
-    return {dd_scale2(dd_div(c.re, n), f), dd_scale2(dd_div(c.im, n), f)};
-}
-__device__ __forceinline__ bool dd_finite(dd a) { return isfinite(a.hi); }
-__device__ __forceinline__ dd dd_shfl(dd a, int lane) {
-    return dd(__shfl_sync(0xffffffffu, a.hi, lane), __shfl_sync(0xffffffffu, a.lo, lane));
 }
 
 // Site values of a vector in shared memory.
@@ -217,7 +193,7 @@ __device__ __forceinline__ dd small_sums(SmallShared &sh, float v[NV], int csize
             if (csize > 2 * n)
 #pragma unroll
                 for (int r = 0; r < n; r++) d[r] = dd_add(d[r], d[r + n]);
-        s = dd_add(d[0], dd(__shfl_xor_sync(0xffffffffu, d[0].hi, 16), __shfl_xor_sync(0xffffffffu, d[0].lo, 16)));
+        s = dd_add(d[0], nshfl_xor(d[0], 16));
     }
     return s;
 }
@@ -340,21 +316,20 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
     int buf = 0;
     // the scalars live in lane c of warp 0
     const dd zero(0.f, 0.f);
-    Cdd rho = {zero, zero}, alpha = rho, omega = rho;
-    dd rr = zero, target2 = zero;
+    Cnum<dd> rho = {zero, zero}, alpha = rho, omega = rho;
+    dd target2 = zero;
     int iters = 0, maxit = 0, status = 4, running = 0;
     {
         const dd q = small_sums<1>(sh, sums, csize, rank, buf);
         buf ^= 1;
         if (threadIdx.x < 32) {
             const int c = threadIdx.x & (SMALL_COLS - 1);
-            const dd n = dd_shfl(q, c);
+            const dd n = nshfl(q, c);
             if (threadIdx.x < SMALL_COLS) {
                 const bool hc = col0 + c < it.ncol;
                 const SolveState *Sc = a.st + it.solve0 + (hc ? col0 + c : 0);
                 running = hc && Sc->sigma > 0 && n.hi > 0.f;
                 rho = {n, zero};
-                rr = n;
                 target2 = dd_mul(dd_of(Sc->delta * Sc->delta), n);
                 maxit = Sc->maxit;
                 status = running ? 0 : 4;
@@ -385,13 +360,13 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
             buf ^= 1;
             if (threadIdx.x < 32) {
                 const int c = threadIdx.x & (SMALL_COLS - 1);
-                const Cdd hv = {dd_shfl(q, 2 * c), dd_shfl(q, 2 * c + 1)};
+                const Cnum<dd> hv = {nshfl(q, 2 * c), nshfl(q, 2 * c + 1)};
                 if (threadIdx.x < SMALL_COLS) {
-                    if (running && ((hv.re.hi == 0.f && hv.im.hi == 0.f) || !dd_finite(hv.re) || !dd_finite(hv.im))) {
+                    if (!running || !bicg_alpha(rho, hv, alpha)) {
+                        alpha = {zero, zero};
+                        if (running) status = 2;
                         running = 0;
-                        status = 2;
                     }
-                    alpha = running ? cdd_div(rho, hv) : Cdd{zero, zero};
                     sh.alpha[c] = f2(alpha.re.hi, alpha.im.hi);
                     sh.upd[c] = running;
                 }
@@ -436,32 +411,16 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
                 const int c = threadIdx.x & (SMALL_COLS - 1);
                 dd w[PART_MAX];
 #pragma unroll
-                for (int k = 0; k < PART_MAX; k++) w[k] = dd_shfl(q, c * PART_MAX + k);
+                for (int k = 0; k < PART_MAX; k++) w[k] = nshfl(q, c * PART_MAX + k);
                 if (threadIdx.x < SMALL_COLS && running) {
-                    // as k_fin<FIN_OMEGA>
-                    const Cdd ts = {w[0], w[1]}, hs = {w[2], w[3]}, ht = {w[4], w[5]};
-                    const dd tt = w[6], ss = w[7];
-                    omega = {zero, zero};
-                    dd r2 = ss;
-                    if (tt.hi > 0.f) {
-                        omega = {dd_div(ts.re, tt), dd_div(ts.im, tt)};
-                        r2 = dd_sub(ss, dd_add(dd_mul(ts.re, omega.re), dd_mul(ts.im, omega.im)));
-                    }
-                    const Cdd rc = csub(hs, cmulc(omega, ht));
+                    Cnum<dd> rc, beta = {zero, zero};
+                    status = bicg_omega(w, target2, omega, rc);
                     iters++;
-                    rr = r2;
-                    if (dd_sub(r2, target2).hi <= 0.f)
-                        status = 1;
-                    else if ((rc.re.hi == 0.f && rc.im.hi == 0.f) || (omega.re.hi == 0.f && omega.im.hi == 0.f) ||
-                             !dd_finite(rc.re) || !dd_finite(rc.im) || !dd_finite(r2))
-                        status = 2;
-                    else if (iters >= maxit)
-                        status = 3;
-                    Cdd beta = {zero, zero};
+                    if (!status && iters >= maxit) status = 3;
                     if (status) {
                         running = 0;
                     } else {
-                        beta = cdd_div(cmulc(rc, alpha), cmulc(rho, omega));
+                        beta = bicg_beta(rc, rho, alpha, omega);
                         rho = rc;
                     }
                     sh.omega[c] = f2(omega.re.hi, omega.im.hi);
@@ -513,7 +472,6 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
     cluster_sync(csize);  // no block leaves while another reads its vectors
     if (rank == 0 && threadIdx.x < SMALL_COLS && col0 + (int)threadIdx.x < it.ncol) {
         SolveState &W = a.st[it.solve0 + col0 + threadIdx.x];
-        W.rr = fmax(dd_to_double(rr), 0.0);
         W.iters = iters;
         W.total_iters += iters;
         W.status = status;
