@@ -21,8 +21,8 @@ struct SolveState {
     double target2;  // inner stopping threshold on |r|^2
     double bnorm2;   // |eta|^2 (FP64)
     double rr64;     // |eta - D_Gamma x|^2 of the current outer cycle (FP64)
-    double sigma;    // |r64| of the current cycle (0: nothing to do)
-    double scale;    // 2 kappa / sigma
+    double sigma;    // about |r64| of the current cycle (0: nothing to do)
+    double scale;    // 2 kappa / sigma, a power of two
     double delta;    // inner relative tolerance of the cycle
     double tol;      // requested relative tolerance
     double floor_delta;  // smallest useful inner tolerance of the storage format
@@ -123,9 +123,9 @@ struct TileCoord {
     int64_t cb;  // column base in the fields
 };
 
-__device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L) {
+__device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L, int blk) {
     TileCoord t;
-    int lb = blockIdx.x - it.blk0;
+    int lb = blk - it.blk0;
     const int cg = fdiv(lb, it.by_nt);
     t.tile = lb - cg * it.ntiles;
     int cl = threadIdx.x / HOP_TS;
@@ -135,6 +135,9 @@ __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L)
     t.valid = (t.col < it.ncol) && (t.h < it.nh) && (cl < L.CG);
     t.cb = it.fbase + (int64_t)t.col * it.nh;
     return t;
+}
+__device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L) {
+    return tile_coord(it, L, (int)blockIdx.x);
 }
 
 // Sums of NV values over the 32 sites of a tile, which are one warp of one column.  Each
@@ -167,23 +170,24 @@ __device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &t
 // Every block starts with this, so it counts: plain FP32 stencil on 48x24^3, 12 columns, 0.287 ms
 // with a copy by one thread, 0.267 from global memory, 0.264 from the
 // parameters.
-__device__ __forceinline__ void load_item(const Launch &L, Item &dst) {
+__device__ __forceinline__ void load_item(const Launch &L, Item &dst, int blk) {
     static_assert(sizeof(Item) % 16 == 0, "copied by 16 bytes");
     constexpr int N = sizeof(Item) / 16;
     if (threadIdx.x < 32) {
         if (L.nitems <= INLINE_ITEMS) {
             int i = 0;
 #pragma unroll
-            for (int k = 1; k < INLINE_ITEMS; k++) i += (k < L.nitems && L.inl[k].blk0 <= (int)blockIdx.x) ? 1 : 0;
+            for (int k = 1; k < INLINE_ITEMS; k++) i += (k < L.nitems && L.inl[k].blk0 <= blk) ? 1 : 0;
             if (threadIdx.x < N)
                 reinterpret_cast<int4 *>(&dst)[threadIdx.x] = reinterpret_cast<const int4 *>(L.inl + i)[threadIdx.x];
         } else {
-            const int4 *src = reinterpret_cast<const int4 *>(L.items + find_item(L.items, L.nitems, blockIdx.x));
+            const int4 *src = reinterpret_cast<const int4 *>(L.items + find_item(L.items, L.nitems, blk));
             if (threadIdx.x < N) reinterpret_cast<int4 *>(&dst)[threadIdx.x] = __ldg(src + threadIdx.x);
         }
     }
     __syncthreads();
 }
+__device__ __forceinline__ void load_item(const Launch &L, Item &dst) { load_item(L, dst, (int)blockIdx.x); }
 
 // ------------------------------------------------------------ hopping kernel
 
@@ -661,10 +665,33 @@ struct ConvArgs {
     int clov;       // k_to_low: apply the clover T^-1 of the site (items that have one)
 };
 
+// The conversions between FP64 fields and FP32 run on the integer pipe (GB300 converts and
+// multiplies two FP64 values per clock and SM: with 24 of each per site-column k_to_low took 119 us
+// for 1.33 M site-columns in FP16, 82 this way; k_accum, 124 us, is bound by its bytes).
+
+// v 2^m rounded to FP32; scale = 2^m.
+__device__ __forceinline__ float float_of(double v, int m, double scale) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), r = b + 0x10000000ull;
+    const int e = (int)((r >> 52) & 0x7FF) + m - 896;
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    if (e >= 1 && e <= 254) return __uint_as_float(sign | ((unsigned)e << 23) | ((unsigned)(r >> 29) & 0x7FFFFFu));
+    return (b << 1) == 0 ? __uint_as_float(sign) : (float)(scale * v);
+}
+__device__ __forceinline__ int scale_exponent(double scale) { return ((__double2hiint(scale) >> 20) & 0x7FF) - 1023; }
+// Storage reals of the compute precision from FP64, and back (exact).
+__device__ __forceinline__ void low_of(double &w, double v, int, double scale) { w = scale * v; }
+__device__ __forceinline__ void low_of(float &w, double v, int m, double scale) { w = float_of(v, m, scale); }
+__device__ __forceinline__ double high_of(double w) { return w; }
+__device__ __forceinline__ double high_of(float w) {
+    const unsigned u = __float_as_uint(w), e = (u >> 23) & 0xFF;
+    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+    return (u << 1) == 0 ? 0.0 : (double)w;
+}
+
 // lo = scale * hi  (scale = 2 kappa / sigma: the normalised defect), times T^-1
 // of the site when a.clov is set
 template <class P>
-__global__ void __launch_bounds__(512) k_to_low(const __grid_constant__ ConvArgs a) {
+__global__ void __launch_bounds__(384) k_to_low(const __grid_constant__ ConvArgs a) {
     using R = typename P::real;
     __shared__ __align__(16) Item it;
     load_item(a.L, it);
@@ -672,18 +699,24 @@ __global__ void __launch_bounds__(512) k_to_low(const __grid_constant__ ConvArgs
     if (!tc.valid) return;
     int64_t i = tc.cb + tc.h;
     const double sc = a.st[it.solve0 + tc.col].scale;
+    const int m = scale_exponent(sc);
     double v[24];
     load_spinor<PF64>(a.hi, i, v);
     R w[24];
 #pragma unroll
-    for (int j = 0; j < 24; j++) w[j] = (R)(sc * v[j]);
+    for (int j = 0; j < 24; j++) {
+        if (sc == 0.0)
+            w[j] = R(0);
+        else
+            low_of(w[j], v[j], m, sc);
+    }
     if (a.clov && it.clovinv) clover_apply<R>(it.clovinv, it.gV, site_row(it, tc.h, a.p), w);
     store_spinor<P>(a.lo, i, w);
 }
 
 // hi += sigma * lo  (FP64 accumulation of the correction)
 template <class P>
-__global__ void __launch_bounds__(512) k_accum(const __grid_constant__ ConvArgs a) {
+__global__ void __launch_bounds__(384) k_accum(const __grid_constant__ ConvArgs a) {
     using R = typename P::real;
     __shared__ __align__(16) Item it;
     load_item(a.L, it);
@@ -697,7 +730,7 @@ __global__ void __launch_bounds__(512) k_accum(const __grid_constant__ ConvArgs 
     double v[24];
     load_spinor<PF64>(a.hi, i, v);
 #pragma unroll
-    for (int j = 0; j < 24; j++) v[j] += sg * (double)w[j];
+    for (int j = 0; j < 24; j++) v[j] = fma(sg, high_of(w[j]), v[j]);
     store_spinor<PF64>(a.hi, i, v);
 }
 
@@ -799,8 +832,9 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
             S.sigma = 0;
             S.scale = 0;
         } else {
-            S.sigma = sqrt(n);
-            S.scale = 2.0 * S.kappa / S.sigma;
+            // a power of two, so that the defect is scaled by its exponent (float_of)
+            S.scale = __hiloint2double(__double2hiint(2.0 * S.kappa / sqrt(n)) & 0x7FF00000, 0);
+            S.sigma = 2.0 * S.kappa / S.scale;
             double d = 0.5 * S.tol * sqrt(S.bnorm2 / n);
             d = fmax(d, S.floor_delta);
             S.delta = fmin(d, 0.1);
@@ -1008,33 +1042,52 @@ static __global__ void __launch_bounds__(384) k_to_fx(const __grid_constant__ Fx
     fx_store_doubles(a.fx, tc.cb + tc.h, v);
 }
 
+// A block of k_hop_fx takes the group's columns in FX_SPLIT parts, FX_MINB blocks to an SM: 16
+// warps of 128 registers instead of 12 of 160 in one block (residual of 16x24^3, 12 columns, FP16
+// solve 48.5 -> 47.6 ms, eighth power 10.04 -> 9.91; 2 x 6 and 3 x 4 columns of 160 registers lose
+// to the links' staging, which every part repeats).
+constexpr int FX_SPLIT = 3, FX_MINB = 4;
+constexpr int FX_MAX_THREADS = HOP_TS * ((HOP_MAX_CG + FX_SPLIT - 1) / FX_SPLIT);
+__host__ __device__ constexpr int fx_cols(int CG) { return (CG + FX_SPLIT - 1) / FX_SPLIT; }
+
 // k_hop at FP64 accuracy: a.in is in block fixed point, the epilogue and its operands are FP64
 // (OUTFX: the plain sums are stored in block fixed point instead, for the next hop).  Blocks as
 // k_hop: the oriented links of a 32-site tile are staged once, as integers, for the columns.
 // About 4300 integer instructions per site-column, 1728 of them multiply-adds, instead of 864 on
 // the FP64 pipe at 1/32 of the rate: 2.10 -> 0.59 ms for the plain sums of 110592 sites x 12
-// columns (16x24^3, one parity).  160 registers (48 of sums, 48 of a neighbour, 24 of its
-// projection), so one block of 12 warps per SM: the multiply-add pipe is 47% busy, the rest waits
-// for neighbours (L2) and for the staging.
+// columns (16x24^3, one parity).  The sums alone are 48 registers, a neighbour 48, its projection
+// 24, so there are few warps: the multiply-add pipe is 47% busy, the rest waits for neighbours (L2)
+// and for the staging.
 template <int EPI, int DOT, bool CLOV, bool OUTFX>
-__global__ void __launch_bounds__(384, 1) k_hop_fx(const __grid_constant__ HopArgs a) {
+__global__ void __launch_bounds__(FX_MAX_THREADS, FX_MINB) k_hop_fx(const __grid_constant__ HopArgs a) {
     constexpr int TS = HOP_TS;
+    // this block's columns: cgh of the group's CG, from part * cgh
+    const int blk = blockIdx.x / FX_SPLIT, part = blockIdx.x % FX_SPLIT, cgh = fx_cols(a.L.CG);
+    if (part * cgh >= a.L.CG) return;
+    auto coord = [&](const Item &it) {
+        TileCoord t = tile_coord(it, a.L, blk);
+        const int cl = threadIdx.x / TS;
+        t.col += part * cgh;
+        t.cb += (int64_t)part * cgh * it.nh;
+        t.valid = t.h < it.nh && t.col < it.ncol && part * cgh + cl < a.L.CG;
+        return t;
+    };
     __shared__ __align__(16) Item it;
     __shared__ int s_nb[8 * TS];
     __shared__ __align__(16) int4 s_u[8 * TS * 9];
-    load_item(a.L, it);
+    load_item(a.L, it, blk);
     if (a.skip) {
-        const int cg = fdiv(blockIdx.x - it.blk0, it.by_nt);
-        const int col = cg * a.L.CG + (int)threadIdx.x;
+        const int cg = fdiv(blk - it.blk0, it.by_nt);
+        const int col = cg * a.L.CG + part * cgh + (int)threadIdx.x;
         int live = 0;
-        if ((int)threadIdx.x < a.L.CG && col < it.ncol) {
+        if ((int)threadIdx.x < cgh && part * cgh + (int)threadIdx.x < a.L.CG && col < it.ncol) {
             const SolveState &S = a.st[it.solve0 + col];
             live = !skipped(S, a.skip);
         }
         if (!__syncthreads_or(live)) return;
     }
     {
-        const int lb = blockIdx.x - it.blk0, tile = lb - fdiv(lb, it.by_nt) * it.ntiles;
+        const int lb = blk - it.blk0, tile = lb - fdiv(lb, it.by_nt) * it.ntiles;
         for (int q = threadIdx.x; q < 8 * TS; q += blockDim.x) {
             const int d = q / TS, h = tile * TS + (q - d * TS);
             int nb = -1;
@@ -1062,7 +1115,7 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(const __grid_constant__ HopAr
         }
     }
     __syncthreads();
-    TileCoord tc = tile_coord(it, a.L);
+    TileCoord tc = coord(it);
     if (a.skip && tc.valid) {
         const SolveState &S = a.st[it.solve0 + tc.col];
         if (skipped(S, a.skip)) tc.valid = false;
@@ -1121,7 +1174,10 @@ __global__ void __launch_bounds__(384, 1) k_hop_fx(const __grid_constant__ HopAr
             }
         }
     }
-    if (DOT != DOT_NONE) warp_partials<DOT != DOT_NONE ? dot_sums(DOT) : 1>(it, tc, sums, a.part);
+    if (DOT != DOT_NONE) {
+        if (part * cgh + (int)(threadIdx.x / TS) >= a.L.CG) tc.col = it.ncol;  // no column: nothing to write
+        warp_partials<DOT != DOT_NONE ? dot_sums(DOT) : 1>(it, tc, sums, a.part);
+    }
 }
 
 // User layout <-> block fixed point (the stencil powers); unpacking multiplies by s.

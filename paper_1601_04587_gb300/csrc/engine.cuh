@@ -38,7 +38,7 @@ inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const F
         c.skip = a.skip;
         k_to_fx<<<nblocks, threads, 0, ctx->stream>>>(c);
         a.in = fx;
-        k_hop_fx<EPI, DOT, CL, false><<<nblocks, threads, 0, ctx->stream>>>(a);
+        k_hop_fx<EPI, DOT, CL, false><<<nblocks * FX_SPLIT, HOP_TS * fx_cols(a.L.CG), 0, ctx->stream>>>(a);
         return 2;
     } else {
         (void)fx;

@@ -277,26 +277,27 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
     const int64_t ie = cb + (own_e ? local_lex(it, ke) >> 1 : 0), io = cb + (own_o ? local_lex(it, ko) >> 1 : 0);
     const SolveState *S = a.st + it.solve0 + (have ? col : 0);
     const float kap = (float)it.kappa, k2 = -kap * kap;
-    const double scale = have ? S->scale : 0.0;
+    const double scale = have ? S->scale : 0.0;  // a power of two, or 0: nothing to correct
+    const int m = scale_exponent(scale);
     __syncthreads();  // links and neighbours are in place
     float2 acc[12], rp[12], x[12], v[12], rh[12], t[12], s[12];
 #pragma unroll
     for (int j = 0; j < 12; j++) t[j] = rp[j] = x[j] = v[j] = rh[j] = f2(0.f, 0.f);
     // normalised defect: odd part to the neighbours, r = r'_e + kappa H_eo r'_o
-    if (own_o) {
+    if (own_o && scale != 0.0) {
         const double2 *f = reinterpret_cast<const double2 *>(a.ro.p) + io;
 #pragma unroll
         for (int j = 0; j < 12; j++) {
             const double2 c = __ldg(f + j * a.ro.stride);
-            t[j] = f2((float)(scale * c.x), (float)(scale * c.y));
+            t[j] = f2(float_of(c.x, m, scale), float_of(c.y, m, scale));
         }
     }
-    if (own_e) {
+    if (own_e && scale != 0.0) {
         const double2 *f = reinterpret_cast<const double2 *>(a.re.p) + ie;
 #pragma unroll
         for (int j = 0; j < 12; j++) {
             const double2 c = __ldg(f + j * a.re.stride);
-            rp[j] = f2((float)(scale * c.x), (float)(scale * c.y));
+            rp[j] = f2(float_of(c.x, m, scale), float_of(c.y, m, scale));
         }
     }
     small_put(sh, SV_T, cc, l, t);
@@ -451,8 +452,8 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
 #pragma unroll
         for (int j = 0; j < 12; j++) {
             double2 c = f[j * a.xe.stride];
-            c.x += sigma * (double)x[j].x;
-            c.y += sigma * (double)x[j].y;
+            c.x = fma(sigma, high_of(x[j].x), c.x);
+            c.y = fma(sigma, high_of(x[j].y), c.y);
             f[j * a.xe.stride] = c;
         }
     }
@@ -464,8 +465,8 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
         for (int j = 0; j < 12; j++) {
             const double2 o = __ldg(g + j * a.ro.stride);
             double2 c = f[j * a.xo.stride];
-            c.x += sigma * (double)fmaf(kap, acc[j].x, (float)(scale * o.x));
-            c.y += sigma * (double)fmaf(kap, acc[j].y, (float)(scale * o.y));
+            c.x = fma(sigma, high_of(fmaf(kap, acc[j].x, float_of(o.x, m, scale))), c.x);
+            c.y = fma(sigma, high_of(fmaf(kap, acc[j].y, float_of(o.y, m, scale))), c.y);
             f[j * a.xo.stride] = c;
         }
     }

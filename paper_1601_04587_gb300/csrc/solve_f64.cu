@@ -55,11 +55,11 @@ int hop_power_fx(ddp_ctx *ctx, const Job &job, int p, const double *psi, double 
         h.p = 0;
         h.in = f[cur][1];
         h.out = f[nxt][0];
-        k_hop_fx<EPI_PLAIN, DOT_NONE, false, true><<<plan.nblocks, plan.TS * plan.CG, 0, st>>>(h);
+        k_hop_fx<EPI_PLAIN, DOT_NONE, false, true><<<plan.nblocks * FX_SPLIT, HOP_TS * fx_cols(plan.CG), 0, st>>>(h);
         h.p = 1;
         h.in = f[cur][0];
         h.out = f[nxt][1];
-        k_hop_fx<EPI_PLAIN, DOT_NONE, false, true><<<plan.nblocks, plan.TS * plan.CG, 0, st>>>(h);
+        k_hop_fx<EPI_PLAIN, DOT_NONE, false, true><<<plan.nblocks * FX_SPLIT, HOP_TS * fx_cols(plan.CG), 0, st>>>(h);
         cur = nxt;
     }
     k_unpack_fx<<<nb, 256, 0, st>>>(pa, f[cur][0], f[cur][1], std::pow(job.kappa, p));
