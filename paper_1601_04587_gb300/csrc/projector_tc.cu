@@ -30,6 +30,7 @@
 // shared-memory layout the MMA descriptor describes (K-major, no swizzle: 8-row x
 // 16-byte core matrices, 128 bytes apart along K, 256 bytes apart between 8-row
 // groups), so that one copy per block stages it.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -455,6 +456,9 @@ struct GemmArgs {
     const uint8_t *Aq, *Bq;
     int a_bytes;      // bytes of one A slice block per K step: TILE_A, or fewer rows (see gram_tc)
     int MT, NT, KS, ksplit;
+    // the column tiles from NTr on are cross products (gram_tc): the first half of the reduction of A
+    // against the second half of column tile nt - NTr, in ksplit / 2 ranges
+    int NTr;
     int ncols;        // NT * TN
     double *part;     // [ksplit][MT * TM][ncols]: sum_d 2^-7d G_d of this block's K range
     int *err;         // set when a wait gave up
@@ -489,7 +493,11 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
     __shared__ uint32_t tbase;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nt = blockIdx.x, mt = blockIdx.y, z = blockIdx.z;
-    const int s0 = (int)((int64_t)a.KS * z / a.ksplit), s1 = (int)((int64_t)a.KS * (z + 1) / a.ksplit);
+    const bool cross = nt >= a.NTr;
+    const int KS = cross ? a.KS / 2 : a.KS, nz = cross ? a.ksplit / 2 : a.ksplit;
+    if (z >= nz) return;
+    const int s0 = (int)((int64_t)KS * z / nz), s1 = (int)((int64_t)KS * (z + 1) / nz);
+    const int64_t b0 = cross ? (int64_t)(nt - a.NTr) * a.KS + KS : (int64_t)nt * a.KS;  // first B block of the reduction
     const int nsteps = s1 - s0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tbase)),
@@ -516,7 +524,7 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
                      "r"((uint32_t)(S * (a.a_bytes + TILE_B)))
                      : "memory");
         bulk_copy(sa, a.Aq + (((int64_t)mt * a.KS + s0 + q) * S) * a.a_bytes, S * a.a_bytes, fb);
-        bulk_copy(sa + S * a.a_bytes, a.Bq + (((int64_t)nt * a.KS + s0 + q) * S) * TILE_B, S * TILE_B, fb);
+        bulk_copy(sa + S * a.a_bytes, a.Bq + ((b0 + s0 + q) * S) * TILE_B, S * TILE_B, fb);
     };
     {
         // ---- MMA issue (thread 0) and accumulator drain (GEMM_THREADS threads)
@@ -776,7 +784,7 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
         g.Bq = Bq;
         g.a_bytes = TILE_A;
         g.MT = MT;
-        g.NT = NT;
+        g.NT = g.NTr = NT;
         g.KS = KS;
         g.ksplit = ksplit;
         g.ncols = ncols;
@@ -804,97 +812,146 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
 // ------------------------------------------------------------ Gram blocks
 //
 // G[i][j] = sum_r conj(A_i[r]) A_j[r] over the rows r of one segment, on the same
-// emulated-FP64 product: A' rows i = [Re A_i | Im A_i], B' rows = [Re A_j | Im A_j]
-// (the real parts, columns j < m) and [Im A_j | -Re A_j] (the imaginary parts,
-// m <= c < 2m), every row and column with its own power-of-two exponent.  The m <= 128
-// rows of A' are stored as R8 = 8 ceil(m / 8) rows per block (the MMA's other rows read
-// whatever follows in shared memory and feed accumulator rows that are never used); the
-// 2m columns of B' span ceil(2m / 64) column tiles.
+// emulated-FP64 product, every column with its own power-of-two exponent.  With R_i and I_i the
+// real and imaginary parts of column i, the reduction of A' = [R | I] runs over two halves:
+//   m > 32: the real parts are A' against the columns B' = [R | I]; the imaginary parts are
+//     X_ij - X_ji with X = sum R_i I_j, which is the first half of A' against the second half of B'
+//     (cross tiles): three quarters of the products, and B' holds the same slices as A'.
+//   m <= 32: real and imaginary parts share one 64-column tile, B' rows [R | I] for j < m and
+//     [I | -R] beyond.
+// The m <= 128 rows of A' are stored as R8 = 8 ceil(m / 8) rows per block (the MMA's other rows
+// read whatever follows in shared memory and feed accumulator rows that are never used).
+//
+// The slices are cut in one pass that reads the columns once and writes 16 bytes per store.  Per
+// time slice of 24^3 sites and 120 columns: maxima 178 -> 61 us (compared as integers: FP64
+// comparisons run on the FP64 pipe), slices 650 -> 258 (were two passes with 2-byte stores), product
+// 456 -> 353 (0.25 at the tensor pipe's rate; the operands' 1.2 GB take 0.18 at the copy rate).
 
 namespace {
 
-// colmax[i] = max over the segment's rows of |Re A_i|, |Im A_i|
-__global__ void __launch_bounds__(256) k_gram_max(const double2 *A, int64_t cs, int m, int64_t r0, int64_t nrow,
-                                                  double *colmax) {
-    const int i = blockIdx.y;
-    double mx = 0;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nrow; r += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = A[(int64_t)i * cs + r0 + r];
-        mx = fmax(mx, fmax(mag(v.x), mag(v.y)));
+// top[i] = the largest high word, without its sign, of the components of column i over the
+// segment's rows
+__global__ void __launch_bounds__(256) k_gram_max(const double2 *A, int64_t cs, int64_t r0, int64_t nrow, unsigned *top) {
+    const double2 *a = A + (int64_t)blockIdx.y * cs + r0;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    unsigned mx = 0;
+    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto take = [&](const double2 &v) {
+        mx = max(mx, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+    };
+    for (; r + 3 * step < nrow; r += 4 * step) {
+        const double2 v0 = __ldg(a + r), v1 = __ldg(a + r + step), v2 = __ldg(a + r + 2 * step), v3 = __ldg(a + r + 3 * step);
+        take(v0);
+        take(v1);
+        take(v2);
+        take(v3);
     }
-    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if ((threadIdx.x & 31) == 0 && mx > 0) atomic_max_pos(colmax + i, mx);
-    (void)m;
+    for (; r < nrow; r += step) take(__ldg(a + r));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(top + blockIdx.y, mx);
+}
+
+// e with |v| < 2^e for every component of the column (0 for a column of zeros, or of values that
+// vanish at the products' accuracy), NONFINITE if one is not finite.
+__global__ void k_gram_exponents(const unsigned *top, int n, int *ex) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int e = (int)(top[i] >> 20);
+    ex[i] = e == 0x7FF ? NONFINITE : e ? e - 1022 : 0;
+}
+
+// Digit p = 6 - k of N in balanced base 128 is bits 7k .. 7k + 6 of N + sum_k 64 128^k, less 64
+// (k < 6); what lies above is digit 0.  Returned as FP32: an exact small integer.
+__device__ __forceinline__ void digits7f(long long N, float q[S]) {
+    constexpr unsigned long long BIAS = 64ull * (1 + (1ull << 7) + (1ull << 14) + (1ull << 21) + (1ull << 28) + (1ull << 35));
+    const long long M = N + (long long)BIAS;
+#pragma unroll
+    for (int k = 0; k < S - 1; k++)
+        q[S - 1 - k] = __int_as_float(0x4B400000 + ((int)(M >> (7 * k)) & 127)) - (12582912.f + 64.f);
+    q[0] = __int_as_float(0x4B400000 + (int)(M >> 42)) - 12582912.f;
+}
+__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<unsigned *>(&h);
 }
 
 struct GramSplitArgs {
     const double2 *A;
     int64_t cs, r0, nrow;  // column stride; the segment's rows
-    int m, R8, KSh, NT;
+    int m, R8, KSh, NT;    // NT column tiles of B'
+    int mixed;             // real and imaginary columns in one tile (m <= 32)
     const int *cexp;       // exponents of the columns
-    __nv_bfloat16 *Aq, *Bq;  // [2 KSh][S][R8 x KSTEP], [NT][2 KSh][S][64 x KSTEP]
+    uint8_t *Aq, *Bq;      // [2 KSh][S][R8 x KSTEP], [NT][2 KSh][S][64 x KSTEP] BF16
 };
 
-__global__ void k_gram_split_A(GramSplitArgs a) {
-    const int tile = a.R8 * KSTEP;
+// Thread per (column, 8 reduction steps): a 16-byte row of a core matrix of every slice.
+// Consecutive threads take consecutive columns, so that 8 of them write one core matrix.
+__global__ void __launch_bounds__(256) k_gram_split(GramSplitArgs a) {
+    const int RB = a.NT * TN;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)a.KSh * tile) return;
-    const int e = (int)(g % tile);
-    const int ksr = (int)(g / tile);
-    int rl, kl;
-    tile_pos(e, rl, kl);
-    const int64_t kx = (int64_t)ksr * KSTEP + kl;
-    __nv_bfloat16 re[S], im[S];
-    const int er = rl < a.m ? a.cexp[rl] : NONFINITE;
-    if (kx < a.nrow && er != NONFINITE) {
-        const double2 v = a.A[(int64_t)rl * a.cs + a.r0 + kx];
+    if (g >= 2 * (int64_t)a.KSh * RB) return;
+    const int row = (int)(g % RB);
+    const int64_t t = g / RB;
+    const int k8 = (int)(t & 1);
+    const int64_t ksr = t >> 1, kx = ksr * KSTEP + 8 * k8;
+    if (a.mixed && row >= a.m && row < 2 * a.m) return;  // written by the thread of column row - m
+    uint4 re[S], im[S];
+    const int er = row < a.m ? a.cexp[row] : NONFINITE;
+#pragma unroll
+    for (int p = 0; p < S; p++) re[p] = im[p] = make_uint4(0, 0, 0, 0);
+    if (er != NONFINITE) {
+        const double2 *src = a.A + (int64_t)row * a.cs + a.r0 + kx;
         const int k = 49 - er;
-        digits7(fixed_of(v.x, k), re);
-        digits7(fixed_of(v.y, k), im);
-    } else {
-        for (int p = 0; p < S; p++) re[p] = im[p] = __double2bfloat16(0.0);
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const double2 z = make_double2(0.0, 0.0);
+            const double2 v0 = kx + 2 * j < a.nrow ? __ldg(src + 2 * j) : z, v1 = kx + 2 * j + 1 < a.nrow ? __ldg(src + 2 * j + 1) : z;
+            float q0[S], q1[S];
+            digits7f(fixed_of(v0.x, k), q0);
+            digits7f(fixed_of(v1.x, k), q1);
+#pragma unroll
+            for (int p = 0; p < S; p++) reinterpret_cast<unsigned *>(&re[p])[j] = pack_bf16(q0[p], q1[p]);
+            digits7f(fixed_of(v0.y, k), q0);
+            digits7f(fixed_of(v1.y, k), q1);
+#pragma unroll
+            for (int p = 0; p < S; p++) reinterpret_cast<unsigned *>(&im[p])[j] = pack_bf16(q0[p], q1[p]);
+        }
     }
-    const int64_t bre = (int64_t)ksr * S, bim = (int64_t)(a.KSh + ksr) * S;
+    // byte offset of (row, k8) within a block: 8-row groups of SBO bytes, core matrices of LBO
+    auto off = [&](int r) { return (r >> 3) * SBO + k8 * LBO + (r & 7) * 16; };
+    const int64_t sre = ksr * S, sim = (a.KSh + ksr) * S;  // first slice of the K steps of either half
+    if (row < a.R8) {
+        const int64_t tile = (int64_t)a.R8 * KSTEP * 2;
+#pragma unroll
+        for (int p = 0; p < S; p++) {
+            *reinterpret_cast<uint4 *>(a.Aq + (sre + p) * tile + off(row)) = re[p];
+            *reinterpret_cast<uint4 *>(a.Aq + (sim + p) * tile + off(row)) = im[p];
+        }
+    }
+    const int64_t b = (int64_t)(row / TN) * 2 * a.KSh * S;
+    const int rb = row % TN;
+#pragma unroll
     for (int p = 0; p < S; p++) {
-        a.Aq[(bre + p) * tile + e] = re[p];
-        a.Aq[(bim + p) * tile + e] = im[p];
+        *reinterpret_cast<uint4 *>(a.Bq + (b + sre + p) * TILE_B + off(rb)) = re[p];
+        *reinterpret_cast<uint4 *>(a.Bq + (b + sim + p) * TILE_B + off(rb)) = im[p];
+    }
+    if (a.mixed && row < a.m) {  // column m + row: [I | -R]
+#pragma unroll
+        for (int p = 0; p < S; p++) {
+            uint4 n = re[p];
+            n.x ^= 0x80008000u;
+            n.y ^= 0x80008000u;
+            n.z ^= 0x80008000u;
+            n.w ^= 0x80008000u;
+            *reinterpret_cast<uint4 *>(a.Bq + (b + sre + p) * TILE_B + off(rb + a.m)) = im[p];
+            *reinterpret_cast<uint4 *>(a.Bq + (b + sim + p) * TILE_B + off(rb + a.m)) = n;
+        }
     }
 }
 
-__global__ void k_gram_split_B(GramSplitArgs a) {
-    const int tile = TN * KSTEP;
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)a.NT * a.KSh * tile) return;
-    const int e = (int)(g % tile);
-    const int64_t t = g / tile;
-    const int ksr = (int)(t % a.KSh), nt = (int)(t / a.KSh);
-    int col, kl;
-    tile_pos(e, col, kl);
-    col += nt * TN;
-    const int64_t kx = (int64_t)ksr * KSTEP + kl;
-    const int j = col < a.m ? col : col - a.m;
-    __nv_bfloat16 lo[S], hi[S];
-    const int ej = col < 2 * a.m ? a.cexp[j] : NONFINITE;
-    if (kx < a.nrow && ej != NONFINITE) {
-        const double2 v = a.A[(int64_t)j * a.cs + a.r0 + kx];
-        const int k = 49 - ej;
-        digits7(fixed_of(col < a.m ? v.x : v.y, k), lo);
-        digits7(fixed_of(col < a.m ? v.y : -v.x, k), hi);
-    } else {
-        for (int p = 0; p < S; p++) lo[p] = hi[p] = __double2bfloat16(0.0);
-    }
-    // tile block (nt, K step, slice), as k_ozaki_gemm reads it
-    const int64_t KS = 2 * (int64_t)a.KSh;
-    const int64_t blo = (nt * KS + ksr) * S, bhi = (nt * KS + a.KSh + ksr) * S;
-    for (int p = 0; p < S; p++) {
-        a.Bq[(blo + p) * tile + e] = lo[p];
-        a.Bq[(bhi + p) * tile + e] = hi[p];
-    }
-}
-
-// G[i][j] = 2^(e_i + e_j - 14) (sum of the K-range partials of the real and the
-// imaginary column), fixed order.
-__global__ void k_gram_finish(const double *part, int ksplit, int ncols, int m, const double *colmax, double2 *G) {
+// G[i][j] = 2^(e_i + e_j - 14) (sum of the K-range partials), fixed order; cross > 0: the first of
+// the cross products' columns, X_ij - X_ji the imaginary part, in ksplit / 2 ranges.
+__global__ void k_gram_finish(const double *part, int ksplit, int ncols, int m, int cross, const int *cexp, double2 *G) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= m * m) return;
     const int i = g / m, j = g % m;
@@ -902,11 +959,20 @@ __global__ void k_gram_finish(const double *part, int ksplit, int ncols, int m, 
     for (int s = 0; s < ksplit; s++) {
         const double *p = part + ((int64_t)s * TM + i) * ncols;
         re += p[j];
-        im += p[m + j];
+        if (!cross) im += p[m + j];
     }
-    const int sc = exponent_of(colmax[i]) + exponent_of(colmax[j]) - 14;
-    double2 v = make_double2(ldexp(re, sc), ldexp(im, sc));
-    if (!isfinite(colmax[i]) || !isfinite(colmax[j])) v = make_double2(NAN, NAN);
+    if (cross) {
+        double x = 0, y = 0;
+        for (int s = 0; s < ksplit / 2; s++) {
+            const double *p = part + (int64_t)s * TM * ncols + cross;
+            x += p[(int64_t)i * ncols + j];
+            y += p[(int64_t)j * ncols + i];
+        }
+        im = x - y;
+    }
+    const int sc = cexp[i] + cexp[j] - 14;
+    double2 v = make_double2(NAN, NAN);
+    if (cexp[i] != NONFINITE && cexp[j] != NONFINITE) v = make_double2(ldexp(re, sc), ldexp(im, sc));
     G[g] = v;
 }
 
@@ -921,20 +987,25 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
     if (m < 1 || m > TM) return DDP_ERR_UNSUPPORTED;
     const int R8 = 8 * ((m + 7) / 8);
     const int a_bytes = R8 * KSTEP * 2;
-    const int NT = (2 * m + TN - 1) / TN, ncols = NT * TN;
+    const bool mixed = 2 * m <= TN;
+    const int NTr = (m + TN - 1) / TN;  // column tiles of B' (mixed: the one that holds both parts)
+    const int NT = mixed ? 1 : 2 * NTr, ncols = NT * TN;
     const int64_t KSh64 = (seg + KSTEP - 1) / KSTEP;
     if (KSh64 > (1 << 28)) return DDP_ERR_UNSUPPORTED;
     const int KSh = (int)KSh64, KS = 2 * KSh;
-    const int ksplit = pick_ksplit(NT, KS);
-    const size_t bA = (size_t)S * KS * a_bytes, bB = (size_t)S * NT * KS * TILE_B;
+    // one wave of CTAs: the cross tiles take half the ranges for half the reduction
+    const int ksplit = mixed ? pick_ksplit(1, KS)
+                             : std::max({2, std::min(2 * (152 / (3 * NTr)), 2 * KSh),
+                                         2 * ((KS + 2 * MAX_STEPS_PER_BLOCK - 1) / (2 * MAX_STEPS_PER_BLOCK))});
+    const size_t bA = (size_t)S * KS * a_bytes, bB = (size_t)S * NTr * KS * TILE_B;
     const size_t bP = (size_t)ksplit * TM * ncols * sizeof(double);
     Arena &ar = ctx->aux;
     ar.reset();
-    DDP_CUDA(ctx, ar.reserve(bA + bB + bP + (size_t)m * 12 + 64 + 7 * 256));
+    DDP_CUDA(ctx, ar.reserve(bA + bB + bP + (size_t)m * 8 + 64 + 7 * 256));
     uint8_t *Aq = (uint8_t *)ar.take(bA);
     uint8_t *Bq = (uint8_t *)ar.take(bB);
     double *part = (double *)ar.take(bP);
-    double *colmax = (double *)ar.take((size_t)m * 8);
+    unsigned *top = (unsigned *)ar.take((size_t)m * 4);
     int *cexp = (int *)ar.take((size_t)m * 4);
     int *err = (int *)ar.take(64);
     const size_t gsm = (size_t)NSTAGE * STAGE;
@@ -942,10 +1013,12 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
     cudaStream_t st = ctx->stream;
     DDP_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), st));
     for (int z = 0; z < nseg; z++) {
-        DDP_CUDA(ctx, cudaMemsetAsync(colmax, 0, (size_t)m * 8, st));
+        DDP_CUDA(ctx, cudaMemsetAsync(top, 0, (size_t)m * 4, st));
         const int64_t r0 = (int64_t)z * seg;
-        k_gram_max<<<dim3((unsigned)std::min<int64_t>(64, (seg + 255) / 256), m), 256, 0, st>>>(A, cs, m, r0, seg,
-                                                                                            colmax);
+        // about 8 blocks per SM over all columns
+        const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((8 * 152 + m - 1) / m, (seg + 1023) / 1024));
+        k_gram_max<<<dim3(nb, m), 256, 0, st>>>(A, cs, r0, seg, top);
+        k_gram_exponents<<<1, TM, 0, st>>>(top, m, cexp);
         GramSplitArgs sa;
         sa.A = A;
         sa.cs = cs;
@@ -954,29 +1027,29 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
         sa.m = m;
         sa.R8 = R8;
         sa.KSh = KSh;
-        sa.NT = NT;
-        k_exponents<<<(m + 255) / 256, 256, 0, st>>>(colmax, m, cexp);
+        sa.NT = NTr;
+        sa.mixed = mixed ? 1 : 0;
         sa.cexp = cexp;
-        sa.Aq = (__nv_bfloat16 *)Aq;
-        sa.Bq = (__nv_bfloat16 *)Bq;
-        const int64_t na = (int64_t)KSh * R8 * KSTEP, nb = (int64_t)NT * KSh * TN * KSTEP;
-        k_gram_split_A<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(sa);
-        k_gram_split_B<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(sa);
+        sa.Aq = Aq;
+        sa.Bq = Bq;
+        const int64_t ns = 2 * (int64_t)KSh * NTr * TN;
+        k_gram_split<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(sa);
         GemmArgs g;
         g.Aq = Aq;
         g.Bq = Bq;
         g.a_bytes = a_bytes;
         g.MT = 1;
         g.NT = NT;
+        g.NTr = mixed ? NT : NTr;
         g.KS = KS;
         g.ksplit = ksplit;
         g.ncols = ncols;
         g.part = part;
         g.err = err;
         k_ozaki_gemm<<<dim3(NT, 1, ksplit), GEMM_BLOCK, gsm, st>>>(g);
-        k_gram_finish<<<(unsigned)((m * m + 255) / 256), 256, 0, st>>>(part, ksplit, ncols, m, colmax,
+        k_gram_finish<<<(unsigned)((m * m + 127) / 128), 128, 0, st>>>(part, ksplit, ncols, m, mixed ? 0 : NTr * TN, cexp,
                                                                        out + (int64_t)z * m * m);
-        ctx->launches += 6;
+        ctx->launches += 5;
         DDP_CUDA(ctx, cudaGetLastError());
     }
     int h = 0;
