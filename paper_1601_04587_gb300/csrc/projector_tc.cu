@@ -131,18 +131,6 @@ __device__ __forceinline__ void pair_of(int r, int m, int &i, int &j) {
     j = i + r;
 }
 
-// spinor component of the source field in the requested form: 0 s = A,
-// 1 s = g5 conj(A), 2 s = -A (g5 = diag(-1, -1, 1, 1) in the chiral basis)
-__device__ __forceinline__ double2 form_of(double2 v, int form, int spin) {
-    if (form == 1) {
-        v.y = -v.y;
-        if (spin < 2) v = make_double2(-v.x, -v.y);
-    } else if (form == 2) {
-        v = make_double2(-v.x, -v.y);
-    }
-    return v;
-}
-
 // ------------------------------------------------------------- pre-passes
 //
 // GB300 runs FP64 arithmetic at a small fraction of its FP32 rate, so the pre-passes
@@ -150,11 +138,15 @@ __device__ __forceinline__ double2 form_of(double2 v, int form, int spin) {
 // sum hi + lo of two floats, 48 significant bits; Dekker's product with fused
 // multiply-adds and Knuth's two-sum), and the 7-bit slices are cut from the integer
 // round(v 2^(49-e)) obtained from the bit pattern of v by shifts.
+//
+// The diquarks are bound by the FP32 pipe (24 complex products of 24 operations on lane pairs for
+// every row and site), the other pre-passes by their stores: a thread cuts 8 steps of the reduction
+// and writes 16 bytes per slice.  Per time slice of 24^3 sites and 24 columns: maxima 37 -> 20 us
+// (were compared in FP64), diquarks 243 -> 196 (were one lane per instruction), slices of the
+// diquarks 162 -> 129 and of the spinors 93 -> 51 (were 2 bytes per store, every spinor cut twice).
 
 // Magnitude used for the shared exponents: +inf for a non-finite value, so that a NaN or
 // an infinity in the input turns the affected outputs into NaN (see k_ozaki_finish).
-__device__ __forceinline__ double mag(double v) { return isfinite(v) ? fabs(v) : (double)INFINITY; }
-
 __device__ __forceinline__ float magf(float v) { return isfinite(v) ? fabsf(v) : INFINITY; }
 
 // 2^k as a float, -126 <= k <= 127.
@@ -183,70 +175,61 @@ __device__ __forceinline__ float2 df_scaled(double v, int f) {
     return make_float2(hi, lo);
 }
 
-// (S, E) += sg * a * b for double-float a, b; (S, E) is an unnormalized sum.
-__device__ __forceinline__ void df_mac(float &S, float &E, float2 a, float2 b, float sg) {
-    const float ah = sg * a.x, al = sg * a.y;
-    const float p = __fmul_rn(ah, b.x);
-    float e = __fmaf_rn(ah, b.x, -p);
-    e = __fmaf_rn(ah, b.y, e);
-    e = __fmaf_rn(al, b.x, e);
-    const float s = __fadd_rn(S, p);
-    const float bb = __fsub_rn(s, S);
-    const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    E = __fadd_rn(E, __fadd_rn(err, e));
-    S = s;
+// (s, e) += a * b lane by lane for double-floats a = ah + al, b = bh + bl; (s, e) is an unnormalized
+// sum (Knuth's two-sum; the rounding errors are collected in e).
+__device__ __forceinline__ void df2_mac(float2 &s, float2 &e, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 neg = make_float2(-1.f, -1.f);  // x - y = fma(y, -1, x)
+    const float2 p = __fmul2_rn(ah, bh);
+    float2 d = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
+    d = __ffma2_rn(ah, bl, d);
+    d = __ffma2_rn(al, bh, d);
+    const float2 t = __fadd2_rn(s, p);
+    const float2 bb = __ffma2_rn(s, neg, t);
+    const float2 u = __ffma2_rn(__ffma2_rn(bb, neg, t), neg, s), w = __ffma2_rn(bb, neg, p);
+    e = __fadd2_rn(e, __fadd2_rn(__fadd2_rn(u, w), d));
+    s = t;
 }
 
-__device__ __forceinline__ float2 df_norm(float S, float E) {
-    const float h = __fadd_rn(S, E);
-    return make_float2(h, __fsub_rn(E, __fsub_rn(h, S)));
+// hi + lo = (s0 + e0) + sg (s1 + e1) of two such sums.
+__device__ __forceinline__ float2 df_join(float s0, float e0, float s1, float e1, float sg) {
+    s1 *= sg;
+    const float s = __fadd_rn(s0, s1), bb = __fsub_rn(s, s0);
+    const float err = __fadd_rn(__fsub_rn(s0, __fsub_rn(s, bb)), __fsub_rn(s1, bb));
+    const float e = __fadd_rn(err, __fmaf_rn(sg, e1, e0)), h = __fadd_rn(s, e);
+    return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
 }
 
-// (S_re, E_re, S_im, E_im) += sg * a * b for double-float complex a, b (float4: re h, re l,
-// im h, im l).
-__device__ __forceinline__ void dfc_mac(float acc[4], float4 a, float4 b, float sg) {
-    const float2 ar = make_float2(a.x, a.y), ai = make_float2(a.z, a.w);
-    const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w);
-    df_mac(acc[0], acc[1], ar, br, sg);
-    df_mac(acc[0], acc[1], ai, bi, -sg);
-    df_mac(acc[2], acc[3], ar, bi, sg);
-    df_mac(acc[2], acc[3], ai, br, sg);
+// Column maxima of the spinors over one time slice: colmax[q], q = (k, alpha), the power of two
+// (with the leading bits) of the largest |Re|, |Im| of s_k(x)_{alpha c} over x and c; infinite for a
+// value that is not finite.  Compared as the integers of their high words: FP64 comparisons run on
+// the FP64 pipe.
+__device__ __forceinline__ unsigned mag_hi(double v) {
+    const unsigned h = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
+    return max(min(h, 0x7FF00000u), (unsigned)(__double2loint(v) != 0));  // bounds a subnormal too
 }
-
-// Column maxima of the spinors over one time slice: colmax[q], q = (k, alpha), the
-// largest |Re|, |Im| of s_k(x)_{alpha c} over x and c.
 __global__ void __launch_bounds__(256) k_colour_max(const double2 *A, int64_t n, int64_t site0, int64_t slice_n,
                                                     int m, double *colmax) {
-    __shared__ double bm[4 * MMAX];
-    const int Q = 4 * m, per = blockDim.x / Q;
+    __shared__ unsigned bm[4 * MMAX];
+    const int Q = 4 * m;
     for (int q = threadIdx.x; q < Q; q += blockDim.x) bm[q] = 0;
     __syncthreads();
-    if (per == 0) {
-        // more columns than threads: each thread takes columns q, q + blockDim.x, ...
-        // over the block's share of the sites
-        for (int q = threadIdx.x; q < Q; q += blockDim.x) {
-            const int k = q / 4, al = q % 4;
-            double mx = 0;
-            for (int64_t x = blockIdx.x; x < slice_n; x += gridDim.x)
-                for (int c = 0; c < 3; c++) {
-                    const double2 v = A[((int64_t)k * n + site0 + x) * 12 + 3 * al + c];
-                    mx = fmax(mx, fmax(mag(v.x), mag(v.y)));
-                }
-            bm[q] = mx;
-        }
-    } else if ((int)threadIdx.x < per * Q) {
-        const int q = threadIdx.x % Q, k = q / 4, al = q % 4;
-        double mx = 0;
-        for (int64_t x = blockIdx.x * (int64_t)per + threadIdx.x / Q; x < slice_n; x += (int64_t)gridDim.x * per)
-            for (int c = 0; c < 3; c++) {
-                const double2 v = A[((int64_t)k * n + site0 + x) * 12 + 3 * al + c];
-                mx = fmax(mx, fmax(mag(v.x), mag(v.y)));
+    // consecutive threads: the spins of a site, then the next columns; groups of threads share the sites
+    const int per = max(1, (int)blockDim.x / Q);
+    if ((int)threadIdx.x < per * Q || per * Q > (int)blockDim.x)
+        for (int q = threadIdx.x % (per * Q); q < per * Q; q += blockDim.x) {
+            const int c4 = q % Q, k = c4 / 4, al = c4 % 4;
+            unsigned mx = 0;
+            for (int64_t x = blockIdx.x * (int64_t)per + q / Q; x < slice_n; x += (int64_t)gridDim.x * per) {
+                const double2 *v = A + ((int64_t)k * n + site0 + x) * 12 + 3 * al;
+                const double2 v0 = __ldg(v), v1 = __ldg(v + 1), v2 = __ldg(v + 2);
+                mx = max(mx, max(max(mag_hi(v0.x), mag_hi(v0.y)), max(mag_hi(v1.x), mag_hi(v1.y))));
+                mx = max(mx, max(mag_hi(v2.x), mag_hi(v2.y)));
             }
-        if (mx > 0) atomic_max_pos(bm + q, mx);
-    }
+            if (mx) atomicMax(bm + c4, mx);
+        }
     __syncthreads();
     for (int q = threadIdx.x; q < Q; q += blockDim.x)
-        if (bm[q] > 0) atomic_max_pos(colmax + q, bm[q]);
+        if (bm[q]) atomicMax(reinterpret_cast<unsigned *>(colmax + q) + 1, bm[q]);  // the high word
 }
 
 // f_k: |s_k(x)| < 2^f_k over the slice (the exponent of the spinor column k).
@@ -289,7 +272,7 @@ __global__ void __launch_bounds__(256) k_colour_E(EArgs a) {
             re = make_float2(-re.x, -re.y);
             im = make_float2(-im.x, -im.y);
         }
-        sh[k * KSTR + c * ESITES + xs] = make_float4(re.x, re.y, im.x, im.y);
+        sh[k * KSTR + c * ESITES + xs] = make_float4(re.x, im.x, re.y, im.y);
     }
     __syncthreads();
     const int nit = a.rows * ESITES;
@@ -306,16 +289,23 @@ __global__ void __launch_bounds__(256) k_colour_E(EArgs a) {
                 const int ca = (c + 1) % 3, cb = (c + 2) % 3;
                 // f(a, b) = s_i(1,a) s_j(0,b) - s_i(0,a) s_j(1,b) + s_i(3,a) s_j(2,b) - s_i(2,a) s_j(3,b);
                 // E^c = i [f(ca, cb) - f(cb, ca)]
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                // P = sum of Re s_i times (Re, Im) s_j, M = of Im s_i: E = i [(P.x - M.y) + i (P.y + M.x)]
+                float2 P = make_float2(0.f, 0.f), Pe = P, M = P, Me = P;
+                auto mac = [&](float4 x, float4 y, float sg) {  // Re hi, Im hi, Re lo, Im lo
+                    const float2 yh = make_float2(y.x, y.y), yl = make_float2(y.z, y.w);
+                    df2_mac(P, Pe, make_float2(sg * x.x, sg * x.x), make_float2(sg * x.z, sg * x.z), yh, yl);
+                    df2_mac(M, Me, make_float2(sg * x.y, sg * x.y), make_float2(sg * x.w, sg * x.w), yh, yl);
+                };
+#pragma unroll
                 for (int t = 0; t < 2; t++) {
                     const float sg = t ? -1.f : 1.f;
                     const int p = t ? cb : ca, q = t ? ca : cb;
-                    dfc_mac(acc, si[(3 + p) * ESITES], sj[q * ESITES], sg);
-                    dfc_mac(acc, si[p * ESITES], sj[(3 + q) * ESITES], -sg);
-                    dfc_mac(acc, si[(9 + p) * ESITES], sj[(6 + q) * ESITES], sg);
-                    dfc_mac(acc, si[(6 + p) * ESITES], sj[(9 + q) * ESITES], -sg);
+                    mac(si[(3 + p) * ESITES], sj[q * ESITES], sg);
+                    mac(si[p * ESITES], sj[(3 + q) * ESITES], -sg);
+                    mac(si[(9 + p) * ESITES], sj[(6 + q) * ESITES], sg);
+                    mac(si[(6 + p) * ESITES], sj[(9 + q) * ESITES], -sg);
                 }
-                const float2 R = df_norm(acc[0], acc[1]), I = df_norm(acc[2], acc[3]);
+                const float2 R = df_join(P.x, Pe.x, M.y, Me.y, -1.f), I = df_join(P.y, Pe.y, M.x, Me.x, 1.f);
                 o[c] = make_float4(-I.x, -I.y, R.x, R.y);  // times i
                 mx = fmaxf(mx, fmaxf(magf(R.x), magf(I.x)));
             }
@@ -353,24 +343,43 @@ __device__ __forceinline__ long long fixed_of(float f, int k) {
     return fixed_round(mant, (ev ? ev : 1) - 150 + k, b >> 31);
 }
 
-// The S balanced base-128 digits of N (|N| <= 2^49 + 1): N = sum_p q_p 128^(S-1-p),
-// q_p in [-64, 63] for p > 0 and |q_0| <= 128; each exact in BF16.
-__device__ __forceinline__ void digits7(long long N, __nv_bfloat16 out[S]) {
+// Digit p = 6 - k of N in balanced base 128 is bits 7k .. 7k + 6 of N + sum_k 64 128^k, less 64
+// (k < 6); what lies above is digit 0.  Returned as FP32: an exact small integer.
+__device__ __forceinline__ void digits7f(long long N, float q[S]) {
+    constexpr unsigned long long BIAS = 64ull * (1 + (1ull << 7) + (1ull << 14) + (1ull << 21) + (1ull << 28) + (1ull << 35));
+    const long long M = N + (long long)BIAS;
 #pragma unroll
-    for (int p = S - 1; p > 0; p--) {
-        int d = (int)(N & 127);
-        if (d >= 64) d -= 128;
-        N = (N - d) >> 7;  // exact: N - d is a multiple of 128
-        out[p] = __int2bfloat16_rn(d);
-    }
-    out[0] = __int2bfloat16_rn((int)N);
+    for (int k = 0; k < S - 1; k++)
+        q[S - 1 - k] = __int_as_float(0x4B400000 + ((int)(M >> (7 * k)) & 127)) - (12582912.f + 64.f);
+    q[0] = __int_as_float(0x4B400000 + (int)(M >> 42)) - 12582912.f;
+}
+__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<unsigned *>(&h);
 }
 
-// (row rl, depth kl) of element e of one tile block in the MMA's shared-memory layout.
-__device__ __forceinline__ void tile_pos(int e, int &rl, int &kl) {
-    constexpr int KC8 = KSTEP / 8;  // core matrices along K
-    rl = ((e >> 3) & 7) + 8 * (e / (64 * KC8));
-    kl = (e & 7) + 8 * ((e >> 6) % KC8);
+// Byte offset of the 16-byte row (row r, depths 8 k8 .. 8 k8 + 7) in a tile block: 8-row groups of
+// SBO bytes, core matrices of LBO.
+__device__ __forceinline__ int tile_offset(int r, int k8) { return (r >> 3) * SBO + k8 * LBO + (r & 7) * 16; }
+__device__ __forceinline__ void put_slices(uint8_t *base, int tile_bytes, const uint4 v[S], bool negate = false) {
+    const unsigned x = negate ? 0x80008000u : 0u;
+#pragma unroll
+    for (int p = 0; p < S; p++)
+        *reinterpret_cast<uint4 *>(base + (int64_t)p * tile_bytes) = make_uint4(v[p].x ^ x, v[p].y ^ x, v[p].z ^ x, v[p].w ^ x);
+}
+// The digits of two consecutive values into word j of every slice.
+__device__ __forceinline__ void put_digits(uint4 v[S], int j, long long n0, long long n1) {
+    float q0[S], q1[S];
+    digits7f(n0, q0);
+    digits7f(n1, q1);
+#pragma unroll
+    for (int p = 0; p < S; p++) {
+        const unsigned w = pack_bf16(q0[p], q1[p]);
+        if (j == 0) v[p].x = w;
+        else if (j == 1) v[p].y = w;
+        else if (j == 2) v[p].z = w;
+        else v[p].w = w;
+    }
 }
 
 struct SplitArgs {
@@ -380,73 +389,82 @@ struct SplitArgs {
     int m, form, rows;
     int MT, NT, KSh;      // tiles; K steps of one half (Re / Im) of the reduction
     const int *rexp, *cexp;  // exponents of the rows of A' and of the spinor columns (k, alpha)
-    __nv_bfloat16 *Aq, *Bq;  // [MT][2 KSh][S][128 x KSTEP], [NT][2 KSh][S][64 x KSTEP]
+    uint8_t *Aq, *Bq;        // [MT][2 KSh][S][128 x KSTEP], [NT][2 KSh][S][64 x KSTEP] BF16
 };
 
-// A' = [Re E | Im E]: thread per (row, kx), writes the slices of both halves.  With
-// |v| < 2^e for the row, v = 2^(e-49) round(v 2^(49-e)) to within half a unit.
-__global__ void k_split_A(SplitArgs a) {
+// A' = [Re E | Im E]: thread per (row, 8 reduction steps), a 16-byte row of a core matrix of every
+// slice of both halves; consecutive threads take consecutive rows, 8 of which are one core matrix.
+// With |v| < 2^e for the row, v = 2^(e-49) round(v 2^(49-e)) to within half a unit.
+__global__ void __launch_bounds__(256) k_split_A(SplitArgs a) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)a.MT * a.KSh * (TM * KSTEP);
-    if (g >= total) return;
-    const int e = (int)(g % (TM * KSTEP));
-    const int64_t t = g / (TM * KSTEP);
-    const int ksr = (int)(t % a.KSh), mt = (int)(t / a.KSh);
-    int rl, kl;
-    tile_pos(e, rl, kl);
-    const int r = mt * TM + rl;
-    const int64_t kx = (int64_t)ksr * KSTEP + kl;
-    __nv_bfloat16 re[S], im[S];
+    const int rows = a.MT * TM;
+    if (g >= 2 * (int64_t)a.KSh * rows) return;
+    const int r = (int)(g % rows);
+    const int64_t t = g / rows, ksr = t >> 1, kx = ksr * KSTEP + 8 * (t & 1);
+    uint4 re[S], im[S];
+#pragma unroll
+    for (int p = 0; p < S; p++) re[p] = im[p] = make_uint4(0, 0, 0, 0);
     const int er = r < a.rows ? a.rexp[r] : NONFINITE;
-    if (kx < a.K && er != NONFINITE) {
-        const float4 v = a.E[(int64_t)r * a.K + kx];
+    if (er != NONFINITE) {
+        const float4 *src = a.E + (int64_t)r * a.K + kx;
         const int k = 49 - er;
-        digits7(fixed_of(v.x, k) + fixed_of(v.y, k), re);
-        digits7(fixed_of(v.z, k) + fixed_of(v.w, k), im);
-    } else {
-        for (int p = 0; p < S; p++) re[p] = im[p] = __double2bfloat16(0.0);
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 v0 = kx + 2 * j < a.K ? __ldg(src + 2 * j) : z, v1 = kx + 2 * j + 1 < a.K ? __ldg(src + 2 * j + 1) : z;
+            put_digits(re, j, fixed_of(v0.x, k) + fixed_of(v0.y, k), fixed_of(v1.x, k) + fixed_of(v1.y, k));
+            put_digits(im, j, fixed_of(v0.z, k) + fixed_of(v0.w, k), fixed_of(v1.z, k) + fixed_of(v1.w, k));
+        }
     }
     // tile block (mt, K step, slice): the S slices of one step lie contiguously
-    const int KS = 2 * a.KSh;
-    const int64_t bre = ((int64_t)mt * KS + ksr) * S, bim = ((int64_t)mt * KS + a.KSh + ksr) * S;
-    for (int p = 0; p < S; p++) {
-        a.Aq[(bre + p) * (TM * KSTEP) + e] = re[p];
-        a.Aq[(bim + p) * (TM * KSTEP) + e] = im[p];
-    }
+    uint8_t *o = a.Aq + ((int64_t)(r / TM) * 2 * a.KSh + ksr) * S * TILE_A + tile_offset(r % TM, (int)(t & 1));
+    put_slices(o, TILE_A, re);
+    put_slices(o + (int64_t)a.KSh * S * TILE_A, TILE_A, im);
 }
 
-// B' rows: col < 4m: [Re s | -Im s]; 4m <= col < 8m: [Im s | Re s]; beyond: zero.
-__global__ void k_split_B(SplitArgs a) {
+// B' rows: col < 4m: [Re s | -Im s]; 4m <= col < 8m: [Im s | Re s]; beyond: zero.  Thread per
+// (spinor column q, 8 reduction steps), which serves both of its rows; and per zero row.
+__global__ void __launch_bounds__(256) k_split_B(SplitArgs a) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)a.NT * a.KSh * (TN * KSTEP);
-    if (g >= total) return;
-    const int e = (int)(g % (TN * KSTEP));
-    const int64_t t = g / (TN * KSTEP);
-    const int ksr = (int)(t % a.KSh), nt = (int)(t / a.KSh);
-    int rl, kl;
-    tile_pos(e, rl, kl);
-    const int col = nt * TN + rl;
-    const int64_t kx = (int64_t)ksr * KSTEP + kl;
-    const int Q = 4 * a.m;
-    const int q = col < Q ? col : col - Q;
-    __nv_bfloat16 lo[S], hi[S];
-    const int eq = col < 2 * Q ? a.cexp[q] : NONFINITE;
-    if (kx < a.K && eq != NONFINITE) {
-        const int k = q / 4, al = q % 4;
-        const int64_t x = kx / 3;
-        const int c = (int)(kx % 3);
-        const double2 v = form_of(a.A[((int64_t)k * a.n + a.site0 + x) * 12 + 3 * al + c], a.form, al);
-        const int sc = 49 - eq;
-        digits7(fixed_of(col < Q ? v.x : v.y, sc), lo);
-        digits7(fixed_of(col < Q ? -v.y : v.x, sc), hi);
-    } else {
-        for (int p = 0; p < S; p++) lo[p] = hi[p] = __double2bfloat16(0.0);
+    const int cols = a.NT * TN, Q = 4 * a.m;
+    if (g >= 2 * (int64_t)a.KSh * (cols - Q)) return;
+    // q < Q: spinor columns; Q <= q: the zero rows 2 Q, 2 Q + 1, ...
+    const int q = (int)(g % (cols - Q));
+    const int64_t t = g / (cols - Q), ksr = t >> 1, kx = ksr * KSTEP + 8 * (t & 1);
+    uint4 re[S], im[S];
+#pragma unroll
+    for (int p = 0; p < S; p++) re[p] = im[p] = make_uint4(0, 0, 0, 0);
+    const int eq = q < Q ? a.cexp[q] : NONFINITE;
+    if (eq != NONFINITE) {
+        const int al = q % 4, k = 49 - eq;
+        const double2 *src = a.A + ((int64_t)(q / 4) * a.n + a.site0) * 12 + 3 * al;
+        auto at = [&](int64_t i) {  // reduction index i = 3 x + c
+            if (i >= a.K) return make_double2(0.0, 0.0);
+            const int64_t x = i / 3;
+            return __ldg(src + x * 12 + (i - 3 * x));
+        };
+        // the form's signs: conj and g5 (form 1), negation (form 2)
+        const bool nre = a.form == 2 || (a.form == 1 && al < 2), nim = a.form == 2 || (a.form == 1 && al >= 2);
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const double2 v0 = at(kx + 2 * j), v1 = at(kx + 2 * j + 1);
+            const long long r0 = fixed_of(v0.x, k), r1 = fixed_of(v1.x, k), i0 = fixed_of(v0.y, k), i1 = fixed_of(v1.y, k);
+            put_digits(re, j, nre ? -r0 : r0, nre ? -r1 : r1);
+            put_digits(im, j, nim ? -i0 : i0, nim ? -i1 : i1);
+        }
     }
-    const int KS = 2 * a.KSh;
-    const int64_t blo = ((int64_t)nt * KS + ksr) * S, bhi = ((int64_t)nt * KS + a.KSh + ksr) * S;
-    for (int p = 0; p < S; p++) {
-        a.Bq[(blo + p) * (TN * KSTEP) + e] = lo[p];
-        a.Bq[(bhi + p) * (TN * KSTEP) + e] = hi[p];
+    const int64_t half = (int64_t)a.KSh * S * TILE_B;
+    auto row = [&](int col) {
+        return a.Bq + ((int64_t)(col / TN) * 2 * a.KSh + ksr) * S * TILE_B + tile_offset(col % TN, (int)(t & 1));
+    };
+    if (q < Q) {
+        put_slices(row(q), TILE_B, re);
+        put_slices(row(q) + half, TILE_B, im, true);
+        put_slices(row(Q + q), TILE_B, im);
+        put_slices(row(Q + q) + half, TILE_B, re);
+    } else {
+        put_slices(row(Q + q), TILE_B, re);
+        put_slices(row(Q + q) + half, TILE_B, re);
     }
 }
 
@@ -774,9 +792,9 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
         k_exponents<<<(Q + 255) / 256, 256, 0, st>>>(colmax, Q, cexp);
         sa.rexp = rexp;
         sa.cexp = cexp;
-        sa.Aq = (__nv_bfloat16 *)Aq;
-        sa.Bq = (__nv_bfloat16 *)Bq;
-        const int64_t na = (int64_t)MT * KSh * TM * KSTEP, nb = (int64_t)NT * KSh * TN * KSTEP;
+        sa.Aq = Aq;
+        sa.Bq = Bq;
+        const int64_t na = 2 * (int64_t)KSh * MT * TM, nb = 2 * (int64_t)KSh * (NT * TN - Q);
         k_split_A<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(sa);
         k_split_B<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(sa);
         GemmArgs g;
@@ -860,21 +878,6 @@ __global__ void k_gram_exponents(const unsigned *top, int n, int *ex) {
     ex[i] = e == 0x7FF ? NONFINITE : e ? e - 1022 : 0;
 }
 
-// Digit p = 6 - k of N in balanced base 128 is bits 7k .. 7k + 6 of N + sum_k 64 128^k, less 64
-// (k < 6); what lies above is digit 0.  Returned as FP32: an exact small integer.
-__device__ __forceinline__ void digits7f(long long N, float q[S]) {
-    constexpr unsigned long long BIAS = 64ull * (1 + (1ull << 7) + (1ull << 14) + (1ull << 21) + (1ull << 28) + (1ull << 35));
-    const long long M = N + (long long)BIAS;
-#pragma unroll
-    for (int k = 0; k < S - 1; k++)
-        q[S - 1 - k] = __int_as_float(0x4B400000 + ((int)(M >> (7 * k)) & 127)) - (12582912.f + 64.f);
-    q[0] = __int_as_float(0x4B400000 + (int)(M >> 42)) - 12582912.f;
-}
-__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<unsigned *>(&h);
-}
-
 struct GramSplitArgs {
     const double2 *A;
     int64_t cs, r0, nrow;  // column stride; the segment's rows
@@ -906,46 +909,23 @@ __global__ void __launch_bounds__(256) k_gram_split(GramSplitArgs a) {
         for (int j = 0; j < 4; j++) {
             const double2 z = make_double2(0.0, 0.0);
             const double2 v0 = kx + 2 * j < a.nrow ? __ldg(src + 2 * j) : z, v1 = kx + 2 * j + 1 < a.nrow ? __ldg(src + 2 * j + 1) : z;
-            float q0[S], q1[S];
-            digits7f(fixed_of(v0.x, k), q0);
-            digits7f(fixed_of(v1.x, k), q1);
-#pragma unroll
-            for (int p = 0; p < S; p++) reinterpret_cast<unsigned *>(&re[p])[j] = pack_bf16(q0[p], q1[p]);
-            digits7f(fixed_of(v0.y, k), q0);
-            digits7f(fixed_of(v1.y, k), q1);
-#pragma unroll
-            for (int p = 0; p < S; p++) reinterpret_cast<unsigned *>(&im[p])[j] = pack_bf16(q0[p], q1[p]);
+            put_digits(re, j, fixed_of(v0.x, k), fixed_of(v1.x, k));
+            put_digits(im, j, fixed_of(v0.y, k), fixed_of(v1.y, k));
         }
     }
-    // byte offset of (row, k8) within a block: 8-row groups of SBO bytes, core matrices of LBO
-    auto off = [&](int r) { return (r >> 3) * SBO + k8 * LBO + (r & 7) * 16; };
     const int64_t sre = ksr * S, sim = (a.KSh + ksr) * S;  // first slice of the K steps of either half
     if (row < a.R8) {
-        const int64_t tile = (int64_t)a.R8 * KSTEP * 2;
-#pragma unroll
-        for (int p = 0; p < S; p++) {
-            *reinterpret_cast<uint4 *>(a.Aq + (sre + p) * tile + off(row)) = re[p];
-            *reinterpret_cast<uint4 *>(a.Aq + (sim + p) * tile + off(row)) = im[p];
-        }
+        const int tile = a.R8 * KSTEP * 2;
+        put_slices(a.Aq + sre * tile + tile_offset(row, k8), tile, re);
+        put_slices(a.Aq + sim * tile + tile_offset(row, k8), tile, im);
     }
-    const int64_t b = (int64_t)(row / TN) * 2 * a.KSh * S;
+    uint8_t *b = a.Bq + (int64_t)(row / TN) * 2 * a.KSh * S * TILE_B;
     const int rb = row % TN;
-#pragma unroll
-    for (int p = 0; p < S; p++) {
-        *reinterpret_cast<uint4 *>(a.Bq + (b + sre + p) * TILE_B + off(rb)) = re[p];
-        *reinterpret_cast<uint4 *>(a.Bq + (b + sim + p) * TILE_B + off(rb)) = im[p];
-    }
+    put_slices(b + sre * TILE_B + tile_offset(rb, k8), TILE_B, re);
+    put_slices(b + sim * TILE_B + tile_offset(rb, k8), TILE_B, im);
     if (a.mixed && row < a.m) {  // column m + row: [I | -R]
-#pragma unroll
-        for (int p = 0; p < S; p++) {
-            uint4 n = re[p];
-            n.x ^= 0x80008000u;
-            n.y ^= 0x80008000u;
-            n.z ^= 0x80008000u;
-            n.w ^= 0x80008000u;
-            *reinterpret_cast<uint4 *>(a.Bq + (b + sre + p) * TILE_B + off(rb + a.m)) = im[p];
-            *reinterpret_cast<uint4 *>(a.Bq + (b + sim + p) * TILE_B + off(rb + a.m)) = n;
-        }
+        put_slices(b + sre * TILE_B + tile_offset(rb + a.m, k8), TILE_B, im);
+        put_slices(b + sim * TILE_B + tile_offset(rb + a.m, k8), TILE_B, re, true);
     }
 }
 
