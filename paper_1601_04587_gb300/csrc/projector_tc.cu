@@ -24,12 +24,12 @@
 // slices with p + q >= S are dropped: each term of the sum is exact to about
 // 2^-47 of its row maximum times its column maximum.
 //
-// Operands reach the tensor cores through a four-stage pipeline of bulk copies
+// Operands reach the tensor cores through a five-stage pipeline of bulk copies
 // (cp.async.bulk, completion on an mbarrier): the split kernels write every
 // (slice, 128- or 64-row tile, 16-deep K step) block contiguously in the
 // shared-memory layout the MMA descriptor describes (K-major, no swizzle: 8-row x
 // 16-byte core matrices, 128 bytes apart along K, 256 bytes apart between 8-row
-// groups), so that one copy per block stages it.
+// groups), so that one copy per block stages it (seven for the columns of large Gram blocks).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -48,9 +48,10 @@ constexpr int CS = 28;        // stages per exact chunk: KC = 448
 constexpr int SBO = 16 * KSTEP, LBO = 128;  // bytes between 8-row groups; between K core matrices
 constexpr int TILE_A = TM * KSTEP * 2, TILE_B = TN * KSTEP * 2;  // bytes
 constexpr int STAGE = S * (TILE_A + TILE_B);
-constexpr int NSTAGE = 4;   // operand buffers in flight
-constexpr int GEMM_THREADS = 512;   // thread 0 streams the operands and issues the MMAs; all drain
+constexpr int NSTAGE = 5;   // operand buffers in flight
+constexpr int GEMM_THREADS = 512;   // all drain; one lane loads, one issues the MMAs
 constexpr int GEMM_BLOCK = GEMM_THREADS;
+constexpr int MMA_WARP = 0, PRODUCER_WARP = 5;  // on different quarters of the SM
 constexpr int DCOLS = TN / (GEMM_THREADS / 128);  // accumulator columns a thread drains
 constexpr int TMEM_COLS = 512;  // S * TN = 448 used
 constexpr int MAX_STEPS_PER_BLOCK = 1 << 16;  // keeps the fixed-point sums far below 2^63
@@ -88,7 +89,7 @@ __device__ __forceinline__ uint64_t globaltimer() {
 
 // Bounded wait for the completion of the mbarrier phase with the given parity.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    const uint64_t t0 = globaltimer();
+    uint64_t t0 = 0;  // read only after some tries: most waits are short
     for (uint32_t it = 0;; it++) {
         uint32_t ok;
         asm volatile("{\n .reg .pred pw;\n mbarrier.try_wait.parity.shared::cta.b64 pw, [%1], %2;\n"
@@ -97,7 +98,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
                      : "r"(bar), "r"(parity)
                      : "memory");
         if (ok) return true;
-        if ((it & 255u) == 255u && globaltimer() - t0 > WAIT_NS) return false;
+        if ((it & 255u) == 255u) {
+            const uint64_t t = globaltimer();
+            if (t0 == 0)
+                t0 = t;
+            else if (t - t0 > WAIT_NS)
+                return false;
+        }
     }
 }
 
@@ -471,7 +478,7 @@ __global__ void __launch_bounds__(256) k_split_B(SplitArgs a) {
 // -------------------------------------------------------------- the product
 
 struct GemmArgs {
-    const uint8_t *Aq, *Bq;
+    const uint8_t *Aq, *Bq;  // Bq null: the columns are the rows of A' (gram_tc)
     int a_bytes;      // bytes of one A slice block per K step: TILE_A, or fewer rows (see gram_tc)
     int MT, NT, KS, ksplit;
     // the column tiles from NTr on are cross products (gram_tc): the first half of the reduction of A
@@ -488,6 +495,14 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
                  : "memory");
 }
 
+// One lane of a converged warp, known to the compiler as such: operands of the MMA and copy
+// instructions stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
 // Barrier 1 over the GEMM_THREADS threads; returns the OR of v over them.
 __device__ __forceinline__ bool drain_barrier_or(bool v) {
     uint32_t r;
@@ -501,21 +516,25 @@ __device__ __forceinline__ bool drain_barrier_or(bool v) {
 
 // One CTA per (64-column tile, 128-row tile, K range): the column tiles of one row tile
 // are neighbours in the launch order, so that the CTAs streaming the same A blocks run at
-// the same time and share them through L2.  Thread 0 streams the operand
-// blocks of each K step into NSTAGE buffers (two bulk copies per step) and issues the
-// MMAs; after every CS steps the sixteen warps drain the seven accumulators (warp w: lanes 32 (w % 4) .. + 31, columns DCOLS (w / 4) .. + DCOLS - 1)
-// into exact 64-bit fixed point.
+// the same time and share them through L2.  One lane of PRODUCER_WARP streams the operand
+// blocks of each K step into NSTAGE buffers (two bulk copies per step), one of MMA_WARP issues
+// the MMAs; after every CS steps the sixteen warps drain the seven accumulators (warp w: lanes
+// 32 (w % 4) .. + 31, columns DCOLS (w / 4) .. + DCOLS - 1) into exact 64-bit fixed point.
+// With loads and MMAs issued by one thread in turn a step took 1550 clocks, of which 900 did not
+// depend on the MMAs (896 at the tensor rate): 282 us for 24 modes on 24^3 sites, 228 with the roles
+// split and five buffers instead of four (141 at the tensor rate; the operands' way from L2, 43 KB a step, is the next bound).
 __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ __align__(8) uint64_t full[NSTAGE], empty[NSTAGE];
     __shared__ uint32_t tbase;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nt = blockIdx.x, mt = blockIdx.y, z = blockIdx.z;
     const bool cross = nt >= a.NTr;
     const int KS = cross ? a.KS / 2 : a.KS, nz = cross ? a.ksplit / 2 : a.ksplit;
     if (z >= nz) return;
     const int s0 = (int)((int64_t)KS * z / nz), s1 = (int)((int64_t)KS * (z + 1) / nz);
-    const int64_t b0 = cross ? (int64_t)(nt - a.NTr) * a.KS + KS : (int64_t)nt * a.KS;  // first B block of the reduction
+    const int ct = cross ? nt - a.NTr : nt;                                 // column tile
+    const int64_t b0 = (a.Bq ? (int64_t)ct * a.KS : 0) + (cross ? KS : 0);  // first B block
     const int nsteps = s1 - s0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tbase)),
@@ -535,17 +554,22 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tbase;
 
-    auto load = [&](int q) {  // thread 0: K step s0 + q into buffer q % NSTAGE (two bulk copies)
+    auto load = [&](int q) {  // producer: K step s0 + q into buffer q % NSTAGE (two bulk copies)
         const int st = q % NSTAGE;
         const uint32_t sa = smem_u32(dsm + st * STAGE), fb = smem_u32(&full[st]);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
                      "r"((uint32_t)(S * (a.a_bytes + TILE_B)))
                      : "memory");
         bulk_copy(sa, a.Aq + (((int64_t)mt * a.KS + s0 + q) * S) * a.a_bytes, S * a.a_bytes, fb);
-        bulk_copy(sa + S * a.a_bytes, a.Bq + ((b0 + s0 + q) * S) * TILE_B, S * TILE_B, fb);
+        if (a.Bq) {
+            bulk_copy(sa + S * a.a_bytes, a.Bq + ((b0 + s0 + q) * S) * TILE_B, S * TILE_B, fb);
+        } else {  // 64 rows of each slice of A'
+            const uint8_t *b = a.Aq + ((b0 + s0 + q) * S) * a.a_bytes + ct * TILE_B;
+#pragma unroll
+            for (int p = 0; p < S; p++) bulk_copy(sa + S * a.a_bytes + p * TILE_B, b + p * a.a_bytes, TILE_B, fb);
+        }
     };
     {
-        // ---- MMA issue (thread 0) and accumulator drain (GEMM_THREADS threads)
         // 2^14 sum_{d<=2} 2^-7d G_d and 2^42 sum_{d>=3} 2^-7d G_d in two's complement (unsigned
         // arithmetic: exact for every accumulator row that holds a result, and defined
         // modulo 2^64 for the padding rows, whose values are discarded)
@@ -553,20 +577,23 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
 #pragma unroll
         for (int c = 0; c < DCOLS; c++) acc_hi[c] = acc_lo[c] = 0;
         bool ok = true, aborted = false;
-        // thread 0: the last step loaded, the last step whose operands arrived, the last
-        // step whose MMAs were committed
-        int loaded = -1, consumed = -1, pend_mma = -1;
-        if (tid == 0)
-            for (int q = 0; q < NSTAGE - 1 && q < nsteps; q++) {
-                load(q);
-                loaded = q;
+        int loaded = 0, issued = 0;  // steps the producer has loaded, steps whose MMAs were committed
+        for (int j0 = 0; j0 < nsteps; j0 += CS) {
+            const int je = min(j0 + CS, nsteps);
+            if (warp == PRODUCER_WARP && elect_one()) {
+                // the buffer of step q is free once the MMAs of step q - NSTAGE have read it: up to
+                // NSTAGE steps of the next chunk are under way while this one's sums are drained
+                for (; ok && loaded < min(je + NSTAGE, nsteps); loaded++) {
+                    if (loaded >= NSTAGE) ok = mbar_wait(smem_u32(&empty[loaded % NSTAGE]), (loaded / NSTAGE - 1) & 1);
+                    if (!ok) break;
+                    load(loaded);
+                }
             }
-        for (int j = 0; j < nsteps; j++) {
-            const int st = j % NSTAGE;
-            if (tid == 0 && ok) {
-                ok = mbar_wait(smem_u32(&full[st]), (j / NSTAGE) & 1);
-                if (ok) {
-                    consumed = j;
+            if (warp == MMA_WARP && elect_one()) {
+                for (int j = j0; j < je; j++) {
+                    const int st = j % NSTAGE;
+                    ok = mbar_wait(smem_u32(&full[st]), (j / NSTAGE) & 1);
+                    if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     // A slices a_bytes apart: with fewer than 128 rows stored, the MMA's
                     // remaining rows read whatever follows and only feed accumulator rows
@@ -585,7 +612,7 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
                             const uint64_t da = da0 + (uint64_t)((p * a.a_bytes) >> 4);
                             const uint64_t db = db0 + (uint64_t)((q0 * TILE_B) >> 4);
                             // the first products of a chunk (p = 0 covers every group) overwrite
-                            const uint32_t accum = (j % CS == 0 && p == 0) ? 0u : 1u;
+                            const uint32_t accum = (j == j0 && p == 0) ? 0u : 1u;
                             asm volatile("{\n .reg .pred pa;\n setp.ne.b32 pa, %4, 0;\n"
                                          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, pa;\n}\n"
                                          ::"r"(dcol), "l"(da), "l"(db), "r"(idesc_n(TN * nq)), "r"(accum)
@@ -595,22 +622,17 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                                  ::"r"(smem_u32(&empty[st]))
                                  : "memory");
-                    pend_mma = j;
-                    const int nxt = j + NSTAGE - 1;
-                    if (nxt < nsteps) {
-                        // its buffer is free once the MMAs of step j - 1 have read it
-                        if (j >= 1) ok = mbar_wait(smem_u32(&empty[(j - 1) % NSTAGE]), ((j - 1) / NSTAGE) & 1);
-                        if (ok) {
-                            load(nxt);
-                            loaded = nxt;
-                        }
-                    }
+                    issued = j + 1;
                 }
-                if (!ok) atomicExch(a.err, 1);
             }
-            if (j % CS == CS - 1 || j == nsteps - 1) {
+            if (!ok) atomicExch(a.err, 1);
+            __syncwarp();
+            loaded = __reduce_max_sync(0xffffffffu, loaded);
+            issued = __reduce_max_sync(0xffffffffu, issued);
+            {
+                const int j = je - 1, st = j % NSTAGE;
                 // every draining thread takes the same branch: the barrier returns the OR
-                if (drain_barrier_or(tid == 0 && !ok)) {
+                if (drain_barrier_or(!ok)) {
                     aborted = true;
                     break;
                 }
@@ -652,11 +674,10 @@ __global__ void __launch_bounds__(GEMM_BLOCK, 1) k_ozaki_gemm(GemmArgs a) {
                 }
             }
         }
-        if (tid == 0) {
-            // after a failed wait: give the copies and MMAs in flight a bounded time to land
-            if (pend_mma >= 0) mbar_wait(smem_u32(&empty[pend_mma % NSTAGE]), (pend_mma / NSTAGE) & 1);
-            for (int q = consumed + 1; q <= loaded; q++) mbar_wait(smem_u32(&full[q % NSTAGE]), (q / NSTAGE) & 1);
-        }
+        // after a failed wait: give the copies and MMAs in flight a bounded time to land
+        if (issued > 0) mbar_wait(smem_u32(&empty[(issued - 1) % NSTAGE]), ((issued - 1) / NSTAGE) & 1);
+        for (int q = max(0, loaded - NSTAGE); q < loaded; q++) mbar_wait(smem_u32(&full[q % NSTAGE]), (q / NSTAGE) & 1);
+        __syncwarp();
         if (!aborted) {
             const int row = mt * TM + 32 * (warp & 3) + lane;
             double *o = a.part + ((int64_t)z * a.MT * TM + row) * a.ncols + nt * TN + DCOLS * (warp >> 2);
@@ -834,7 +855,9 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
 // real and imaginary parts of column i, the reduction of A' = [R | I] runs over two halves:
 //   m > 32: the real parts are A' against the columns B' = [R | I]; the imaginary parts are
 //     X_ij - X_ji with X = sum R_i I_j, which is the first half of A' against the second half of B'
-//     (cross tiles): three quarters of the products, and B' holds the same slices as A'.
+//     (cross tiles): three quarters of the products.  B' holds the same slices as A', so only A' is
+//     stored, and a column tile is read as 64 rows of each of its slices (rows beyond R8 are those of
+//     the next slice and feed columns that are never used).
 //   m <= 32: real and imaginary parts share one 64-column tile, B' rows [R | I] for j < m and
 //     [I | -R] beyond.
 // The m <= 128 rows of A' are stored as R8 = 8 ceil(m / 8) rows per block (the MMA's other rows
@@ -842,8 +865,8 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
 //
 // The slices are cut in one pass that reads the columns once and writes 16 bytes per store.  Per
 // time slice of 24^3 sites and 120 columns: maxima 178 -> 61 us (compared as integers: FP64
-// comparisons run on the FP64 pipe), slices 650 -> 258 (were two passes with 2-byte stores), product
-// 456 -> 353 (0.25 at the tensor pipe's rate; the operands' 1.2 GB take 0.18 at the copy rate).
+// comparisons run on the FP64 pipe), slices 650 -> 224 (were two passes with 2-byte stores and both
+// operands; the bytes take 130 at the copy rate), product 456 -> 282 (188 at the tensor pipe's rate).
 
 namespace {
 
@@ -881,16 +904,16 @@ __global__ void k_gram_exponents(const unsigned *top, int n, int *ex) {
 struct GramSplitArgs {
     const double2 *A;
     int64_t cs, r0, nrow;  // column stride; the segment's rows
-    int m, R8, KSh, NT;    // NT column tiles of B'
+    int m, R8, KSh;
     int mixed;             // real and imaginary columns in one tile (m <= 32)
     const int *cexp;       // exponents of the columns
-    uint8_t *Aq, *Bq;      // [2 KSh][S][R8 x KSTEP], [NT][2 KSh][S][64 x KSTEP] BF16
+    uint8_t *Aq, *Bq;      // [2 KSh][S][R8 x KSTEP]; mixed: [2 KSh][S][64 x KSTEP]; BF16
 };
 
 // Thread per (column, 8 reduction steps): a 16-byte row of a core matrix of every slice.
 // Consecutive threads take consecutive columns, so that 8 of them write one core matrix.
 __global__ void __launch_bounds__(256) k_gram_split(GramSplitArgs a) {
-    const int RB = a.NT * TN;
+    const int RB = a.mixed ? TN : a.R8;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (g >= 2 * (int64_t)a.KSh * RB) return;
     const int row = (int)(g % RB);
@@ -919,13 +942,13 @@ __global__ void __launch_bounds__(256) k_gram_split(GramSplitArgs a) {
         put_slices(a.Aq + sre * tile + tile_offset(row, k8), tile, re);
         put_slices(a.Aq + sim * tile + tile_offset(row, k8), tile, im);
     }
-    uint8_t *b = a.Bq + (int64_t)(row / TN) * 2 * a.KSh * S * TILE_B;
-    const int rb = row % TN;
-    put_slices(b + sre * TILE_B + tile_offset(rb, k8), TILE_B, re);
-    put_slices(b + sim * TILE_B + tile_offset(rb, k8), TILE_B, im);
-    if (a.mixed && row < a.m) {  // column m + row: [I | -R]
-        put_slices(b + sre * TILE_B + tile_offset(rb + a.m, k8), TILE_B, im);
-        put_slices(b + sim * TILE_B + tile_offset(rb + a.m, k8), TILE_B, re, true);
+    if (!a.mixed) return;
+    uint8_t *bre = a.Bq + sre * TILE_B, *bim = a.Bq + sim * TILE_B;
+    put_slices(bre + tile_offset(row, k8), TILE_B, re);
+    put_slices(bim + tile_offset(row, k8), TILE_B, im);
+    if (row < a.m) {  // column m + row: [I | -R]
+        put_slices(bre + tile_offset(row + a.m, k8), TILE_B, im);
+        put_slices(bim + tile_offset(row + a.m, k8), TILE_B, re, true);
     }
 }
 
@@ -977,13 +1000,14 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
     const int ksplit = mixed ? pick_ksplit(1, KS)
                              : std::max({2, std::min(2 * (152 / (3 * NTr)), 2 * KSh),
                                          2 * ((KS + 2 * MAX_STEPS_PER_BLOCK - 1) / (2 * MAX_STEPS_PER_BLOCK))});
-    const size_t bA = (size_t)S * KS * a_bytes, bB = (size_t)S * NTr * KS * TILE_B;
+    // the last column tile of the last slice may read up to a full tile of 128 rows
+    const size_t bA = (size_t)S * KS * a_bytes + TILE_A, bB = mixed ? (size_t)S * KS * TILE_B : 0;
     const size_t bP = (size_t)ksplit * TM * ncols * sizeof(double);
     Arena &ar = ctx->aux;
     ar.reset();
     DDP_CUDA(ctx, ar.reserve(bA + bB + bP + (size_t)m * 8 + 64 + 7 * 256));
     uint8_t *Aq = (uint8_t *)ar.take(bA);
-    uint8_t *Bq = (uint8_t *)ar.take(bB);
+    uint8_t *Bq = mixed ? (uint8_t *)ar.take(bB) : nullptr;
     double *part = (double *)ar.take(bP);
     unsigned *top = (unsigned *)ar.take((size_t)m * 4);
     int *cexp = (int *)ar.take((size_t)m * 4);
@@ -1007,12 +1031,11 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
         sa.m = m;
         sa.R8 = R8;
         sa.KSh = KSh;
-        sa.NT = NTr;
         sa.mixed = mixed ? 1 : 0;
         sa.cexp = cexp;
         sa.Aq = Aq;
         sa.Bq = Bq;
-        const int64_t ns = 2 * (int64_t)KSh * NTr * TN;
+        const int64_t ns = 2 * (int64_t)KSh * (mixed ? TN : R8);
         k_gram_split<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(sa);
         GemmArgs g;
         g.Aq = Aq;
