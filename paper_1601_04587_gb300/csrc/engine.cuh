@@ -24,11 +24,27 @@
 
 namespace ddp {
 
+// Launches kernel k; chained: as a programmatic dependent of the kernel before it in the stream
+// (see chain_wait).
+template <class Args>
+inline void launch_kernel(ddp_ctx *ctx, void (*k)(Args), int nblocks, int threads, const Args &a, bool chained) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)nblocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = ctx->stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, k, a);  // an error stays pending, as with <<<>>>
+}
+
 // One application of the hopping term (CL: with the clover term of the items that have one).
 // FP64: the input is brought into block fixed point in fx (a field of its size) first.
 // Returns the number of kernels launched.
 template <class Q, int EPI, int DOT, bool CL = false>
-inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const FieldView &fx) {
+inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const FieldView &fx, bool chained = false) {
     if constexpr (Q::IS64) {
         FxArgs c;
         c.L = a.L;
@@ -43,7 +59,7 @@ inline int launch_hop(ddp_ctx *ctx, int nblocks, int threads, HopArgs a, const F
     } else {
         (void)fx;
         for (int j = 0; j < 6; j++) a.off[j] = (int64_t)j * a.in.stride * (int64_t)sizeof(typename Q::chunk);
-        k_hop<Q, EPI, DOT, CL><<<nblocks, threads, 0, ctx->stream>>>(a);
+        launch_kernel(ctx, k_hop<Q, EPI, DOT, CL>, nblocks, threads, a, chained);
         return 1;
     }
 }
@@ -128,6 +144,7 @@ struct Engine {
     cudaGraphExec_t loop_exec = nullptr;
     cudaGraph_t loop_graph = nullptr;
     long launches = 0;
+    bool chained = false;      // kernels are launched as dependents of one another (see chain_wait)
     int grid = 0, solves = 0;  // blocks and columns of the next launches: of all items, or of the large ones
     bool clov = false;  // some item of the plan has a clover term
 
@@ -154,7 +171,7 @@ struct Engine {
 
     template <class Q, int EPI, int DOT, bool CL = false>
     void hop(const HopArgs &a) {
-        launches += launch_hop<Q, EPI, DOT, CL>(ctx, grid, threads, a, EPI == EPI_RESID ? fx_outer : fx_inner);
+        launches += launch_hop<Q, EPI, DOT, CL>(ctx, grid, threads, a, EPI == EPI_RESID ? fx_outer : fx_inner, chained);
     }
 
     template <class Q, int OP>
@@ -171,7 +188,7 @@ struct Engine {
         a.t = t;
         a.st = d_st;
         a.part = part;
-        k_blas<Q, OP><<<grid, threads, 0, ctx->stream>>>(a);
+        launch_kernel(ctx, k_blas<Q, OP>, grid, threads, a, chained);
         launches++;
     }
 
@@ -186,7 +203,7 @@ struct Engine {
         a.loop_mode = FIN == FIN_OMEGA ? loop_mode : 0;
         a.loop = loop_handle;
         using R = typename std::conditional<FIN == FIN_BNORM || FIN == FIN_RESID, double, typename P::real>::type;
-        k_fin<FIN, R><<<solves, FIN_THREADS, 0, ctx->stream>>>(a);
+        launch_kernel(ctx, k_fin<FIN, R>, solves, FIN_THREADS, a, chained);
         launches++;
     }
 
@@ -233,10 +250,12 @@ struct Engine {
         blas<P, OP_XRP_UPDATE>(A);                                                      // x, r, p
     }
     void iteration_body() {
+        chained = !P::IS64;  // the FP64 stencil's kernels do not take part
         if (clov)
             iteration_body_t<true>();
         else
             iteration_body_t<false>();
+        chained = false;
     }
 
     // The inner loop of the large items as a graph (nothing to build without any).
