@@ -82,30 +82,4 @@ __device__ __forceinline__ Cdd cscale(double s, Cdd a) {
     return {dd_scale2(a.re, f), dd_scale2(a.im, f)};
 }
 
-// ------------------------------------------------------------- sums of products, two lanes at a time
-
-// (s, e) += a * b lane by lane for double-floats a = ah + al, b = bh + bl; (s, e) is an unnormalized
-// sum (Knuth's two-sum; the rounding errors are collected in e).
-__device__ __forceinline__ void df2_mac(float2 &s, float2 &e, float2 ah, float2 al, float2 bh, float2 bl) {
-    const float2 neg = make_float2(-1.f, -1.f);  // x - y = fma(y, -1, x)
-    const float2 p = __fmul2_rn(ah, bh);
-    float2 d = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
-    d = __ffma2_rn(ah, bl, d);
-    d = __ffma2_rn(al, bh, d);
-    const float2 t = __fadd2_rn(s, p);
-    const float2 bb = __ffma2_rn(s, neg, t);
-    const float2 u = __ffma2_rn(__ffma2_rn(bb, neg, t), neg, s), w = __ffma2_rn(bb, neg, p);
-    e = __fadd2_rn(e, __fadd2_rn(__fadd2_rn(u, w), d));
-    s = t;
-}
-
-// hi + lo = (s0 + e0) + sg (s1 + e1) of two such sums.
-__device__ __forceinline__ dd df_join(float s0, float e0, float s1, float e1, float sg) {
-    s1 *= sg;
-    const float s = __fadd_rn(s0, s1), bb = __fsub_rn(s, s0);
-    const float err = __fadd_rn(__fsub_rn(s0, __fsub_rn(s, bb)), __fsub_rn(s1, bb));
-    const float e = __fadd_rn(err, __fmaf_rn(sg, e1, e0)), h = __fadd_rn(s, e);
-    return dd(h, __fsub_rn(e, __fsub_rn(h, s)));
-}
-
 }  // namespace ddp

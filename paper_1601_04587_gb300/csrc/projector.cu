@@ -157,31 +157,23 @@ __global__ void k_apply_rinv(double2 *A, int64_t cs, int m, const double2 *Rinv)
     }
 }
 
-// The same update in double-FP32 arithmetic (the A entries split from their bits, R^-1 staged in
-// shared memory): GB300's FP64 rate is about 1/64 of its FP32 rate.  Up to RINV_MMAX_ALL columns
-// R^-1 is staged whole; beyond, the TJ columns of each output tile are staged in turn (the same
-// products in the same order).  Bound by the FP32 pipe: a complex product is added with 24 lane-pair
-// instructions (the two parts of A times the pair Re, Im of R^-1, unnormalized sums) where
-// normalizing every product and sum took 72 single ones: 48 columns of 8 x 16^3 sites 1300 -> 949 us
-// (584 at the FP32 rate).
+// The same update in double-FP32 arithmetic (the A entries split from their bits,
+// R^-1 staged in shared memory): GB300's FP64 rate is about 1/64 of its FP32 rate.
+// Up to RINV_MMAX_ALL columns R^-1 is staged whole; beyond, the TJ columns of each
+// output tile are staged in turn (the same products in the same order).
 constexpr int RINV_MMAX_ALL = 32, RINV_MMAX = TC_MMAX, RINV_TJ = 8;
 __global__ void __launch_bounds__(128) k_apply_rinv_dd(double2 *A, int64_t cs, int m, const double2 *Rinv) {
     constexpr int TJ = RINV_TJ;
     constexpr int SR = RINV_MMAX_ALL * RINV_MMAX_ALL > RINV_MMAX * TJ ? RINV_MMAX_ALL * RINV_MMAX_ALL : RINV_MMAX * TJ;
-    __shared__ float4 sR[SR];  // Re hi, Im hi, Re lo, Im lo; [i][stride], zero beyond column m
+    __shared__ Cdd sR[SR];
     const bool whole = m <= RINV_MMAX_ALL;
-    const int stride = whole ? (m + TJ - 1) / TJ * TJ : TJ;
-    // R^-1 [i][j0 .. j0 + stride) for i < rows
-    auto stage = [&](int rows, int j0) {
-        for (int e = threadIdx.x; e < rows * stride; e += blockDim.x) {
-            const int i = e / stride, j = j0 + e % stride;
-            const double2 c = j < m ? Rinv[(int64_t)i * m + j] : make_double2(0.0, 0.0);
-            const dd re = dd_of(c.x), im = dd_of(c.y);
-            sR[e] = make_float4(re.hi, im.hi, re.lo, im.lo);
+    if (whole) {
+        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+            const double2 c = Rinv[e];
+            sR[e] = {dd_of(c.x), dd_of(c.y)};
         }
         __syncthreads();
-    };
-    if (whole) stage(m, 0);
+    }
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     // rows beyond the field still take part in the staging barriers of the tiles
     const bool row = r < cs;
@@ -189,40 +181,32 @@ __global__ void __launch_bounds__(128) k_apply_rinv_dd(double2 *A, int64_t cs, i
     for (int j0 = ((m - 1) / TJ) * TJ; j0 >= 0; j0 -= TJ) {
         const int jmax = min(m, j0 + TJ);
         if (!whole) {
+            // R^-1 [i][j0 .. jmax) for i < jmax, at sR[i * TJ + (j - j0)]
             __syncthreads();  // the previous tile's reads are done
-            stage(jmax, j0);
+            for (int e = threadIdx.x; e < jmax * TJ; e += blockDim.x) {
+                const int i = e / TJ, j = j0 + e % TJ;
+                const double2 c = j < m ? Rinv[(int64_t)i * m + j] : make_double2(0.0, 0.0);
+                sR[e] = {dd_of(c.x), dd_of(c.y)};
+            }
+            __syncthreads();
         }
         if (!row) continue;
-        const float4 *R = sR + (whole ? j0 : 0);
-        // P = sum of Re A (Re, Im) R^-1, M = of Im A: A R^-1 = (P.x - M.y) + i (P.y + M.x)
-        float2 P[TJ], Pe[TJ], M[TJ], Me[TJ];
+        Cdd acc[TJ];
 #pragma unroll
-        for (int t = 0; t < TJ; t++) P[t] = Pe[t] = M[t] = Me[t] = make_float2(0.f, 0.f);
-        auto mac = [&](int t, dd re, dd im, float4 c) {
-            const float2 ch = make_float2(c.x, c.y), cl = make_float2(c.z, c.w);
-            df2_mac(P[t], Pe[t], make_float2(re.hi, re.hi), make_float2(re.lo, re.lo), ch, cl);
-            df2_mac(M[t], Me[t], make_float2(im.hi, im.hi), make_float2(im.lo, im.lo), ch, cl);
-        };
-#pragma unroll 2
-        for (int i = 0; i < j0; i++) {
+        for (int t = 0; t < TJ; t++) acc[t] = {dd(0.f, 0.f), dd(0.f, 0.f)};
+        for (int i = 0; i < jmax; i++) {
             const double2 a = A[(int64_t)i * cs + r];
-            const dd re = dd_of_bits(a.x), im = dd_of_bits(a.y);
+            const Cdd v = {dd_of_bits(a.x), dd_of_bits(a.y)};
 #pragma unroll
-            for (int t = 0; t < TJ; t++) mac(t, re, im, R[i * stride + t]);
-        }
-        for (int i = j0; i < jmax; i++) {  // the triangle: columns j >= i
-            const double2 a = A[(int64_t)i * cs + r];
-            const dd re = dd_of_bits(a.x), im = dd_of_bits(a.y);
-#pragma unroll
-            for (int t = 0; t < TJ; t++)
-                if (i <= j0 + t) mac(t, re, im, R[i * stride + t]);
+            for (int t = 0; t < TJ; t++) {
+                const int j = j0 + t;
+                if (j >= m || i > j) continue;
+                acc[t] = cadd(acc[t], cmulc(v, whole ? sR[i * m + j] : sR[i * TJ + t]));
+            }
         }
 #pragma unroll
         for (int t = 0; t < TJ; t++)
-            if (j0 + t < m)
-                A[(int64_t)(j0 + t) * cs + r] =
-                    make_double2(dd_to_double(df_join(P[t].x, Pe[t].x, M[t].y, Me[t].y, -1.f)),
-                                 dd_to_double(df_join(P[t].y, Pe[t].y, M[t].x, Me[t].x, 1.f)));
+            if (j0 + t < m) A[(int64_t)(j0 + t) * cs + r] = make_double2(dd_to_double(acc[t].re), dd_to_double(acc[t].im));
     }
 }
 
@@ -349,6 +333,7 @@ __global__ void k_embed(EmbedArgs a) {
 // form: 0 s = A, 1 s = g5 conj(A) (the spinor of phi^+ D^-1), 2 s = -A.
 // One block per (slice z, chunk of sites, i); its threads own (j, k, alpha) outputs.
 
+constexpr int CB_SITES = 32;   // sites staged per pass
 constexpr int CB_MMAX = 32;    // largest number of columns
 
 struct BaryArgs {

@@ -34,7 +34,6 @@
 #include <cmath>
 #include <cstring>
 
-#include "ddfloat.cuh"
 #include "ddp_host.h"
 
 using namespace ddp;
@@ -183,6 +182,30 @@ __device__ __forceinline__ float2 df_scaled(double v, int f) {
     return make_float2(hi, lo);
 }
 
+// (s, e) += a * b lane by lane for double-floats a = ah + al, b = bh + bl; (s, e) is an unnormalized
+// sum (Knuth's two-sum; the rounding errors are collected in e).
+__device__ __forceinline__ void df2_mac(float2 &s, float2 &e, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 neg = make_float2(-1.f, -1.f);  // x - y = fma(y, -1, x)
+    const float2 p = __fmul2_rn(ah, bh);
+    float2 d = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
+    d = __ffma2_rn(ah, bl, d);
+    d = __ffma2_rn(al, bh, d);
+    const float2 t = __fadd2_rn(s, p);
+    const float2 bb = __ffma2_rn(s, neg, t);
+    const float2 u = __ffma2_rn(__ffma2_rn(bb, neg, t), neg, s), w = __ffma2_rn(bb, neg, p);
+    e = __fadd2_rn(e, __fadd2_rn(__fadd2_rn(u, w), d));
+    s = t;
+}
+
+// hi + lo = (s0 + e0) + sg (s1 + e1) of two such sums.
+__device__ __forceinline__ float2 df_join(float s0, float e0, float s1, float e1, float sg) {
+    s1 *= sg;
+    const float s = __fadd_rn(s0, s1), bb = __fsub_rn(s, s0);
+    const float err = __fadd_rn(__fsub_rn(s0, __fsub_rn(s, bb)), __fsub_rn(s1, bb));
+    const float e = __fadd_rn(err, __fmaf_rn(sg, e1, e0)), h = __fadd_rn(s, e);
+    return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
+}
+
 // Column maxima of the spinors over one time slice: colmax[q], q = (k, alpha), the power of two
 // (with the leading bits) of the largest |Re|, |Im| of s_k(x)_{alpha c} over x and c; infinite for a
 // value that is not finite.  Compared as the integers of their high words: FP64 comparisons run on
@@ -289,9 +312,9 @@ __global__ void __launch_bounds__(256) k_colour_E(EArgs a) {
                     mac(si[(9 + p) * ESITES], sj[(6 + q) * ESITES], sg);
                     mac(si[(6 + p) * ESITES], sj[(9 + q) * ESITES], -sg);
                 }
-                const dd R = df_join(P.x, Pe.x, M.y, Me.y, -1.f), I = df_join(P.y, Pe.y, M.x, Me.x, 1.f);
-                o[c] = make_float4(-I.hi, -I.lo, R.hi, R.lo);  // times i
-                mx = fmaxf(mx, fmaxf(magf(R.hi), magf(I.hi)));
+                const float2 R = df_join(P.x, Pe.x, M.y, Me.y, -1.f), I = df_join(P.y, Pe.y, M.x, Me.x, 1.f);
+                o[c] = make_float4(-I.x, -I.y, R.x, R.y);  // times i
+                mx = fmaxf(mx, fmaxf(magf(R.x), magf(I.x)));
             }
         }
         for (int off = ESITES / 2; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
