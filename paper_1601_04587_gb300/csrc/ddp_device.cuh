@@ -127,6 +127,31 @@ __device__ __forceinline__ unsigned int f2b(float a, float b) {
     return *reinterpret_cast<unsigned int *>(&h);
 }
 
+// A load of data that kernels write: spinor fields, their scales, partial sums.  Never through the
+// read-only path (__ldg): that one is for memory that does not change while the reading kernel is
+// resident, and the kernels of an iteration are resident before their predecessor has ended (see
+// chain_wait).  A plain load is ordered behind the wait, for the compiler and in the caches.  Links,
+// work tables and clover matrices, which no kernel of a solve writes, keep __ldg.
+template <class C>
+__device__ __forceinline__ C ld_field(const C *p) {
+    return *p;
+}
+// The same where the loads are to be issued in the order they are written in.
+__device__ __forceinline__ float4 ld_field_here(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_field_here(const uint4 *p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+
 template <class P>
 __device__ __forceinline__ void load_spinor(const FieldView &f, int64_t i, typename P::real v[24]);
 
@@ -135,7 +160,7 @@ __device__ __forceinline__ void load_spinor<PF64>(const FieldView &f, int64_t i,
     const double2 *b = reinterpret_cast<const double2 *>(f.p);
 #pragma unroll
     for (int j = 0; j < 12; j++) {
-        double2 c = __ldg(b + j * f.stride + i);
+        double2 c = ld_field(b + j * f.stride + i);
         v[2 * j] = c.x;
         v[2 * j + 1] = c.y;
     }
@@ -145,7 +170,7 @@ __device__ __forceinline__ void load_spinor<PF32>(const FieldView &f, int64_t i,
     const float4 *b = reinterpret_cast<const float4 *>(f.p);
 #pragma unroll
     for (int j = 0; j < 6; j++) {
-        float4 c = __ldg(b + j * f.stride + i);
+        float4 c = ld_field(b + j * f.stride + i);
         v[4 * j] = c.x;
         v[4 * j + 1] = c.y;
         v[4 * j + 2] = c.z;
@@ -155,10 +180,10 @@ __device__ __forceinline__ void load_spinor<PF32>(const FieldView &f, int64_t i,
 template <>
 __device__ __forceinline__ void load_spinor<PF16>(const FieldView &f, int64_t i, float v[24]) {
     const uint4 *b = reinterpret_cast<const uint4 *>(f.p);
-    float s = __ldg(f.scale + i);
+    float s = ld_field(f.scale + i);
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-        uint4 c = __ldg(b + j * f.stride + i);
+        uint4 c = ld_field(b + j * f.stride + i);
         float2 a0 = h2f(c.x), a1 = h2f(c.y), a2 = h2f(c.z), a3 = h2f(c.w);
         v[8 * j + 0] = s * a0.x;
         v[8 * j + 1] = s * a0.y;
@@ -175,7 +200,7 @@ __device__ __forceinline__ void load_spinor<PBF16>(const FieldView &f, int64_t i
     const uint4 *b = reinterpret_cast<const uint4 *>(f.p);
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-        uint4 c = __ldg(b + j * f.stride + i);
+        uint4 c = ld_field(b + j * f.stride + i);
         float2 a0 = b2f(c.x), a1 = b2f(c.y), a2 = b2f(c.z), a3 = b2f(c.w);
         v[8 * j + 0] = a0.x;
         v[8 * j + 1] = a0.y;
@@ -192,14 +217,16 @@ __device__ __forceinline__ void load_spinor<PBF16>(const FieldView &f, int64_t i
 // scale, which is returned in *s (1 for the other formats).
 // off: the byte offsets of the storage chunks, kernel parameters, so that no strides are held in
 // registers.
-template <class P>
+// IN_ORDER: see ld_field_here.
+template <class P, bool IN_ORDER>
 __device__ __forceinline__ void load_pairs(const FieldView &f, const int64_t *off, int64_t i, float2 v[12], float *s) {
     using C = typename P::chunk;
     const char *b = reinterpret_cast<const char *>(f.p) + i * (int64_t)sizeof(C);
-    *s = P::SCALED ? __ldg(f.scale + i) : 1.f;
+    *s = P::SCALED ? ld_field(f.scale + i) : 1.f;
 #pragma unroll
     for (int j = 0; j < P::NCH; j++) {
-        const C c = __ldg(reinterpret_cast<const C *>(b + off[j]));
+        const C *q = reinterpret_cast<const C *>(b + off[j]);
+        const C c = IN_ORDER ? ld_field_here(q) : ld_field(q);
         if constexpr (P::NCH == 6) {
             v[2 * j] = make_float2(c.x, c.y);
             v[2 * j + 1] = make_float2(c.z, c.w);

@@ -104,7 +104,7 @@ __device__ __forceinline__ bool skipped(const SolveState &S, int skip) {
 // successor start (chain_next, always after chain_wait: when a kernel starts, all but its direct
 // predecessor are complete).  Every block of a chained kernel waits before it ends, so that a
 // completed kernel implies that all before it are complete.  Without the launch attribute both do
-// nothing.  What it hides is each kernel's start, its item and, in the stencils, the staging of the
+// nothing.  What kernels write is read with plain loads throughout (ld_field).  What it hides is each kernel's start, its item and, in the stencils, the staging of the
 // first wave's links behind the tail of the kernel before: 8 kernels an iteration, 12 columns FP32,
 // 8^4 block 2.84 -> 2.47 ms, 4x32^3 slab 34.5 -> 33.6, 16x24^3 FP16 48.1 -> 46.2.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -286,7 +286,6 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
         }
         if (clov && EPI == EPI_RHS) clover_apply<R>(it.clovinv, it.gV, row, o);
     }
-    store_spinor<P>(a.out, i, o);
     if (DOT == DOT_RHAT) {
         R r[24];
         load_spinor<typename ShadowOf<P>::type>(a.rh, i, r);
@@ -322,7 +321,13 @@ __device__ __forceinline__ void hop_store_epilogue(const HopArgs &a, const Item 
         for (int j = 0; j < 24; j++) n += o[j] * o[j];
         sums[DOT == DOT_TS ? 6 : 0] = n;
     }
+    store_spinor<P>(a.out, i, o);  // last: no load moves above a store
 }
+
+// The FP32 stencil of the five products has no registers to spare: its loads stay where they are
+// written, a few at a time.
+template <class P, int DOT>
+constexpr bool HOP_IN_ORDER = std::is_same<P, PF32>::value && DOT == DOT_TS;
 
 // The same for the low-precision formats without a clover term, one storage chunk at a time (few
 // registers live beside the sums) and in two-lane arithmetic.
@@ -335,16 +340,34 @@ __device__ __forceinline__ void hop_store_pairs(const HopArgs &a, float kap, int
     constexpr bool WITH_V1 = EPI != EPI_PLAIN, WITH_RH = DOT == DOT_RHAT || DOT == DOT_TS;
     const float cw = EPI == EPI_DIRAC ? 1.f / (2.f * kap) : 1.f;
     const float ca = EPI == EPI_DIRAC ? -0.5f : EPI == EPI_MHAT ? -kap * kap : kap;
-    const float sw = (WITH_V1 && P::SCALED) ? __ldg(a.v1.scale + i) : 1.f;
-    const float sr = (WITH_RH && SH::SCALED) ? __ldg(a.rh.scale + i) : 1.f;
+    const float sw = (WITH_V1 && P::SCALED) ? ld_field(a.v1.scale + i) : 1.f;
+    const float sr = (WITH_RH && SH::SCALED) ? ld_field(a.rh.scale + i) : 1.f;
     float2 oo = f2(0.f, 0.f), ww = oo, ow = oo, rw = oo, ro = oo;  // (x.re y.re, x.im y.im) sums
     float owi = 0.f, rwi = 0.f, roi = 0.f;                          // imaginary parts
-    uint4 q = make_uint4(0, 0, 0, 0);
+    // The chunks of v1 and rh are requested AHEAD of their use: they are data that kernels write, so
+    // no load of them moves above the stores in between.  All at once, but for the five products in
+    // FP32, one chunk.  32x24^3, 12 columns, FP32, with the loads at their use / so: (rh, v) 0.242 /
+    // 0.208 ms, (t, s) 0.258 / 0.217 (0.226 without HOP_IN_ORDER).
+    constexpr bool HALF = std::is_same<P, PF32>::value;  // FP32 chunk j of rh: half j % 2 of BF16 chunk j / 2
+    constexpr bool TIGHT = HOP_IN_ORDER<P, DOT>;
+    constexpr int AHEAD = TIGHT ? 1 : P::NCH - 1;
+    using CR = typename SH::chunk;
+    C nw[P::NCH];
+    CR nr[P::NCH];
+    auto request = [&](int j) {
+        const C *w = reinterpret_cast<const C *>(a.v1.p) + j * a.v1.stride + i;
+        const CR *r = reinterpret_cast<const CR *>(a.rh.p) + (HALF ? j / 2 : j) * a.rh.stride + i;
+        if (WITH_V1) nw[j] = TIGHT ? ld_field_here(w) : ld_field(w);
+        if (WITH_RH && !(HALF && j % 2)) nr[j] = TIGHT ? ld_field_here(r) : ld_field(r);
+    };
+#pragma unroll
+    for (int j = 0; j < AHEAD; j++) request(j);
 #pragma unroll
     for (int j = 0; j < P::NCH; j++) {
         float2 w[NC], r[NC];
+        if (j + AHEAD < P::NCH) request(j + AHEAD);
         if (WITH_V1) {
-            chunk_pairs<P>(__ldg(reinterpret_cast<const C *>(a.v1.p) + j * a.v1.stride + i), w);
+            chunk_pairs<P>(nw[j], w);
 #pragma unroll
             for (int c = 0; c < NC; c++) {
                 if (P::SCALED) w[c] = __fmul2_rn(f2(sw, sw), w[c]);
@@ -353,13 +376,12 @@ __device__ __forceinline__ void hop_store_pairs(const HopArgs &a, float kap, int
         }
         if (!P::SCALED) reinterpret_cast<C *>(a.out.p)[j * a.out.stride + i] = pairs_chunk<P>(acc + j * NC);
         if (WITH_RH) {
-            if constexpr (std::is_same<P, PF32>::value) {
-                // FP32 chunk j is half j % 2 of BF16 chunk j / 2
-                if (j % 2 == 0) q = __ldg(reinterpret_cast<const uint4 *>(a.rh.p) + (j / 2) * a.rh.stride + i);
+            if constexpr (HALF) {
+                const CR &q = nr[j - j % 2];
                 r[0] = b2f(j % 2 ? q.z : q.x);
                 r[1] = b2f(j % 2 ? q.w : q.y);
             } else {
-                chunk_pairs<P>(__ldg(reinterpret_cast<const C *>(a.rh.p) + j * a.rh.stride + i), r);
+                chunk_pairs<SH>(nr[j], r);
                 if (SH::SCALED)
 #pragma unroll
                     for (int c = 0; c < NC; c++) r[c] = __fmul2_rn(f2(sr, sr), r[c]);
@@ -436,7 +458,8 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(const __grid_constant
     if (!early) chain_wait();
     if (a.skip) {
         // a block whose columns are all finished has nothing to stage or compute (the flags are set
-        // by k_fin, which is complete: it never directly precedes a stencil)
+        // by k_fin, which is complete: it never directly precedes a stencil; and within a loop a
+        // flag only goes from 1 to 2 to 0, so a column that is seen finished stays so)
         const int col = tc0.col - (int)threadIdx.x / TS + (int)threadIdx.x;
         int live = 0;
         if ((int)threadIdx.x < a.L.CG && col < it.ncol) live = !skipped(a.st[it.solve0 + col], a.skip);
@@ -483,7 +506,7 @@ __global__ void __launch_bounds__(384, DDP_HOP_MINB) k_hop(const __grid_constant
             if (nb >= 0) {                                                \
                 float2 v[12];                                             \
                 float f;                                                  \
-                load_pairs<P>(a.in, a.off, tc.cb + nb, v, &f);           \
+                load_pairs<P, HOP_IN_ORDER<P, DOT>>(a.in, a.off, tc.cb + nb, v, &f); \
                 f2_hop_step<D, P::SCALED>(v, s_u + ((D) * TS + sl) * 9, acc, f); \
             }                                                             \
         }
@@ -615,34 +638,41 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v), one pass (beta
             // is known beforehand, see FIN_OMEGA): 5 spinors read and 3 written, where the update
             // of x and r with its dot products and that of p took 6.5 and 4.  One storage chunk at
-            // a time (the fields do not alias), so few registers and many loads in flight.
+            // a time, the next one requested before this one is stored (x, p and r are written, so
+            // no load moves above a store by itself): few registers and many loads in flight.
             using C = typename P::chunk;
             constexpr int NR = 24 / P::NCH;
-            const C *__restrict__ cx_ = reinterpret_cast<const C *>(a.x.p);
-            const C *__restrict__ cp_ = reinterpret_cast<const C *>(a.p.p);
-            const C *__restrict__ cs_ = reinterpret_cast<const C *>(a.s.p);
-            const C *__restrict__ ct_ = reinterpret_cast<const C *>(a.t.p);
-            const C *__restrict__ cv_ = reinterpret_cast<const C *>(a.v.p);
-            C *__restrict__ ox = reinterpret_cast<C *>(a.x.p);
-            C *__restrict__ orr = reinterpret_cast<C *>(a.r.p);
-            C *__restrict__ op = reinterpret_cast<C *>(a.p.p);
+            C *const fx = reinterpret_cast<C *>(a.x.p), *const fp = reinterpret_cast<C *>(a.p.p);
+            C *const fr = reinterpret_cast<C *>(a.r.p);
+            const C *const fs = reinterpret_cast<const C *>(a.s.p), *const ft = reinterpret_cast<const C *>(a.t.p);
+            const C *const fv = reinterpret_cast<const C *>(a.v.p);
             const auto al = scalar_value(S.alpha, R(0)), om = scalar_value(S.omega, R(0)), be = scalar_value(S.beta, R(0));
             const R ar = al.x, ai = al.y, wr = om.x, wi = om.y, br = be.x, bi = be.y;
+            C n[5];
+            auto request = [&](int64_t o) {
+                n[0] = ld_field(fx + o);
+                n[1] = ld_field(fp + o);
+                n[2] = ld_field(fs + o);
+                n[3] = ld_field(ft + o);
+                n[4] = ld_field(fv + o);
+            };
+            request(i);
 #pragma unroll
             for (int j = 0; j < P::NCH; j++) {
                 const int64_t o = j * a.x.stride + i;
                 R x[NR], p[NR], s[NR], t[NR], v[NR];
-                chunk_to_reals<P>(__ldg(cx_ + o), x);
-                chunk_to_reals<P>(__ldg(cp_ + o), p);
-                chunk_to_reals<P>(__ldg(cs_ + o), s);
-                chunk_to_reals<P>(__ldg(ct_ + o), t);
-                chunk_to_reals<P>(__ldg(cv_ + o), v);
+                chunk_to_reals<P>(n[0], x);
+                chunk_to_reals<P>(n[1], p);
+                chunk_to_reals<P>(n[2], s);
+                chunk_to_reals<P>(n[3], t);
+                chunk_to_reals<P>(n[4], v);
+                if (j + 1 < P::NCH) request(o + a.x.stride);
 #pragma unroll
                 for (int k = 0; k < NR / 2; k++)
                     xrp_update(x + 2 * k, p + 2 * k, s + 2 * k, t + 2 * k, v + 2 * k, ar, ai, wr, wi, br, bi);
-                ox[o] = reals_to_chunk<P>(x);
-                orr[o] = reals_to_chunk<P>(s);
-                op[o] = reals_to_chunk<P>(p);
+                fx[o] = reals_to_chunk<P>(x);
+                fr[o] = reals_to_chunk<P>(s);
+                fp[o] = reals_to_chunk<P>(p);
             }
         } else if (OP == OP_XRP_UPDATE) {  // the same with a whole site-column at a time (its scale)
             R x[24], p[24], s[24], t[24], v[24];
@@ -804,10 +834,10 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
         for (int t = threadIdx.x; t < nt; t += FIN_THREADS) {
             R c[NV];
 #pragma unroll
-            for (int k = 0; k < NV; k++) c[k] = __ldg(A + (int64_t)t * NV + k);
+            for (int k = 0; k < NV; k++) c[k] = ld_field(A + (int64_t)t * NV + k);
 #pragma unroll
             for (int k = 0; k < NV; k++) nsum(v[k], c[k]);
-            if (two) nsum(v[0], __ldg(B + t));
+            if (two) nsum(v[0], ld_field(B + t));
         }
     }
 #pragma unroll
