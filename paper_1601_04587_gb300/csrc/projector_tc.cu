@@ -871,14 +871,15 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
 namespace {
 
 // top[i] = the largest high word, without its sign, of the components of column i over the
-// segment's rows
+// segment's rows; at least 1 if a component is not zero
 __global__ void __launch_bounds__(256) k_gram_max(const double2 *A, int64_t cs, int64_t r0, int64_t nrow, unsigned *top) {
     const double2 *a = A + (int64_t)blockIdx.y * cs + r0;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    unsigned mx = 0;
+    unsigned mx = 0, low = 0;
     int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     auto take = [&](const double2 &v) {
         mx = max(mx, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+        low |= (unsigned)(__double2loint(v.x) | __double2loint(v.y));
     };
     for (; r + 3 * step < nrow; r += 4 * step) {
         const double2 v0 = __ldg(a + r), v1 = __ldg(a + r + step), v2 = __ldg(a + r + 2 * step), v3 = __ldg(a + r + 3 * step);
@@ -888,17 +889,18 @@ __global__ void __launch_bounds__(256) k_gram_max(const double2 *A, int64_t cs, 
         take(v3);
     }
     for (; r < nrow; r += step) take(__ldg(a + r));
+    mx = max(mx, (unsigned)(low != 0));  // subnormals below 2^-1042 have no bit in their high word
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) atomicMax(top + blockIdx.y, mx);
 }
 
-// e with |v| < 2^e for every component of the column (0 for a column of zeros, or of values that
-// vanish at the products' accuracy), NONFINITE if one is not finite.
+// e with |v| < 2^e for every component of the column (0 for a column of zeros), NONFINITE if one is
+// not finite.  A column of subnormals, t its largest high word: |v| < (t + 1) 2^32 2^-1074.
 __global__ void k_gram_exponents(const unsigned *top, int n, int *ex) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int e = (int)(top[i] >> 20);
-    ex[i] = e == 0x7FF ? NONFINITE : e ? e - 1022 : 0;
+    ex[i] = e == 0x7FF ? NONFINITE : e ? e - 1022 : top[i] ? 32 - __clz(top[i]) - 1042 : 0;
 }
 
 struct GramSplitArgs {

@@ -72,3 +72,33 @@ def test_colourless_spinors_at_tile_edges(env, m, box, form):
     g5 = oracle.gamma()[4]
     s = {0: A, 1: np.einsum("ab,mnbc->mnac", g5, np.conj(A)), 2: -A}[form]
     assert _rel(X.cpu().numpy(), projector.colourless_spinors(L, *box, s)) < TOL
+
+
+@pytest.mark.parametrize("m", [5, 33])      # one shared tile, and cross products
+def test_gram_of_subnormal_columns_with_large_ones(env, m):
+    """Columns of subnormals, of all sizes and below 2^-1042 only, against one of size 1e150: their
+    products are ordinary numbers."""
+    ddp, ctx, gid = env
+    box = ((0, 0, 0, 0), (2, 4, 4, 4))
+    n = oracle.box_sites(box[1])
+    A = synth.random_spinor(m, n, 77)
+    rng = np.random.default_rng(1)
+    for c, bits in ((0, 52), (1, 30)):
+        k = rng.integers(-(1 << bits) + 1, 1 << bits, size=(2,) + A[c].shape).astype(np.float64)
+        A[c] = k[0] * 5e-324 + 1j * (k[1] * 5e-324)
+    A[2] *= 1e150
+    did = ddp.ddp_set_domain(ctx, gid, *box)
+    M = torch.zeros((L[0], m, m), dtype=torch.complex128, device="cuda")
+    ddp.ddp_gram_slices(ctx, did, torch.from_numpy(A).cuda(), m, M)
+    ddp.ddp_free_domain(ctx, did)
+    got = M.cpu().numpy()
+    B = A.copy()
+    B[:2] *= 2.0 ** 1000                    # exact
+    for t in range(2):
+        rows = slice(64 * t, 64 * (t + 1))
+        for c in (0, 1):
+            x, y = B[c, rows].reshape(-1), B[2, rows].reshape(-1)
+            want = np.vdot(x, y)
+            size = np.linalg.norm(x) * np.linalg.norm(y)
+            assert abs(got[t, c, 2] * 2.0 ** 1000 - want) < TOL * size
+            assert abs(got[t, 2, c] * 2.0 ** 1000 - np.conj(want)) < TOL * size
