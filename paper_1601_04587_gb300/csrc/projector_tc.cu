@@ -709,26 +709,56 @@ int pick_ksplit(int tiles, int KS) {
     return std::max(best, (KS + MAX_STEPS_PER_BLOCK - 1) / MAX_STEPS_PER_BLOCK);
 }
 
-// X[i][j][k][alpha] = X[j][i][k][alpha] = 2^(e_row + e_col - 14) sum over the K-range
-// partials (fixed order).
-__global__ void k_ozaki_finish(const double *part, int ksplit, int prow, int ncols, int m, int rows,
-                               const double *rowmax, const double *colmax, double2 *X) {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int Q = 4 * m;
-    if (g >= (int64_t)rows * Q) return;
-    const int r = (int)(g / Q), q = (int)(g % Q);
-    double re = 0, im = 0;
-    for (int s = 0; s < ksplit; s++) {
-        const double *p = part + ((int64_t)s * prow + r) * ncols;
-        re += p[q];
-        im += p[Q + q];
+// The sums over the K ranges of a product's elements, in a fixed order.  A block of FIN_THREADS has
+// FIN_THREADS / G elements; thread u E + e adds the ranges u, u + G, ... of element e, and thread e
+// the G sums.  One thread adding up to 152 ranges waited for every load: Gram block of 8 columns on
+// 8^3 sites 43 us, 12 with G = 8; 8 columns of colourless spinors on 4^3 sites 10 and 6.  Few ranges
+// come with many elements, which fill the chip with G = 1.
+constexpr int FIN_THREADS = 256;
+int fin_groups(int ksplit) { return ksplit >= 16 ? 8 : 1; }
+struct RangeSums {
+    int E, e, u;
+    __device__ explicit RangeSums(int G) : E(FIN_THREADS / G), e(threadIdx.x % E), u(threadIdx.x / E) {}
+    __device__ int64_t element() const { return blockIdx.x * (int64_t)E + e; }
+    // v[k] = sum of n[k] values at p[k], step apart; to be used by the threads with u = 0
+    template <int NV>
+    __device__ void sums(bool valid, const double *const p[NV], const int n[NV], int64_t step, double v[NV]) const {
+        __shared__ double sh[NV][FIN_THREADS];
+        const int G = FIN_THREADS / E;
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            v[k] = 0;
+            if (valid)
+                for (int s = u; s < n[k]; s += G) v[k] += __ldg(p[k] + s * step);
+            sh[k][threadIdx.x] = v[k];
+        }
+        __syncthreads();
+        if (u == 0)
+            for (int g = 1; g < G; g++)
+#pragma unroll
+                for (int k = 0; k < NV; k++) v[k] += sh[k][g * E + e];
     }
+};
+
+// X[i][j][k][alpha] = X[j][i][k][alpha] = 2^(e_row + e_col - 14) sum over the K-range
+// partials.
+__global__ void __launch_bounds__(FIN_THREADS) k_ozaki_finish(const double *part, int ksplit, int G, int prow, int ncols, int m,
+                                                              int rows, const double *rowmax, const double *colmax, double2 *X) {
+    const RangeSums rs(G);
+    const int64_t g = rs.element();
+    const int Q = 4 * m;
+    const int r = (int)(g / Q), q = (int)(g % Q);
+    const double *row = part + (int64_t)r * ncols, *const p[2] = {row + q, row + Q + q};
+    const int n[2] = {ksplit, ksplit};
+    double v2[2];
+    rs.sums<2>(r < rows, p, n, (int64_t)prow * ncols, v2);
+    if (r >= rows || rs.u) return;
     // the splits carried v = 2^(e - 49) N = 2^(e - 7) sum_p q_p 2^(-7p) for each operand
     int i, j;
     pair_of(r, m, i, j);
     const int sc = exponent_of(rowmax[r]) + column_exponent(colmax, i) + column_exponent(colmax, j) +
                    exponent_of(colmax[q]) - 14;
-    double2 v = make_double2(ldexp(re, sc), ldexp(im, sc));
+    double2 v = make_double2(ldexp(v2[0], sc), ldexp(v2[1], sc));
     if (!isfinite(rowmax[r]) || !isfinite(colmax[q])) v = make_double2(NAN, NAN);  // a non-finite input
     X[((int64_t)i * m + j) * Q + q] = v;
     if (i != j) X[((int64_t)j * m + i) * Q + q] = v;
@@ -763,10 +793,9 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
     uint8_t *Aq = (uint8_t *)ar.take(bA);
     uint8_t *Bq = (uint8_t *)ar.take(bB);
     double *part = (double *)ar.take(bP);
-    double *rowmax = (double *)ar.take((size_t)rows * 8);
-    double *colmax = (double *)ar.take((size_t)Q * 8);
-    int *rexp = (int *)ar.take((size_t)rows * 4);
-    int *cexp = (int *)ar.take((size_t)Q * 4);
+    // rows, then spinor columns
+    double *rowmax = (double *)ar.take((size_t)(rows + Q) * 8), *colmax = rowmax + rows;
+    int *rexp = (int *)ar.take((size_t)(rows + Q) * 4), *cexp = rexp + rows;
     int *err = (int *)ar.take(64);
     const int es = m <= ES_SMALL_MMAX ? ES_SMALL : ES_LARGE;
     const size_t esm = (size_t)m * colour_kstride(es) * sizeof(float4);
@@ -778,8 +807,7 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
     DDP_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), st));
     for (int z = 0; z < nslice; z++) {
         const int64_t site0 = (int64_t)z * slice_n;
-        DDP_CUDA(ctx, cudaMemsetAsync(rowmax, 0, (size_t)rows * 8, st));
-        DDP_CUDA(ctx, cudaMemsetAsync(colmax, 0, (size_t)Q * 8, st));
+        DDP_CUDA(ctx, cudaMemsetAsync(rowmax, 0, (size_t)(rows + Q) * 8, st));
         EArgs ea;
         ea.A = A;
         ea.n = n;
@@ -809,8 +837,7 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
         sa.MT = MT;
         sa.NT = NT;
         sa.KSh = KSh;
-        k_exponents<<<(rows + 255) / 256, 256, 0, st>>>(rowmax, rows, rexp);
-        k_exponents<<<(Q + 255) / 256, 256, 0, st>>>(colmax, Q, cexp);
+        k_exponents<<<(rows + Q + 255) / 256, 256, 0, st>>>(rowmax, rows + Q, rexp);
         sa.rexp = rexp;
         sa.cexp = cexp;
         sa.Aq = Aq;
@@ -831,9 +858,10 @@ int colourless_tc(ddp_ctx *ctx, const double2 *A, int64_t n, int m, int form, in
         g.err = err;
         k_ozaki_gemm<<<dim3(NT, MT, ksplit), GEMM_BLOCK, gsm, st>>>(g);
         const int64_t nx = (int64_t)rows * Q;
-        k_ozaki_finish<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(
-            part, ksplit, prow, ncols, m, rows, rowmax, colmax, X + (int64_t)((o0 + z) % L0) * m * m * Q);
-        ctx->launches += 8;
+        const int G = fin_groups(ksplit), per = FIN_THREADS / G;
+        k_ozaki_finish<<<(unsigned)((nx + per - 1) / per), FIN_THREADS, 0, st>>>(
+            part, ksplit, G, prow, ncols, m, rows, rowmax, colmax, X + (int64_t)((o0 + z) % L0) * m * m * Q);
+        ctx->launches += 7;
         DDP_CUDA(ctx, cudaGetLastError());
     }
     int h = 0;
@@ -954,31 +982,24 @@ __global__ void __launch_bounds__(256) k_gram_split(GramSplitArgs a) {
     }
 }
 
-// G[i][j] = 2^(e_i + e_j - 14) (sum of the K-range partials), fixed order; cross > 0: the first of
-// the cross products' columns, X_ij - X_ji the imaginary part, in ksplit / 2 ranges.
-__global__ void k_gram_finish(const double *part, int ksplit, int ncols, int m, int cross, const int *cexp, double2 *G) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= m * m) return;
+// G[i][j] = 2^(e_i + e_j - 14) (sum of the K-range partials); cross > 0: the first of the cross
+// products' columns, X_ij - X_ji the imaginary part, in ksplit / 2 ranges.
+__global__ void __launch_bounds__(FIN_THREADS) k_gram_finish(const double *part, int ksplit, int G, int ncols, int m, int cross,
+                                                             const int *cexp, double2 *out) {
+    const RangeSums rs(G);
+    const int g = (int)rs.element();
+    const bool valid = g < m * m;
     const int i = g / m, j = g % m;
-    double re = 0, im = 0;
-    for (int s = 0; s < ksplit; s++) {
-        const double *p = part + ((int64_t)s * TM + i) * ncols;
-        re += p[j];
-        if (!cross) im += p[m + j];
-    }
-    if (cross) {
-        double x = 0, y = 0;
-        for (int s = 0; s < ksplit / 2; s++) {
-            const double *p = part + (int64_t)s * TM * ncols + cross;
-            x += p[(int64_t)i * ncols + j];
-            y += p[(int64_t)j * ncols + i];
-        }
-        im = x - y;
-    }
+    const double *ri = part + (int64_t)i * ncols, *rj = part + (int64_t)j * ncols;
+    const double *const p[3] = {ri + j, ri + (cross ? cross : m) + j, rj + cross + i};
+    const int n[3] = {ksplit, cross ? ksplit / 2 : ksplit, cross ? ksplit / 2 : 0};
+    double s[3];
+    rs.sums<3>(valid, p, n, (int64_t)TM * ncols, s);
+    if (!valid || rs.u) return;
     const int sc = cexp[i] + cexp[j] - 14;
     double2 v = make_double2(NAN, NAN);
-    if (cexp[i] != NONFINITE && cexp[j] != NONFINITE) v = make_double2(ldexp(re, sc), ldexp(im, sc));
-    G[g] = v;
+    if (cexp[i] != NONFINITE && cexp[j] != NONFINITE) v = make_double2(ldexp(s[0], sc), ldexp(s[1] - s[2], sc));
+    out[g] = v;
 }
 
 }  // namespace
@@ -1052,8 +1073,9 @@ int gram_tc(ddp_ctx *ctx, const double2 *A, int64_t cs, int m, int64_t seg, int 
         g.part = part;
         g.err = err;
         k_ozaki_gemm<<<dim3(NT, 1, ksplit), GEMM_BLOCK, gsm, st>>>(g);
-        k_gram_finish<<<(unsigned)((m * m + 127) / 128), 128, 0, st>>>(part, ksplit, ncols, m, mixed ? 0 : NTr * TN, cexp,
-                                                                       out + (int64_t)z * m * m);
+        const int G = fin_groups(ksplit), per = FIN_THREADS / G;
+        k_gram_finish<<<(unsigned)((m * m + per - 1) / per), FIN_THREADS, 0, st>>>(part, ksplit, G, ncols, m, mixed ? 0 : NTr * TN,
+                                                                               cexp, out + (int64_t)z * m * m);
         ctx->launches += 5;
         DDP_CUDA(ctx, cudaGetLastError());
     }
