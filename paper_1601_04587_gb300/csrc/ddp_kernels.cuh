@@ -14,10 +14,10 @@ namespace ddp {
 
 // ------------------------------------------------------------ solver state
 
-// Per solve (one column of one request).  The scalars of the inner recurrence are of the format's
-// scalar type (recur.cuh): FP64, or double-FP32 in the same 8 bytes; scalar() reads them.
+// Per solve (one column of one request).
 struct SolveState {
-    double2 rho, alpha, omega, beta;
+    double2 rho, alpha, omega, beta, inv;   // the inner recurrence (recur.cuh)
+    float2 alpha32, omega32, beta32;         // the same rounded, for the vector updates in FP32
     double target2;  // inner stopping threshold on |r|^2
     double bnorm2;   // |eta|^2 (FP64)
     double rr64;     // |eta - D_Gamma x|^2 of the current outer cycle (FP64)
@@ -39,17 +39,13 @@ struct SolveState {
     double kappa;
 };
 
-template <class T>
-__device__ __forceinline__ Cnum<T> &scalar(double2 &v) {
-    static_assert(sizeof(Cnum<T>) == sizeof(double2), "same storage");
-    return reinterpret_cast<Cnum<T> &>(v);
+__device__ __forceinline__ void set_scalar(double2 &v, float2 &v32, Cnum c) {
+    v = c;
+    v32 = make_float2((float)c.x, (float)c.y);
 }
-// A scalar of the recurrence in the compute precision (for double-FP32 its high part: no conversion).
-__device__ __forceinline__ double2 scalar_value(const double2 &v, double) { return v; }
-__device__ __forceinline__ float2 scalar_value(const double2 &v, float) {
-    const float4 c = reinterpret_cast<const float4 &>(v);
-    return make_float2(c.x, c.z);
-}
+// A scalar of the recurrence in the compute precision.
+__device__ __forceinline__ double2 scalar_value(const double2 &v, const float2 &, double) { return v; }
+__device__ __forceinline__ float2 scalar_value(const double2 &, const float2 &v32, float) { return v32; }
 
 struct LoopCtl {
     unsigned long long arrived;  // this iteration: columns decided (low half), columns going on (high half)
@@ -155,8 +151,8 @@ __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L)
 // Sums of NV values over the 32 sites of a tile, which are one warp of one column.  Each
 // thread's products and the warp's sums are formed in the compute precision R (FP32 for the
 // low-precision formats: FP64 arithmetic is a small fraction of GB300's FP32 rate); the sums over
-// tiles, in the scalar kernels, are FP64 or double-FP32.  Fixed order: results do not depend on the batch
-// around them.  The lanes split the values as the distance halves (9 shuffles for 8 values, not
+// tiles, in the scalar kernels, have at least the precision of FP64 (recur.cuh).  Fixed order:
+// results do not depend on the batch around them.  The lanes split the values as the distance halves (9 shuffles for 8 values, not
 // 40): value k ends in lanes k * 32 / NV and following.
 template <int NV, typename R>
 __device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &tc, R v[NV], Partials part) {
@@ -626,7 +622,7 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             R r[24], v[24];
             load_spinor<P>(a.r, i, r);
             load_spinor<P>(a.v, i, v);
-            const auto al = scalar_value(S.alpha, R(0));
+            const auto al = scalar_value(S.alpha, S.alpha32, R(0));
             const R ar = al.x, ai = al.y;
 #pragma unroll
             for (int j = 0; j < 12; j++) {
@@ -646,7 +642,8 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             C *const fr = reinterpret_cast<C *>(a.r.p);
             const C *const fs = reinterpret_cast<const C *>(a.s.p), *const ft = reinterpret_cast<const C *>(a.t.p);
             const C *const fv = reinterpret_cast<const C *>(a.v.p);
-            const auto al = scalar_value(S.alpha, R(0)), om = scalar_value(S.omega, R(0)), be = scalar_value(S.beta, R(0));
+            const auto al = scalar_value(S.alpha, S.alpha32, R(0)), om = scalar_value(S.omega, S.omega32, R(0)),
+                       be = scalar_value(S.beta, S.beta32, R(0));
             const R ar = al.x, ai = al.y, wr = om.x, wi = om.y, br = be.x, bi = be.y;
             C n[5];
             auto request = [&](int64_t o) {
@@ -681,7 +678,8 @@ __global__ void __launch_bounds__(384) k_blas(const __grid_constant__ BlasArgs a
             load_spinor<P>(a.s, i, s);
             load_spinor<P>(a.t, i, t);
             load_spinor<P>(a.v, i, v);
-            const auto al = scalar_value(S.alpha, R(0)), om = scalar_value(S.omega, R(0)), be = scalar_value(S.beta, R(0));
+            const auto al = scalar_value(S.alpha, S.alpha32, R(0)), om = scalar_value(S.omega, S.omega32, R(0)),
+                       be = scalar_value(S.beta, S.beta32, R(0));
             const R ar = al.x, ai = al.y, wr = om.x, wi = om.y, br = be.x, bi = be.y;
 #pragma unroll
             for (int k = 0; k < 12; k++)
@@ -737,11 +735,7 @@ __device__ __forceinline__ int scale_exponent(double scale) { return ((__double2
 __device__ __forceinline__ void low_of(double &w, double v, int, double scale) { w = scale * v; }
 __device__ __forceinline__ void low_of(float &w, double v, int m, double scale) { w = float_of(v, m, scale); }
 __device__ __forceinline__ double high_of(double w) { return w; }
-__device__ __forceinline__ double high_of(float w) {
-    const unsigned u = __float_as_uint(w), e = (u >> 23) & 0xFF;
-    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
-    return (u << 1) == 0 ? 0.0 : (double)w;
-}
+__device__ __forceinline__ double high_of(float w) { return wide(w); }
 
 // lo = scale * hi  (scale = 2 kappa / sigma: the normalised defect), times T^-1
 // of the site when a.clov is set
@@ -804,16 +798,14 @@ struct FinArgs {
     cudaGraphConditionalHandle loop;
 };
 
-// One block per solve: fixed-order sum of the solve's tile partials (in R), then the scalar
+// One block per solve: fixed-order sum of the solve's tile partials (of type R), then the scalar
 // recurrences of BiCGStab or of the defect correction.  FIN_OMEGA finds omega and the scalars of
-// the next iteration from the five products of the (t, s) stencil (bicg_omega), so that x, r and p
-// are updated in one pass and an iteration has two reductions.  (r, r) is then good to the rounding
-// of the sums times (s, s), an inner stopping criterion; the true residual of the outer cycle
-// decides convergence.
+// the next iteration from the five products of the (t, s) stencil (bicg_omega, which says how good
+// they are), so that x, r and p are updated in one pass and an iteration has two reductions.
 constexpr int FIN_THREADS = 256;
 template <int FIN, typename R>
 __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
-    using T = typename ScalarOf<R>::type;
+    using T = typename SumOf<R>::type;
     constexpr int NV = FIN == FIN_OMEGA ? PART_MAX : FIN == FIN_ALPHA ? 2 : 1;
     constexpr bool two = (FIN == FIN_BNORM || FIN == FIN_RESID);
     __shared__ T sh[FIN_THREADS / 32][NV];
@@ -824,10 +816,11 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
     const int nt = S.ntiles, active = S.active;
     const int64_t base = S.pbase;
     // the state the recurrence starts from, read while the partials are on their way
-    Cnum<T> rho = scalar<T>(S.rho), alpha = scalar<T>(S.alpha);
+    const Cnum rho = S.rho, inv = S.inv;
+    const double target2 = S.target2;
     T v[NV];
 #pragma unroll
-    for (int k = 0; k < NV; k++) nset(v[k], 0.0);
+    for (int k = 0; k < NV; k++) sum_zero(v[k]);
     const bool wanted = !(FIN == FIN_ALPHA || FIN == FIN_OMEGA) || active == 1;
     if (wanted) {
         const R *A = reinterpret_cast<const R *>(a.A.d) + base * NV, *B = reinterpret_cast<const R *>(a.B.d) + base;
@@ -836,12 +829,10 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
 #pragma unroll
             for (int k = 0; k < NV; k++) c[k] = ld_field(A + (int64_t)t * NV + k);
 #pragma unroll
-            for (int k = 0; k < NV; k++) nsum(v[k], c[k]);
-            if (two) nsum(v[0], ld_field(B + t));
+            for (int k = 0; k < NV; k++) sum_add(v[k], c[k]);
+            if (two) sum_add(v[0], ld_field(B + t));
         }
     }
-#pragma unroll
-    for (int k = 0; k < NV; k++) nsum_end(v[k]);
     // the lanes split the values as the distance halves: value k ends in lane k * 32 / NV
     int off = 16;
 #pragma unroll
@@ -850,33 +841,35 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
 #pragma unroll
         for (int i = 0; i < n / 2; i++) {
             const T keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
-            v[i] = nadd(keep, nshfl_xor(send, off));
+            v[i] = sum_join(keep, sum_shfl_xor(send, off));
         }
     }
 #pragma unroll
-    for (; off > 0; off >>= 1) v[0] = nadd(v[0], nshfl_xor(v[0], off));
+    for (; off > 0; off >>= 1) v[0] = sum_join(v[0], sum_shfl_xor(v[0], off));
     if ((lane & (32 / NV - 1)) == 0) sh[warp][lane / (32 / NV)] = v[0];
     __syncthreads();
     if (warp != 0) return;
-    T q;
-    nset(q, 0.0);
+    double q = 0.0;
     if (lane < NV) {
-        const T p0 = nadd(sh[0][lane], sh[1][lane]), p1 = nadd(sh[2][lane], sh[3][lane]), p2 = nadd(sh[4][lane], sh[5][lane]),
-                p3 = nadd(sh[6][lane], sh[7][lane]);
-        q = nadd(nadd(p0, p1), nadd(p2, p3));
-    }
+        T p[FIN_THREADS / 32];
 #pragma unroll
-    for (int k = 0; k < NV; k++) v[k] = nshfl(q, k);
+        for (int k = 0; k < FIN_THREADS / 32; k++) p[k] = sh[k][lane];
+#pragma unroll
+        for (int n = FIN_THREADS / 64; n > 0; n >>= 1)
+#pragma unroll
+            for (int k = 0; k < n; k++) p[k] = sum_join(p[2 * k], p[2 * k + 1]);
+        q = sum_value(p[0]);
+    }
+    double w[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) w[k] = __shfl_sync(0xffffffffu, q, k);
     if (lane != 0) return;
-    T zero, one;
-    nset(zero, 0.0);
-    nset(one, 1.0);
-    const Cnum<T> c0 = {zero, zero}, c1 = {one, zero};
+    const Cnum c0 = cn(0.0, 0.0), c1 = cn(1.0, 0.0);
     if constexpr (FIN == FIN_BNORM) {
-        S.bnorm2 = v[0];
-        S.outer_done = S.outer_done || (v[0] == 0.0);
+        S.bnorm2 = w[0];
+        S.outer_done = S.outer_done || (w[0] == 0.0);
     } else if constexpr (FIN == FIN_RESID) {
-        const double n = v[0];
+        const double n = w[0];
         if (S.outer_done) {  // converged earlier: its residual was not recomputed
             S.sigma = 0;
             S.scale = 0;
@@ -897,27 +890,27 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
             S.delta = fmin(d, 0.1);
         }
     } else if constexpr (FIN == FIN_INIT) {
-        T d2;
-        nset(d2, S.delta * S.delta);
-        scalar<T>(S.rho) = {v[0], zero};
-        reinterpret_cast<T &>(S.target2) = nmul(d2, v[0]);
+        S.rho = cn(w[0], 0.0);
+        S.target2 = S.delta * S.delta * w[0];
         S.iters = 0;
-        const bool act = (S.sigma > 0) && npositive(v[0]);
+        const bool act = (S.sigma > 0) && (w[0] > 0);
         S.active = act ? 1 : 0;
         S.status = act ? 0 : 4;
-        scalar<T>(S.alpha) = act ? c1 : c0;
-        scalar<T>(S.omega) = act ? c1 : c0;
-        scalar<T>(S.beta) = c0;
+        set_scalar(S.alpha, S.alpha32, act ? c1 : c0);
+        set_scalar(S.omega, S.omega32, act ? c1 : c0);
+        set_scalar(S.beta, S.beta32, c0);
     } else if constexpr (FIN == FIN_ALPHA) {
         if (active == 1) {
-            if (bicg_alpha(rho, Cnum<T>{v[0], v[1]}, alpha)) {
-                scalar<T>(S.alpha) = alpha;
+            Cnum alpha, hv;
+            if (bicg_alpha(rho, cn(w[0], w[1]), alpha, hv)) {
+                S.inv = hv;
+                set_scalar(S.alpha, S.alpha32, alpha);
             } else {
                 S.active = 0;
                 S.status = 2;
-                scalar<T>(S.alpha) = c0;
-                scalar<T>(S.omega) = c0;
-                scalar<T>(S.beta) = c0;
+                set_scalar(S.alpha, S.alpha32, c0);
+                set_scalar(S.omega, S.omega32, c0);
+                set_scalar(S.beta, S.beta32, c0);
             }
         } else {
             S.active = 0;  // its last update has been made
@@ -925,20 +918,20 @@ __global__ void __launch_bounds__(FIN_THREADS) k_fin(FinArgs a) {
     } else if constexpr (FIN == FIN_OMEGA) {
         int going = 0;
         if (active == 1) {
-            Cnum<T> omega, rc;
-            int status = bicg_omega(v, reinterpret_cast<T &>(S.target2), omega, rc);
+            Cnum omega, rc, beta;
+            int status = bicg_omega(w, target2, inv, omega, rc, beta);
             const int iters = S.iters + 1;
             S.iters = iters;
             S.total_iters++;
             if (!status && iters >= S.maxit) status = 3;
-            scalar<T>(S.omega) = omega;
+            set_scalar(S.omega, S.omega32, omega);
             if (status) {
                 S.active = 2;
                 S.status = status;
-                scalar<T>(S.beta) = c0;
+                set_scalar(S.beta, S.beta32, c0);
             } else {
-                scalar<T>(S.beta) = bicg_beta(rc, rho, alpha, omega);
-                scalar<T>(S.rho) = rc;
+                set_scalar(S.beta, S.beta32, beta);
+                S.rho = rc;
                 going = 1;
             }
         }

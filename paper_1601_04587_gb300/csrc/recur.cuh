@@ -1,127 +1,149 @@
-// Scalar recurrences of BiCGStab (van der Vorst) in FP64 or in double-FP32.
+// Scalar recurrences of BiCGStab (van der Vorst) in FP64, and the sums they start from.
 //
-// The FP64 storage format computes its sums and scalars in FP64.  The low-precision formats use
-// double-FP32 (48 bits, ddfloat.cuh) beyond the FP32 sum of a tile's 32 sites: GB300 issues two
-// FP64 operations per clock and SM, so that the sums over tiles and the divisions of one iteration
-// took 15.8 + 5.3 us for 12 columns of 16x24^3 in FP64 (k_fin of (t, s) and of (rh, v)), 6.6 + 3.9
-// in double-FP32, and the vector updates no longer convert their scalars from FP64 in every thread
-// (FP16 x, r, p update 98 -> 82 us).  The summands are good to 24 bits and the results are rounded
-// to FP32 when used.
+// A tile's 32 sites are summed in the compute precision of the storage format; the sums over tiles
+// and the recurrences are FP64, or more.  GB300 issues two FP64 operations per clock and SM, so the
+// sums over tiles of FP32 values are formed on the FP32 pipe, in three floats: every addition is
+// split exactly (Knuth's two-sum) and only the third float, about 2^-48 of the sum, is rounded, 2^-72
+// where FP64 has 2^-53.  One conversion to FP64 at the end.  The recurrences are FP64 operations of
+// one lane, with reciprocals in the place of divisions and both of an iteration's second half
+// started from the sums; their results are stored in FP32 beside the FP64 scalars, so that the
+// vector updates convert nothing.  k_fin of (t, s) and of (rh, v), 12 columns of 16x24^3: 15.8 + 5.3
+// us with FP64 sums, one launch after another; chained (where a duration holds the wait for the
+// kernel before) 13.8 + 9.8 so, 11.6 + 9.0 with sums and scalars of 48 bits, which is less than the
+// reductions are to have.  The whole 8^4 propagator 2.49 / 2.56 ms with 48 bits / so, 16x24^3 in FP16
+// the same to 0.2%; the columns come out bit for bit alike in most solves.
 #pragma once
 
-#include "ddfloat.cuh"
+#include <cuda_runtime.h>
+#include <math.h>
+#include <string.h>
+
+#define DDP_HD __host__ __device__ __forceinline__
 
 namespace ddp {
 
+struct Sum3 {
+    float hi, mid, lo;
+};
+
 template <typename R>
-struct ScalarOf {  // of a format that computes in R
+struct SumOf {  // the sum of values of type R
     using type = double;
 };
 template <>
-struct ScalarOf<float> {
-    using type = dd;
+struct SumOf<float> {
+    using type = Sum3;
 };
 
-__device__ __forceinline__ double nadd(double a, double b) { return a + b; }
-__device__ __forceinline__ double nsub(double a, double b) { return a - b; }
-__device__ __forceinline__ double nmul(double a, double b) { return a * b; }
-__device__ __forceinline__ double ndiv(double a, double b) { return a / b; }
-__device__ __forceinline__ bool nfinite(double a) { return isfinite(a); }
-__device__ __forceinline__ bool npositive(double a) { return a > 0; }
-__device__ __forceinline__ bool nzero(double a) { return a == 0; }
-__device__ __forceinline__ dd nadd(dd a, dd b) { return dd_add(a, b); }
-__device__ __forceinline__ dd nsub(dd a, dd b) { return dd_sub(a, b); }
-__device__ __forceinline__ dd nmul(dd a, dd b) { return dd_mul(a, b); }
-// a / b to about 2^-45: the FP32 quotient and that of the remainder
-__device__ __forceinline__ dd ndiv(dd a, dd b) {
-    const float q = a.hi / b.hi;
-    const dd r = dd_sub(a, dd_mul(dd(q, 0.f), b));
-    return dd_renorm(q, r.hi / b.hi);
+// s + e = a + b exactly, s = a + b rounded (sums only: nothing to contract)
+DDP_HD void two_sum(float a, float b, float &s, float &e) {
+    s = a + b;
+    const float t = s - a;
+    e = (a - (s - t)) + (b - t);
 }
-__device__ __forceinline__ bool nfinite(dd a) { return isfinite(a.hi); }
-__device__ __forceinline__ bool npositive(dd a) { return a.hi > 0.f; }
-__device__ __forceinline__ bool nzero(dd a) { return a.hi == 0.f; }
 
-// A summand joins a running sum (nsum_end: the low part of a double-FP32 sum is renormalised).
-__device__ __forceinline__ void nsum(double &s, double v) { s += v; }
-__device__ __forceinline__ void nsum_end(double &) {}
-__device__ __forceinline__ void nsum(dd &s, float v) {
-    const float t = __fadd_rn(s.hi, v), b = __fsub_rn(t, s.hi);
-    s.lo = __fadd_rn(s.lo, __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, b)), __fsub_rn(v, b)));
-    s.hi = t;
+DDP_HD void sum_zero(double &s) { s = 0.0; }
+DDP_HD void sum_zero(Sum3 &s) { s = {0.f, 0.f, 0.f}; }
+// s += v
+DDP_HD void sum_add(double &s, double v) { s += v; }
+DDP_HD void sum_add(Sum3 &s, float v) {
+    float h, m, e;
+    two_sum(s.hi, v, h, e);
+    s.hi = h;
+    two_sum(s.mid, e, m, e);
+    s.mid = m;
+    s.lo += e;
 }
-__device__ __forceinline__ void nsum_end(dd &s) { s = dd_renorm(s.hi, s.lo); }
+DDP_HD double sum_join(double a, double b) { return a + b; }
+DDP_HD Sum3 sum_join(const Sum3 &a, const Sum3 &b) {
+    Sum3 s;
+    float e, f, g, m;
+    two_sum(a.hi, b.hi, s.hi, e);
+    two_sum(a.mid, b.mid, m, f);
+    two_sum(m, e, s.mid, g);
+    s.lo = (a.lo + b.lo) + (f + g);
+    return s;
+}
+// Every FP64 instruction of a warp, conversions and comparisons among them, takes 16 clocks of the
+// SM's FP64 pipe, whatever the number of active lanes: what integers can do, they do here.
+// A float as a double.
+DDP_HD double wide(float w) {
+#ifdef __CUDA_ARCH__
+    const unsigned u = __float_as_uint(w), e = (u >> 23) & 0xFF;
+    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+    return (u << 1) == 0 ? 0.0 : (double)w;
+#else
+    return (double)w;
+#endif
+}
+// The bits of a double, and three questions to them.
+DDP_HD unsigned long long bits_of(double v) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long b;
+    memcpy(&b, &v, sizeof(b));
+    return b;
+#endif
+}
+DDP_HD bool is_zero(double v) { return (bits_of(v) << 1) == 0; }
+DDP_HD bool is_finite(double v) { return ((bits_of(v) >> 52) & 0x7FF) != 0x7FF; }
+DDP_HD bool is_positive(double v) { return bits_of(v) - 1 < 0x7FF0000000000000ull; }  // infinity among them
+DDP_HD double sum_value(double s) { return s; }
+DDP_HD double sum_value(const Sum3 &s) {
+    // a sum that is not finite has no parts
+    return isfinite(s.hi) ? wide(s.hi) + (wide(s.mid) + wide(s.lo)) : (double)s.hi;
+}
+__device__ __forceinline__ double sum_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ Sum3 sum_shfl_xor(const Sum3 &a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.mid, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
 
-__device__ __forceinline__ double nshfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ dd nshfl_xor(dd a, int o) {
-    return dd(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o));
-}
-__device__ __forceinline__ double nshfl(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
-__device__ __forceinline__ dd nshfl(dd a, int l) {
-    return dd(__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l));
-}
-__device__ __forceinline__ void nset(double &a, double v) { a = v; }
-__device__ __forceinline__ void nset(dd &a, double v) { a = dd_of(v); }
+using Cnum = double2;
+DDP_HD Cnum cn(double re, double im) { return make_double2(re, im); }
+DDP_HD Cnum cn_mul(Cnum a, Cnum b) { return cn(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+DDP_HD Cnum cn_mulc(Cnum a, Cnum b) { return cn(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y); }  // a conj(b)
+DDP_HD Cnum cn_scale(Cnum a, double r) { return cn(a.x * r, a.y * r); }
+DDP_HD double cn_norm(Cnum a) { return a.x * a.x + a.y * a.y; }
+DDP_HD bool cn_zero(Cnum a) { return is_zero(a.x) && is_zero(a.y); }
+DDP_HD bool cn_finite(Cnum a) { return is_finite(a.x) && is_finite(a.y); }
 
-template <class T>
-struct Cnum {
-    T re, im;
-};
-template <class T>
-__device__ __forceinline__ Cnum<T> cn_mul(Cnum<T> a, Cnum<T> b) {
-    return {nsub(nmul(a.re, b.re), nmul(a.im, b.im)), nadd(nmul(a.re, b.im), nmul(a.im, b.re))};
-}
-__device__ __forceinline__ Cnum<double> cn_div(Cnum<double> a, Cnum<double> b) {
-    const double d = b.re * b.re + b.im * b.im;
-    return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
-}
-__device__ __forceinline__ Cnum<dd> cn_div(Cnum<dd> a, Cnum<dd> b) {
-    // b scaled by a power of two, so that its square stays in range
-    const int e = 127 - (int)((__float_as_uint(fmaxf(fabsf(b.re.hi), fabsf(b.im.hi))) >> 23) & 0xFF);
-    const float f = __int_as_float((127 + max(-126, min(126, e))) << 23);
-    b = {dd_scale2(b.re, f), dd_scale2(b.im, f)};
-    const dd n = dd_add(dd_mul(b.re, b.re), dd_mul(b.im, b.im));
-    const Cnum<dd> c = cn_mul(a, Cnum<dd>{b.re, dd_neg(b.im)});
-    return {dd_scale2(ndiv(c.re, n), f), dd_scale2(ndiv(c.im, n), f)};
-}
-template <class T>
-__device__ __forceinline__ bool cn_zero(Cnum<T> a) { return nzero(a.re) && nzero(a.im); }
-template <class T>
-__device__ __forceinline__ bool cn_finite(Cnum<T> a) { return nfinite(a.re) && nfinite(a.im); }
-
-// alpha = rho / (rh, v); false: the recurrence has broken down.
-template <class T>
-__device__ __forceinline__ bool bicg_alpha(Cnum<T> rho, Cnum<T> hv, Cnum<T> &alpha) {
+// alpha = rho / (rh, v), and inv = 1 / (rh, v) for bicg_omega; false: the recurrence has broken down.
+DDP_HD bool bicg_alpha(Cnum rho, Cnum hv, Cnum &alpha, Cnum &inv) {
     if (cn_zero(hv) || !cn_finite(hv)) return false;
-    alpha = cn_div(rho, hv);
+    const double r = 1.0 / cn_norm(hv);
+    inv = cn(hv.x * r, -hv.y * r);
+    alpha = cn_mul(rho, inv);
     return true;
 }
 
 // omega and, before r is formed, the scalars of the next iteration, from the products
 // w = (t, s), (rh, s), (rh, t), (t, t), (s, s) of the (t, s) stencil: with r = s - omega t,
-//   rc = (rh, r) = (rh, s) - omega (rh, t),   rr = (r, r) = (s, s) - |(t, s)|^2 / (t, t).
+//   rc = (rh, r) = (rh, s) - omega (rh, t),   rr = (r, r) = (s, s) - |(t, s)|^2 / (t, t),
+//   beta = (rc / rho) (alpha / omega) = rc inv / omega,   1 / omega = (t, t) conj((t, s)) / |(t, s)|^2,
+// so that both reciprocals start from the sums at once.
+// The errors of rc and rr are those of the products, 2^-24 of |rh| |s| and (s, s) in the
+// low-precision formats, where sums over r itself would have 2^-24 of |rh| |r| and (r, r): omega
+// minimises |r|, so |r| < |s|, and what is lost is the factor by which this half step shrinks the
+// residual, once and not over the iterations.  (rh, s) is zero but for rounding (alpha makes it so),
+// and rr only ends the inner loop: the FP64 true residual of the outer cycle decides convergence.
 // Returns 1 when the column has converged, 2 when the recurrence has broken down, 0 to go on.
-template <class T>
-__device__ __forceinline__ int bicg_omega(const T w[8], T target2, Cnum<T> &omega, Cnum<T> &rc) {
-    const Cnum<T> ts = {w[0], w[1]}, hs = {w[2], w[3]}, ht = {w[4], w[5]};
-    T zero;
-    nset(zero, 0.0);
-    omega = {zero, zero};
-    T rr = w[7];
-    if (npositive(w[6])) {
-        omega = {ndiv(ts.re, w[6]), ndiv(ts.im, w[6])};
-        rr = nsub(rr, nadd(nmul(ts.re, omega.re), nmul(ts.im, omega.im)));
+DDP_HD int bicg_omega(const double w[8], double target2, Cnum inv, Cnum &omega, Cnum &rc, Cnum &beta) {
+    const Cnum ts = cn(w[0], w[1]);
+    const double tt = w[6], n = cn_norm(ts);
+    const Cnum g = cn_scale(cn_mulc(inv, ts), tt * (1.0 / n));
+    omega = cn(0.0, 0.0);
+    double rr = w[7];
+    if (is_positive(tt)) {
+        const double r = 1.0 / tt;
+        omega = cn_scale(ts, r);
+        rr -= n * r;
     }
-    const Cnum<T> m = cn_mul(omega, ht);
-    rc = {nsub(hs.re, m.re), nsub(hs.im, m.im)};
-    if (nfinite(rr) && !npositive(nsub(rr, target2))) return 1;
-    return cn_zero(rc) || cn_zero(omega) || !cn_finite(rc) || !nfinite(rr) ? 2 : 0;
-}
-
-// beta = (rc / rho) (alpha / omega)
-template <class T>
-__device__ __forceinline__ Cnum<T> bicg_beta(Cnum<T> rc, Cnum<T> rho, Cnum<T> alpha, Cnum<T> omega) {
-    return cn_div(cn_mul(rc, alpha), cn_mul(rho, omega));
+    const Cnum m = cn_mul(omega, cn(w[4], w[5]));
+    rc = cn(w[2] - m.x, w[3] - m.y);
+    beta = cn_mul(rc, g);
+    if (is_finite(rr) && rr <= target2) return 1;
+    return cn_zero(rc) || cn_zero(omega) || !cn_finite(rc) || !is_finite(rr) ? 2 : 0;
 }
 
 }  // namespace ddp

@@ -14,7 +14,7 @@
 // all take the same decisions.
 //
 // Arithmetic is FP32 on FP32 vectors for every storage format (links as stored); sums over sites
-// are FP32 within a warp, double-FP32 beyond, as in the per-step kernels (recur.cuh).
+// are FP32 within a warp, three floats beyond, scalars FP64, as in the per-step kernels (recur.cuh).
 //
 // What bounds it is latency: a block's 8 warps spend about 5000 cycles on an application of the
 // hopping term (2700 of them shared-memory wavefronts), 1000 on a barrier.  Propagators of 12
@@ -53,7 +53,7 @@ struct SmallShared {
     float2 link[2][8][SMALL_SITES][9];                // the hop's oriented link, per output parity
     float4 vec[3][SMALL_COLS][6][SMALL_SITES];        // p, s (and r), odd intermediate
     short nb[2][8][SMALL_SITES];                      // -1, or block << 7 | site, | SMALL_NEG
-    float2 slot[2][SMALL_MAX_CLUSTER][SMALL_COLS * PART_MAX];  // partial sums of every block, double-buffered
+    float4 slot[2][SMALL_MAX_CLUSTER][SMALL_COLS * PART_MAX];  // partial sums of every block, double-buffered
     float warp[SMALL_THREADS / 32][PART_MAX];
     float2 alpha[SMALL_COLS], omega[SMALL_COLS], beta[SMALL_COLS];
     int go[SMALL_COLS];                               // the column goes on iterating
@@ -149,7 +149,7 @@ __device__ __forceinline__ void f2_dot(float &re, float &im, float2 a, float2 b)
 // Sums of NV values over a column's sites, over all blocks of the cluster: on return lane c * NV + k
 // of warp 0 of every block holds value k of column c.  buf alternates between calls.
 template <int NV>
-__device__ __forceinline__ dd small_sums(SmallShared &sh, float v[NV], int csize, unsigned rank, int buf) {
+__device__ __forceinline__ double small_sums(SmallShared &sh, float v[NV], int csize, unsigned rank, int buf) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int off = 16;
 #pragma unroll
@@ -170,32 +170,33 @@ __device__ __forceinline__ dd small_sums(SmallShared &sh, float v[NV], int csize
     for (int q = threadIdx.x; q < NT * csize; q += SMALL_THREADS) {
         const int t = q % NT, r = q / NT, c = t / NV, k = t % NV;
         const float *w = &sh.warp[c * (SMALL_SITES / 32)][k];
-        const dd s = dd_add(dd_add(dd(w[0], 0.f), dd(w[PART_MAX], 0.f)), dd_add(dd(w[2 * PART_MAX], 0.f), dd(w[3 * PART_MAX], 0.f)));
+        Sum3 s = {w[0], 0.f, 0.f};
+#pragma unroll
+        for (int n = 1; n < SMALL_SITES / 32; n++) sum_add(s, w[n * PART_MAX]);
         const unsigned a = cluster_addr((unsigned)__cvta_generic_to_shared(&sh.slot[buf][rank][t]), (unsigned)r);
-        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(s.hi), "f"(s.lo) : "memory");
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %3};" ::"r"(a), "f"(s.hi), "f"(s.mid), "f"(s.lo) : "memory");
     }
     cluster_sync(csize);
-    dd s(0.f, 0.f);
-    if (warp == 0) {
+    if (warp != 0) return 0.0;
+    {
         // two lanes per value: even and odd blocks, each as a tree
         const int t = lane & 15, odd = lane >> 4;
-        dd d[SMALL_MAX_CLUSTER / 2];
+        Sum3 d[SMALL_MAX_CLUSTER / 2];
 #pragma unroll
         for (int r = 0; r < SMALL_MAX_CLUSTER / 2; r++) {
-            d[r] = dd(0.f, 0.f);
+            sum_zero(d[r]);
             if (t < NT && 2 * r + odd < csize) {
-                const float2 f = sh.slot[buf][2 * r + odd][t];
-                d[r] = dd(f.x, f.y);
+                const float4 f = sh.slot[buf][2 * r + odd][t];
+                d[r] = {f.x, f.y, f.z};
             }
         }
 #pragma unroll
         for (int n = SMALL_MAX_CLUSTER / 4; n > 0; n >>= 1)
             if (csize > 2 * n)
 #pragma unroll
-                for (int r = 0; r < n; r++) d[r] = dd_add(d[r], d[r + n]);
-        s = dd_add(d[0], nshfl_xor(d[0], 16));
+                for (int r = 0; r < n; r++) d[r] = sum_join(d[r], d[r + n]);
+        return sum_value(sum_join(d[0], sum_shfl_xor(d[0], 16)));
     }
-    return s;
 }
 
 template <class P>
@@ -316,22 +317,22 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
     small_put(sh, SV_S, cc, l, rp);
     int buf = 0;
     // the scalars live in lane c of warp 0
-    const dd zero(0.f, 0.f);
-    Cnum<dd> rho = {zero, zero}, alpha = rho, omega = rho;
-    dd target2 = zero;
+    const Cnum c0 = cn(0.0, 0.0);
+    Cnum rho = c0, alpha = c0, inv = c0;
+    double target2 = 0.0;
     int iters = 0, maxit = 0, status = 4, running = 0;
     {
-        const dd q = small_sums<1>(sh, sums, csize, rank, buf);
+        const double q = small_sums<1>(sh, sums, csize, rank, buf);
         buf ^= 1;
         if (threadIdx.x < 32) {
             const int c = threadIdx.x & (SMALL_COLS - 1);
-            const dd n = nshfl(q, c);
+            const double n = __shfl_sync(0xffffffffu, q, c);
             if (threadIdx.x < SMALL_COLS) {
                 const bool hc = col0 + c < it.ncol;
                 const SolveState *Sc = a.st + it.solve0 + (hc ? col0 + c : 0);
-                running = hc && Sc->sigma > 0 && n.hi > 0.f;
-                rho = {n, zero};
-                target2 = dd_mul(dd_of(Sc->delta * Sc->delta), n);
+                running = hc && Sc->sigma > 0 && n > 0.0;
+                rho = cn(n, 0.0);
+                target2 = Sc->delta * Sc->delta * n;
                 maxit = Sc->maxit;
                 status = running ? 0 : 4;
                 sh.go[c] = running;
@@ -357,18 +358,18 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
             }
         }
         {
-            const dd q = small_sums<2>(sh, sums, csize, rank, buf);
+            const double q = small_sums<2>(sh, sums, csize, rank, buf);
             buf ^= 1;
             if (threadIdx.x < 32) {
                 const int c = threadIdx.x & (SMALL_COLS - 1);
-                const Cnum<dd> hv = {nshfl(q, 2 * c), nshfl(q, 2 * c + 1)};
+                const Cnum hv = cn(__shfl_sync(0xffffffffu, q, 2 * c), __shfl_sync(0xffffffffu, q, 2 * c + 1));
                 if (threadIdx.x < SMALL_COLS) {
-                    if (!running || !bicg_alpha(rho, hv, alpha)) {
-                        alpha = {zero, zero};
+                    if (!running || !bicg_alpha(rho, hv, alpha, inv)) {
+                        alpha = c0;
                         if (running) status = 2;
                         running = 0;
                     }
-                    sh.alpha[c] = f2(alpha.re.hi, alpha.im.hi);
+                    sh.alpha[c] = f2((float)alpha.x, (float)alpha.y);
                     sh.upd[c] = running;
                 }
             }
@@ -406,26 +407,26 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1) k_small(const __grid_constan
             }
         }
         {
-            const dd q = small_sums<PART_MAX>(sh, sums, csize, rank, buf);
+            const double q = small_sums<PART_MAX>(sh, sums, csize, rank, buf);
             buf ^= 1;
             if (threadIdx.x < 32) {
                 const int c = threadIdx.x & (SMALL_COLS - 1);
-                dd w[PART_MAX];
+                double w[PART_MAX];
 #pragma unroll
-                for (int k = 0; k < PART_MAX; k++) w[k] = nshfl(q, c * PART_MAX + k);
+                for (int k = 0; k < PART_MAX; k++) w[k] = __shfl_sync(0xffffffffu, q, c * PART_MAX + k);
                 if (threadIdx.x < SMALL_COLS && running) {
-                    Cnum<dd> rc, beta = {zero, zero};
-                    status = bicg_omega(w, target2, omega, rc);
+                    Cnum omega, rc, beta;
+                    status = bicg_omega(w, target2, inv, omega, rc, beta);
                     iters++;
                     if (!status && iters >= maxit) status = 3;
                     if (status) {
                         running = 0;
+                        beta = c0;
                     } else {
-                        beta = bicg_beta(rc, rho, alpha, omega);
                         rho = rc;
                     }
-                    sh.omega[c] = f2(omega.re.hi, omega.im.hi);
-                    sh.beta[c] = f2(beta.re.hi, beta.im.hi);
+                    sh.omega[c] = f2((float)omega.x, (float)omega.y);
+                    sh.beta[c] = f2((float)beta.x, (float)beta.y);
                 }
                 if (threadIdx.x < SMALL_COLS) sh.go[c] = running;
             }
