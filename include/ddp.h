@@ -303,11 +303,12 @@ int ddp_poll(ddp_ctx *ctx, uint64_t ticket, int *done, ddp_solve_info *info);
  * "tile_cols" (columns per block, 1..12, 0 = automatic), "tuned_cols_fp64" ...
  * "tuned_cols_bf16" (a remembered autotuner choice, 0 = none), "tuned_carveout_fp64" ...
  * "tuned_carveout_bf16" (the autotuner's stencil carveout for that storage format,
- * percent, -1 = the driver's choice, -2 = none: "stencil_carveout" applies), "conditional" (1: the
+ * percent, -1 = the driver's choice, -2 = none: "stencil_carveout" if it was set, else 70 for
+ * FP64 and 28 for the other formats), "conditional" (1: the
  * inner loop is a device-driven CUDA-graph WHILE node; 0: host-polled graph
  * chunks), "stencil_carveout" (preferred shared-memory share of the unified L1 /
- * shared memory for the inner-loop stencils, percent; default 28, -1 = the driver's
- * choice), "contraction_double_fp32" (1, the default: the nucleon contraction of
+ * shared memory for the inner-loop stencils of all formats, percent, -1 = the driver's
+ * choice; reads 28 until it is set), "contraction_double_fp32" (1, the default: the nucleon contraction of
  * ddp_contract in double-FP32 arithmetic, relative error about 1e-13; 0: FP64),
  * "projector_tensor_cores" (1, the default: the Gram blocks and colourless
  * spinor sums of the projector cut, m <= 128, run as an emulated-FP64 product on the
@@ -349,8 +350,8 @@ int ddp_time_hop(ddp_ctx *ctx, int domain_id, double kappa, int ncol, int precis
 /* Autotuner: times the three inner-loop stencil variants on the domain (ncol
  * columns, the given storage format, iters launches each) for every admissible
  * number of columns per thread block (the block shape, 32 sites x columns) and
- * every candidate shared-memory carveout of the stencils (28, 50, 100 percent of the
- * unified L1 / shared memory), keeps the pair with the shortest stencil time per
+ * every candidate shared-memory carveout of the stencils (28, for FP64 70, 50 and 100 percent
+ * of the unified L1 / shared memory), keeps the pair with the shortest stencil time per
  * BiCGStab iteration (2 x PLAIN + SCHUR_RHAT + SCHUR_TS) for that storage format in
  * the context (used by every later solve with that format; ddp_get_param
  * "tuned_cols_<format>" and "tuned_carveout_<format>" read it back) and returns the

@@ -390,7 +390,9 @@ def autotune_cached(ctx, domain_id, n_sites, kappa, ncol, precision, cache_path=
     to $DDP_TUNE_CACHE.  A cached choice is applied without timing."""
     import json
     path = cache_path or os.environ.get("DDP_TUNE_CACHE")
-    key = f"{_PREC_NAMES[int(precision)]}/ncol{int(ncol)}/sites2^{max(0, int(n_sites).bit_length() - 1)}"
+    # the FP64 stencil is the integer one: choices remembered for another do not fit it
+    stencil = {"fp64": "fp64int"}.get(_PREC_NAMES[int(precision)], _PREC_NAMES[int(precision)])
+    key = f"{stencil}/ncol{int(ncol)}/sites2^{max(0, int(n_sites).bit_length() - 1)}"
     cache = {}
     if path and os.path.exists(path):
         with open(path) as f:

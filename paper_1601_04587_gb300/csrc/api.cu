@@ -1247,6 +1247,7 @@ int ddp_set_param(ddp_ctx *ctx, const char *name, double value) {
     else if (n == "stencil_carveout") {
         if (value < -1 || value > 100) return DDP_ERR_INVALID_ARG;
         p.carveout = (int)value;
+        p.carveout_set = true;
     }
     else if (n == "tuned_cols_fp64" || n == "tuned_cols_fp32" || n == "tuned_cols_fp16" || n == "tuned_cols_bf16") {
         if (value < 0 || value > HOP_MAX_CG) return DDP_ERR_INVALID_ARG;
@@ -1296,7 +1297,7 @@ int ddp_autotune(ddp_ctx *ctx, int domain_id, double kappa, int ncol, int precis
                  float *best_ms) {
     if (!ctx || ncol < 1 || precision < 0 || precision > 3 || iters < 1) return DDP_ERR_INVALID_ARG;
     const int cands[] = {12, 8, 6, 4, 3, 2, 1};
-    const int carves[] = {28, 50, 100};
+    const int carves[] = {default_carveout(precision), 50, 100};
     const int weight[3] = {2, 1, 1};
     const int saved = ctx->prm.CG, saved_cv = ctx->prm.carveout_prec[precision];
     int best = 0, best_cv = carves[0];

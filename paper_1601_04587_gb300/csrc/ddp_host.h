@@ -82,11 +82,11 @@ struct EngineParams {
     int CG_prec[4] = {0, 0, 0, 0};  // columns per block chosen by ddp_autotune, per storage format
     int use_conditional = 1;    // device-driven while loop in a CUDA graph
     int host_chunk = 16;        // iterations per host check without conditional nodes
-    // preferred shared-memory carveout of the inner-loop stencils, percent (-1: the driver's
-    // choice): 28 rounds up to the smallest carveout that holds three 19.6 KB blocks and
-    // leaves the rest of the unified memory (about 192 KB) as L1 for the neighbour gathers
+    // preferred shared-memory carveout of the inner-loop stencils of all formats, percent (-1: the
+    // driver's choice); not in force until it is set
     int carveout = 28;
-    // the carveout ddp_autotune chose for a storage format (-2: none, use carveout)
+    bool carveout_set = false;
+    // the carveout ddp_autotune chose for a storage format (-2: none)
     int carveout_prec[4] = {-2, -2, -2, -2};
     int small_sites = SMALL_MAX_NH;  // largest domain (sites per parity) solved on chip in one kernel (0: none)
     int contract_dd = 1;        // nucleon contraction in double-FP32 arithmetic (0: FP64)
@@ -96,9 +96,17 @@ struct EngineParams {
     int overlap_downloads = 1;
 };
 
-// The stencil carveout of a storage format: the autotuner's choice, else the context's.
+// The carveout that holds the resident blocks a format's stencil is built for and leaves the rest
+// of the unified memory as L1 for the neighbour gathers: three blocks of 19.6 KB (28 rounds up to
+// the smallest carveout that does), four of 38.1 KB for the integer FP64 stencil.  With 28 only one
+// of the latter is resident: 16x24^3, 12 columns, plain / (rh, v) / (t, s) 1.70 / 2.04 / 2.54 ms
+// with 28, 0.78 / 0.95 / 1.22 with 50, 0.69 / 0.80 / 1.04 with 70, 0.73 / 0.86 / 1.11 with 100.
+inline int default_carveout(int prec) { return prec == DDP_PREC_FP64 ? 70 : 28; }
+// The stencil carveout of a storage format: the autotuner's choice, else the context's if it was
+// set, else the format's own.
 inline int carveout_for(const EngineParams &p, int prec) {
-    return (prec >= 0 && prec < 4 && p.carveout_prec[prec] != -2) ? p.carveout_prec[prec] : p.carveout;
+    if (p.carveout_prec[prec] != -2) return p.carveout_prec[prec];
+    return p.carveout_set ? p.carveout : default_carveout(prec);
 }
 
 // A growable device arena owned by the context.
