@@ -576,6 +576,12 @@ int ddp_destroy(ddp_ctx *ctx) {
         cudaStreamSynchronize(ctx->copy_stream);
         cudaStreamDestroy(ctx->copy_stream);
     }
+    for (auto &s : ctx->side) {
+        if (s.stream) cudaStreamSynchronize(s.stream);
+        if (s.stream) cudaStreamDestroy(s.stream);
+        if (s.done) cudaEventDestroy(s.done);
+    }
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     cudaStreamDestroy(ctx->stream);
     delete ctx;
     return DDP_OK;

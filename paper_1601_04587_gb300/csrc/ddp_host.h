@@ -148,6 +148,13 @@ struct ddp_ctx {
     ddp::Arena results;   // device-resident propagators and series terms of ddp_propagator_series
     ddp::Arena aux;       // partial sums of the projector-cut kernels
     cudaStream_t copy_stream = nullptr;  // device-to-host copies overlapped with compute (created on first use)
+    // work beside the work stream between a fork and a join of it (created on first use)
+    struct Side {
+        cudaStream_t stream = nullptr;
+        cudaEvent_t done = nullptr;
+    };
+    std::vector<Side> side;
+    cudaEvent_t ev_fork = nullptr;
     void *serve = nullptr;
     int max_cluster = -1;  // largest cluster of the small-domain kernel the device runs (-1: not asked yet)
     // instrumentation: per-kernel-class launch counts of the last solve

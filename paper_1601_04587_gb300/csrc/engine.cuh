@@ -500,21 +500,61 @@ struct Engine {
         conv(false, tmp, xo);
         return DDP_OK;
     }
-    int correction(bool r_is_eta) {
-        int rc = DDP_OK;
-        if constexpr (!P::IS64) {
-            for (const Plan::Small &g : plan.small)
-                if ((rc = correct_small(g, r_is_eta))) return rc;
-        }
+    int correct_large(bool r_is_eta) {
         if (!plan.nlarge) return DDP_OK;
         large_items();
-        rc = clov ? correction_t<true>(r_is_eta) : correction_t<false>(r_is_eta);
+        const int rc = clov ? correction_t<true>(r_is_eta) : correction_t<false>(r_is_eta);
         all_items();
         return rc;
     }
+    // The groups of small items, one per cluster size, and the large items have nothing in common
+    // and each of them fills a part of the SMs only: they run beside one another, the groups on
+    // streams of their own between a fork and a join of the work stream.  One after another (FP32,
+    // 12 columns): clusters of 1 to 8 blocks 3.53 ms, with an 8^4 block 5.29, so 1.35 and 2.78; all by the
+    // per-step kernels 1.94 and 2.73.
+    int correction(bool r_is_eta) {
+        if constexpr (P::IS64) {
+            return correct_large(r_is_eta);
+        } else {
+            // the longest first; without large items one group stays on the work stream
+            const int n = (int)plan.small.size(), nside = plan.nlarge ? n : std::max(0, n - 1);
+            int rc = fork(nside);
+            if (rc) return rc;
+            for (int i = 0; i < n && !rc; i++) {
+                rc = correct_small(plan.small[n - 1 - i], r_is_eta, i < nside ? ctx->side[i].stream : ctx->stream);
+                if (!rc && i < nside && cudaEventRecord(ctx->side[i].done, ctx->side[i].stream) != cudaSuccess)
+                    rc = set_cuda_error(ctx, cudaGetLastError(), "end of a group of small domains");
+            }
+            if (!rc) rc = correct_large(r_is_eta);
+            for (int i = 0; i < nside; i++) {
+                const cudaError_t e = rc ? cudaStreamSynchronize(ctx->side[i].stream)
+                                         : cudaStreamWaitEvent(ctx->stream, ctx->side[i].done, 0);
+                if (e != cudaSuccess && !rc) rc = set_cuda_error(ctx, e, "join of the small domains");
+            }
+            return rc;
+        }
+    }
+    // The first n side streams wait for what the work stream has been given so far.
+    int fork(int n) {
+        if (!n) return DDP_OK;
+        if (!ctx->ev_fork) DDP_CUDA(ctx, cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
+        while ((int)ctx->side.size() < n) {
+            ddp_ctx::Side s;
+            DDP_CUDA(ctx, cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming));
+            const cudaError_t e = cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking);
+            if (e != cudaSuccess) {
+                cudaEventDestroy(s.done);
+                return set_cuda_error(ctx, e, "side stream");
+            }
+            ctx->side.push_back(s);
+        }
+        DDP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
+        for (int i = 0; i < n; i++) DDP_CUDA(ctx, cudaStreamWaitEvent(ctx->side[i].stream, ctx->ev_fork, 0));
+        return DDP_OK;
+    }
 
     // One correction of the small items of one cluster size (small.cuh), in one kernel.
-    int correct_small(const Plan::Small &g, bool r_is_eta) {
+    int correct_small(const Plan::Small &g, bool r_is_eta, cudaStream_t stream) {
         SmallArgs a;
         a.items = d_items + g.item0;
         a.nitems = g.nitems;
@@ -527,7 +567,7 @@ struct Engine {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         small_config<P>(cfg, attr, g.csize, g.nclusters);
-        cfg.stream = ctx->stream;
+        cfg.stream = stream;
         DDP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_small<P>, a));
         launches++;
         return DDP_OK;
