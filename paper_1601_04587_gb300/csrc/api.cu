@@ -47,6 +47,29 @@ Arena::~Arena() {
     if (base) cudaFree(base);
 }
 
+// f(job, psi, out) for the columns of an FP64 stencil call on n sites: all at once, or, where the
+// device has no memory for their block fixed-point fields beside the FP64 ones, fewer at a time (a
+// column's result does not depend on the others).
+template <class F>
+static int by_columns(const Job &job, int64_t n, const double *psi, double *out, F f) {
+    int step = job.ncol;
+    for (int c = 0; c < job.ncol;) {
+        Job part = job;
+        part.ncol = std::min(step, job.ncol - c);
+        const int64_t off = (int64_t)c * n * 24;
+        const int rc = f(part, psi + off, out + off);
+        if (rc == DDP_ERR_OOM && part.ncol > 1) {
+            cudaGetLastError();
+            step = (part.ncol + 1) / 2;
+        } else if (rc) {
+            return rc;
+        } else {
+            c += part.ncol;
+        }
+    }
+    return DDP_OK;
+}
+
 void make_plan(const std::vector<Job> &jobs, int prec, const EngineParams &prm, Plan &plan) {
     int maxcol = 1;
     for (auto &j : jobs) maxcol = std::max(maxcol, j.ncol);
@@ -824,7 +847,11 @@ int ddp_apply_dirac(ddp_ctx *ctx, int domain_id, double kappa, double csw, const
     j.ncol = ncol;
     if (csw != 0.0 && (rc = clover_for(ctx, *const_cast<GaugeDev *>(g), kappa, csw, &j.clov))) return rc;
     switch (precision) {
-        case DDP_PREC_FP64: rc = apply_dirac_impl<PF64>(ctx, j, (const double *)si.dev, (double *)so.dev, precision); break;
+        case DDP_PREC_FP64:
+            rc = by_columns(j, d->n, (const double *)si.dev, (double *)so.dev, [&](const Job &q, const double *in, double *to) {
+                return apply_dirac_impl<PF64>(ctx, q, in, to, precision);
+            });
+            break;
         case DDP_PREC_MIXED_FP32: rc = apply_dirac_impl<PF32>(ctx, j, (const double *)si.dev, (double *)so.dev, precision); break;
         case DDP_PREC_MIXED_FP16: rc = apply_dirac_impl<PF16>(ctx, j, (const double *)si.dev, (double *)so.dev, precision); break;
         default: rc = apply_dirac_impl<PBF16>(ctx, j, (const double *)si.dev, (double *)so.dev, precision); break;
@@ -855,7 +882,9 @@ int ddp_hop_power(ddp_ctx *ctx, int domain_id, double kappa, int p, const double
     memcpy(j.e, d->e, sizeof(j.e));
     j.kappa = kappa;
     j.ncol = ncol;
-    if ((rc = hop_power_fx(ctx, j, p, (const double *)si.dev, (double *)so.dev))) return rc;
+    rc = by_columns(j, d->n, (const double *)si.dev, (double *)so.dev,
+                    [&](const Job &q, const double *in, double *to) { return hop_power_fx(ctx, q, p, in, to); });
+    if (rc) return rc;
     if ((rc = so.copy_out())) return rc;
     DDP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return DDP_OK;

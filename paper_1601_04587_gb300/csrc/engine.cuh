@@ -332,9 +332,11 @@ struct Engine {
 
     // ----------------------------------------------------------- building blocks
 
+    // a partial slot: the most sums of a stencil in the compute precision, or one FP64 norm
+    static constexpr size_t PART_BYTES = PART_MAX * sizeof(typename P::real);
     static size_t bytes_needed(int64_t cap, int64_t npart, int nitems, int nsolve) {
         return 6 * field_bytes<PF64>(cap) + 9 * field_bytes<P>(cap) +
-               (size_t)npart * (PART_MAX + 1) * sizeof(double) + 2048 + (size_t)nitems * sizeof(Item) +
+               (size_t)npart * (PART_BYTES + sizeof(double)) + 2048 + (size_t)nitems * sizeof(Item) +
                (size_t)nsolve * sizeof(SolveState) + sizeof(LoopCtl) + 8192;
     }
 
@@ -368,7 +370,7 @@ struct Engine {
         static_assert((P::NCH * 5 + ShadowOf<P>::type::NCH) * 16 >= PFX::NCH * 16 + 4, "fixed-point field over the inner fields");
         fx_outer = fx_over(r);
         fx_inner = fx_over(re64);
-        A.d = a.take(npart * PART_MAX * sizeof(double));
+        A.d = a.take(npart * PART_BYTES);
         B.d = a.take(npart * sizeof(double));  // true-residual norms only
         d_items = (Item *)a.take(nitems * sizeof(Item));
         d_st = (SolveState *)a.take(nsolve * sizeof(SolveState));

@@ -52,8 +52,9 @@ struct Server : ServerBase {
         eng.prec = precision;
         max_active = maxact;
         nsolve_cap = MAX_NCOL * maxact;
-        // bytes per site-column of capacity (fields) plus the per-tile partials
-        double per = (double)Engine<P>::bytes_needed(1 << 20, 0, 0, 0) / (1 << 20) + (PART_MAX + 1) * 8.0 / 32.0;
+        // bytes per site-column of capacity (fields) plus 48 for the partials of a tile (they are 40
+        // in the low-precision formats and 72 in FP64, 1 in 4000 beyond the budget)
+        double per = (double)Engine<P>::bytes_needed(1 << 20, 0, 0, 0) / (1 << 20) + 48.0 / 32.0;
         cap = (int64_t)((double)budget / per);
         cap = (cap / 32) * 32;
         if (cap < 1024) return DDP_ERR_OOM;
