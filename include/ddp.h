@@ -142,14 +142,22 @@ int ddp_domain_sites(ddp_ctx *ctx, int domain_id, int64_t *n_sites, int64_t *glo
  * O(a)-improvement (clover) term c_sw (i/4) sum_{mu,nu} sigma_{mu nu} F_{mu nu}(x)
  * with the clover-leaf field strength F = (Q_{mu nu} - Q_{nu mu}) / 8 of the whole
  * gauge field (the improved operator the footnotes of Sec. 4 and Sec. 5 refer to);
- * the term is site-local, so D_Gamma keeps it at every site of the domain. */
+ * the term is site-local, so D_Gamma keeps it at every site of the domain.
+ * Accuracy of the hopping term in FP64 (here, in ddp_hop_power and in every true
+ * residual): it is summed in block fixed point, 57 bits below the largest component
+ * of a site's neighbours.  The error of an output component is about 2^-57 of that
+ * component, less than FP64 arithmetic makes of a product with it; but a neighbour
+ * component smaller than it by a factor f keeps 57 - log2(f) bits, and none from f = 2^57
+ * on, where FP64 arithmetic would keep 53 of its own as long as nothing larger is added
+ * to it (links with zeros, as in a unit gauge field). */
 int ddp_apply_dirac(ddp_ctx *ctx, int domain_id, double kappa, double csw, const double *psi, double *out, int ncol,
                     int precision);
 
 /* out = (kappa D_hop)^p psi on the domain, in FP64: p applications of the
  * hopping term of D_Gamma (the Dirichlet-masked stencil of Sec. 2, with
  * 2 kappa D = 1 - kappa D_hop of Sec. 5), each scaled by kappa.  This is the
- * operator of the hopping-parameter-expanded trace, Eq. HPEtr:
+ * operator of the hopping-parameter-expanded trace, Eq. HPEtr (accuracy: see
+ * ddp_apply_dirac):
  * tr{g5 D^-1} = kappa^p tr{g5 D_hop^p D^-1} for p <= 8.  With
  * psi = D_Gamma^-1 g5 eta (ddp_solve_sources) and p = 8,
  * ddp_contract(DDP_CONTRACT_PSEUDO_NOISE, out, eta = g5 eta) is the expanded

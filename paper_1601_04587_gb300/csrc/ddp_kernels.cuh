@@ -100,9 +100,10 @@ __device__ __forceinline__ bool skipped(const SolveState &S, int skip) {
 // successor start (chain_next, always after chain_wait: when a kernel starts, all but its direct
 // predecessor are complete).  Every block of a chained kernel waits before it ends, so that a
 // completed kernel implies that all before it are complete.  Without the launch attribute both do
-// nothing.  What kernels write is read with plain loads throughout (ld_field).  What it hides is each kernel's start, its item and, in the stencils, the staging of the
-// first wave's links behind the tail of the kernel before: 8 kernels an iteration, 12 columns FP32,
-// 8^4 block 2.84 -> 2.47 ms, 4x32^3 slab 34.5 -> 33.6, 16x24^3 FP16 48.1 -> 46.2.
+// nothing.  What kernels write is read with plain loads throughout (ld_field).  What it hides is
+// each kernel's start, its item and, in the stencils, the staging of the first wave's links behind
+// the tail of the kernel before: 8 kernels an iteration, 12 columns FP32, 8^4 block 2.84 -> 2.47 ms,
+// 4x32^3 slab 34.5 -> 33.6, 16x24^3 FP16 48.1 -> 46.2.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -152,8 +153,8 @@ __device__ __forceinline__ TileCoord tile_coord(const Item &it, const Launch &L)
 // thread's products and the warp's sums are formed in the compute precision R (FP32 for the
 // low-precision formats: FP64 arithmetic is a small fraction of GB300's FP32 rate); the sums over
 // tiles, in the scalar kernels, have at least the precision of FP64 (recur.cuh).  Fixed order:
-// results do not depend on the batch around them.  The lanes split the values as the distance halves (9 shuffles for 8 values, not
-// 40): value k ends in lanes k * 32 / NV and following.
+// results do not depend on the batch around them.  The lanes split the values as the distance halves
+// (9 shuffles for 8 values, not 40): value k ends in lanes k * 32 / NV and following.
 template <int NV, typename R>
 __device__ __forceinline__ void warp_partials(const Item &it, const TileCoord &tc, R v[NV], Partials part) {
     const int lane = threadIdx.x & 31;
@@ -1103,11 +1104,12 @@ __host__ __device__ constexpr int fx_cols(int CG) { return (CG + FX_SPLIT - 1) /
 // k_hop at FP64 accuracy: a.in is in block fixed point, the epilogue and its operands are FP64
 // (OUTFX: the plain sums are stored in block fixed point instead, for the next hop).  Blocks as
 // k_hop: the oriented links of a 32-site tile are staged once, as integers, for the columns.
-// About 4300 integer instructions per site-column, 1728 of them multiply-adds, instead of 864 on
-// the FP64 pipe at 1/32 of the rate: 2.10 -> 0.59 ms for the plain sums of 110592 sites x 12
+// About 6000 instructions per site-column, 1728 of them the widening multiply-adds and 1700 not of
+// the hop (staging, which each of the FX_SPLIT parts repeats, and the epilogue), instead of 864
+// on the FP64 pipe at 1/32 of the rate: 2.10 -> 0.56 ms for the plain sums of 110592 sites x 12
 // columns (16x24^3, one parity).  The sums alone are 48 registers, a neighbour 48, its projection
-// 24, so there are few warps: the multiply-add pipe is 47% busy, the rest waits for neighbours (L2)
-// and for the staging.
+// 24, so there are few warps (16 an SM): the multiply-add pipe is 55% busy, issue 35%, the rest
+// waits for neighbours (L2) and for the staging.
 template <int EPI, int DOT, bool CLOV, bool OUTFX>
 __global__ void __launch_bounds__(FX_MAX_THREADS, FX_MINB) k_hop_fx(const __grid_constant__ HopArgs a) {
     constexpr int TS = HOP_TS;

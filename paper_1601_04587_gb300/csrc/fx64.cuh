@@ -19,7 +19,11 @@
 // component of the neighbours in all, where a chain of FP64 multiply-adds makes 2^-53 of each
 // partial sum.  Against quad precision (relative, a 5x5x4x4 box, neighbouring time slices alike
 // or a factor e^3 apart): one application 0.75e-16, FP64 arithmetic 1.5e-16; eighth power
-// 1.6e-16, FP64 arithmetic 2.2e-16.
+// 1.6e-16, FP64 arithmetic 2.2e-16.  These are errors against the norm: a component that is smaller
+// than the largest of its site-column and of the eight neighbours by a factor f keeps 57 - log2(f)
+// bits, and none from f = 2^57 on.  With links that mix colours and spins every output component
+// holds products of the largest one, whose rounding in FP64 arithmetic is 2^-53; only where such
+// products vanish (links with zeros) would FP64 arithmetic keep more of the small ones.
 //
 // A site-column that holds a NaN or an infinity keeps its raw doubles under the exponent
 // FX_RAW, and an output with such a neighbour is evaluated in FP64 arithmetic (fx_slow), so that

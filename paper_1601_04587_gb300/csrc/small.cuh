@@ -18,12 +18,13 @@
 //
 // What bounds it is latency: a block's 8 warps spend about 5000 cycles on an application of the
 // hopping term (2700 of them shared-memory wavefronts), 1000 on a barrier.  Propagators of 12
-// columns, FP32, per-step kernels -> this kernel, one alone / 64 in a batch: 4^4 1.49 -> 0.55 /
-// 3.74 -> 2.31 ms, 8x4^3 1.68 -> 0.64 / 5.99 -> 3.82, 8x8x4x4 1.95 -> 0.72 / 9.83 -> 6.95, 8^3x4
-// 2.21 -> 0.81 / 18.2 -> 16.9.  With 16 blocks a cluster an 8^4 block alone gained as much (2.79 ->
-// 1.20) but 64 of them lost (37.4 -> 54.0: clusters wait for their slowest block and fill 128 of
-// 152 SMs), so the path ends at 8 blocks.  Two threads per site-column (one spin of the projection
-// each) and one row of links rebuilt from the other two were slower.
+// columns, FP32, per-step kernels / this kernel: one alone 4^4 1.21 / 0.56 ms, 8x4^3 1.33 / 0.62,
+// 8x8x4x4 1.34 / 0.67, 8^3x4 1.55 / 0.77; 64 in a batch 2.94 / 2.37, 4.66 / 3.84, 7.47 / 6.67, 13.9 /
+// 15.9 (8 of 8^3x4 2.60 / 2.60).  The largest domains gain alone and lose in large batches of their
+// like: eight blocks of one SM each wait for their slowest.  With 16 blocks a cluster an 8^4 block
+// alone went 2.79 -> 1.20, 64 of them 37.4 -> 54.0, so the path ends at 8 blocks.  Two threads per
+// site-column (one spin of the projection each) and one row of links rebuilt from the other two
+// were slower.
 //
 // A request takes this path by its own size alone, so its result does not depend on what else is
 // solved with it.
